@@ -115,18 +115,15 @@ typedef struct sls_options {
                               and the screened kernel (SLS_KERNEL_AUTO or _FILTERED); costs
                               140 bytes of device memory per 32 nodes.  The batched and
                               allocation-free forms compute every tile; the server rejects it. */
-    int32_t numbering;     /* FP64: 0 (default) lets the library renumber a mesh of at least
-                              2^20 nodes, 1 keeps the caller's numbering, 2 renumbers at any
-                              size (binary32 meshes keep it: their pass gains nothing).
-                              Form A: every window of 128 consecutive ids lists its nodes by
-                              incident-triangle count, then degree (fixed nodes last, ties by
-                              id); Form B: the same inside each colour class's range.  The 32
-                              lanes of a warp then run loops of similar length (the pass's
-                              loops run to the warp's longest).  The windows
-                              stay where they are, so the gathers keep their locality.  Costs
-                              two kernels and 8 bytes per node at creation, which only larger
-                              meshes repay.  Not done with skip_unchanged (its 32-node tiles
-                              would lose their locality).  Every call still reads and writes
+    int32_t numbering;     /* FP64, screened kernel: 0 (default) and 2 deal the nodes of every
+                              window of 128 consecutive ids to the lanes of its block by ring
+                              length (the 32 lanes of a warp then run loops of similar
+                              length), and renumber a Form-A mesh of at least 8192 nodes whose
+                              numbering is not local (more than 45% of its triangles' edges
+                              leave their window) along a Z-order curve, at creation (8 bytes
+                              per node for the maps); 1 keeps the caller's order in both.  Not
+                              done with skip_unchanged (its 32-node tiles are the caller's),
+                              nor for binary32 meshes.  Every call still reads and writes
                               coordinates, decisions and node ids in the caller's numbering;
                               results are identical.                                         */
     void *stream;          /* cudaStream_t to run on; NULL = a stream owned by the handle    */
@@ -139,8 +136,9 @@ typedef struct sls_info {
     double max_d2_last;    /* largest squared move in the last executed pass                  */
     int64_t fp64_fallbacks;/* accept tests the screened kernel re-did in FP64 (last call)     */
     int64_t launches;      /* kernel launches issued by the last sls_smooth call (passes
-                              launched after the tolerance was met return at once; 0 from
-                              the batched and served forms)                                 */
+                              launched after the tolerance was met return at once; a small
+                              mesh's passes share one launch; 0 from the batched and served
+                              forms)                                                        */
     int64_t nodes_skipped; /* node updates not recomputed by the last sls_smooth call
                               (skip_unchanged: the nodes of the skipped tiles, summed over
                               its passes)                                                   */
@@ -238,7 +236,7 @@ sls_status sls_trim_memory(size_t keep_bytes);
 
 /* ---- batched form: many meshes of uneven size, one graph launch --------
  * Each mesh keeps its own device buffers, iteration count and tolerance; the
- * batch adds a job table and a list of 32-node work items, and runs round r
+ * batch adds a job table and a list of 128-node work items, and runs round r
  * (pass r of every mesh with passes left) as one kernel launch; all rounds of
  * a call are replayed from one CUDA graph.  Results are bit-identical to
  * smoothing each mesh alone with sls_smooth. */
@@ -249,9 +247,9 @@ sls_status sls_trim_memory(size_t keep_bytes);
  * their coordinates in place.  The coordinates at packing time are saved for
  * sls_batch_reset.  The launch shape is autotuned by timing one full batch
  * smooth per candidate, restoring the saved coordinates after each trial:
- * the chunk of consecutive 32-node tasks a warp takes (one contiguous share
- * of the list per warp, 64 in a grid stride, or 32 claimed in order from a
- * per-round counter) and, with opt == NULL or
+ * the chunk of consecutive 128-node tasks a block takes (one contiguous
+ * share of the list per block, 64 in a grid stride, or 32 claimed in order
+ * from a per-round counter) and, with opt == NULL or
  * opt->block_size == 0, the block size (64 or 128 threads); an explicit
  * block_size must be 32, 64, 96 or 128 (SLS_ERR_INVALID otherwise). */
 sls_status sls_batch_create(sls_mesh *const *meshes, int32_t k, const int32_t *iters,
@@ -269,9 +267,9 @@ sls_status sls_batch_get_coords(const sls_batch *batch, int32_t j, double *xy_ou
 sls_status sls_batch_reset(sls_batch *batch);
 
 /* The launch shape in use (chosen by the autotuner, or set below): threads
- * per block and the warp chunk (> 0: tasks per chunk in a grid stride; < 0:
+ * per block and the block's chunk (> 0: tasks per chunk in a grid stride; < 0:
  * chunks of -chunk tasks claimed in order from a per-round counter; 0: one
- * contiguous share of the task list per warp).  Either pointer may be NULL. */
+ * contiguous share of the task list per block).  Either pointer may be NULL. */
 sls_status sls_batch_shape(const sls_batch *batch, int32_t *block, int64_t *chunk);
 
 /* Sets the launch shape (block 32, 64, 96 or 128; |chunk| <= 2^20) for the
@@ -284,7 +282,7 @@ sls_status sls_batch_destroy(sls_batch *batch);
 /* ---- served form: jobs arrive over time (continuous batching) -----------
  * A scheduler thread admits queued jobs in arrival order while a bound on
  * their device footprint (coordinates, adjacency, statistics and the
- * adjacency build's scratch, about 70n + 84m bytes) fits the memory budget;
+ * adjacency build's scratch, about 194n + 108m bytes) fits the memory budget;
  * a job is also admitted when the server holds nothing else.  Builder
  * threads, each with its own stream, upload admitted jobs and build their
  * adjacency on the device (stream-ordered allocations from the library's
@@ -299,8 +297,7 @@ sls_status sls_batch_destroy(sls_batch *batch);
  * memory) that sls_submit accepts (0 = unlimited); beyond it sls_submit
  * returns SLS_ERR_BUSY.  opt: FP64 Form A with the AoS layout only
  * (SLS_ERR_INVALID otherwise).  opt's numbering applies to every job as to
- * a single mesh (by default jobs of 2^20 nodes or more are renumbered;
- * results in the caller's numbering; 4 bytes per node more while held).
+ * a single mesh (results in the caller's numbering).
  * Jobs take their device memory from the library's
  * pool (see sls_trim_memory); their inputs and results wait in page-locked
  * host memory, of which the server keeps up to 4 GiB for reuse until it is

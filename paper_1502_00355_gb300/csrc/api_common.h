@@ -10,6 +10,22 @@
 #include "device.cuh"
 #include "internal.h"
 
+namespace sls {
+
+// The window stream of a mesh's screened pass (window.cuh), in device memory
+// from the library's pool.
+struct WindowStream {
+    uint32_t *hdr = nullptr, *rows = nullptr;
+    int64_t count = 0;                  // windows
+    int width = 0;                      // nodes per window
+    WindowShape shape;
+    size_t rows_bytes = 0;
+    std::vector<int64_t> first_window;  // of every segment, and the end
+    void release(cudaStream_t s);
+};
+
+}  // namespace sls
+
 struct sls_mesh {
     sls_options opt{};
     int64_t n = 0, m = 0, n_free = 0;
@@ -24,12 +40,14 @@ struct sls_mesh {
     uint32_t *adj = nullptr;      // node_off[n] words
     uint64_t adj_words = 0;
     uint32_t *node_order = nullptr;  // n_free: processing order of the free nodes (Form A: none)
-    uint32_t *perm = nullptr;     // renumbered mesh: internal id -> the caller's id (Form B: colour
-                                  // classes contiguous; Form A: grouped by loop length in windows)
+    sls::WindowStream windows;    // what the screened pass reads
+    uint32_t *perm = nullptr;     // renumbered mesh (Form B: colour classes contiguous; Form A:
+                                  // along a Z-order curve): internal id -> the caller's id
     uint32_t *inv = nullptr;      // the caller's id -> internal id
     std::vector<int64_t> colour_off; // segments of node_order: one per colour (Form B), else one
     int32_t *tri = nullptr;       // 3m, for the histogram
-    sls::PassStats *stats = nullptr;  // one record per pass of a call
+    sls::PassStats *stats = nullptr;  // one record per pass of a call; the record before the first
+                                      // holds the blocks' barrier of the resident form
     int stats_cap = 0;
     sls::PassStats *h_stats = nullptr;  // pinned, one record
     uint8_t *accept = nullptr;    // n, when record_accept
@@ -40,6 +58,7 @@ struct sls_mesh {
     size_t l2_win_max = 0;        //            largest access-policy window the device accepts
     unsigned *xfer_bad = nullptr; // gather/scatter: set when an id was out of range
     int block = 256, grid = 0;
+    bool resident = false;        // all passes of a call in one launch (pass_screened.cu)
     bool screened = true;         // screened kernel (else the plain FP64 kernel)
     sls_info last{};
 };
@@ -70,40 +89,42 @@ struct DeviceAdjacency {
     uint32_t *node_off = nullptr;  // n+1
     uint32_t *adj = nullptr;       // adj_words
     uint64_t adj_words = 0;
+    uint32_t *perm = nullptr, *inv = nullptr;  // spatially renumbered: new id -> the caller's, and back
     int64_t n_free = 0;
     double diag = 0.0;
 };
 // Validates the mesh and builds its adjacency from device copies of the
-// coordinates (AoS) and triangles; every allocation is stream-ordered on s
-// when `async` (the caller then frees the outputs with cudaFreeAsync).
+// coordinates (AoS) and triangles, with stream-ordered allocations on s (the
+// caller frees the outputs).  renumber: a mesh whose numbering is not local
+// may be renumbered first, d_xy and d_tri with it.
 // SLS_ERR_NOT_FOUND = a node is in too many triangles: use the host build.
-sls_status build_device_adjacency(int64_t n, int64_t m, const double *d_xy, const int32_t *d_tri,
-                                  const uint8_t *h_boundary, bool async, cudaStream_t s, DeviceAdjacency &out);
+sls_status build_device_adjacency(int64_t n, int64_t m, double *d_xy, int32_t *d_tri, const uint8_t *h_boundary,
+                                  bool renumber, cudaStream_t s, DeviceAdjacency &out);
+// Whether options o let the build renumber a mesh: the screened Form-A pass
+// (Form B's colouring follows the caller's numbering, skip_unchanged's tiles
+// are the caller's) unless the caller's numbering is to be kept.
+inline bool numbers_spatially(const sls_options &o)
+{
+    return o.form == 0 && o.precision != 32 && o.kernel != SLS_KERNEL_FP64 && !o.skip_unchanged && o.numbering != 1;
+}
 // Device memory of the handles (memory.cu): stream-ordered allocations from
 // the library's pool on the current device, which keeps freed memory for
 // later handles (sls_trim_memory returns it).  Allocate and free on the
 // stream that uses the buffer; pool_free ignores NULL.
 cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t s);
 void pool_free(void *p, cudaStream_t s);
-// Form A's grouped numbering of a built adjacency (mesh_build_gpu.cu): nodes
-// listed by incident-triangle count and degree inside windows of 128 ids;
-// neighbour ids renumbered in place, *node_off replaced by the permuted
-// offsets; *perm_out (new -> old id) and, if inv_out is not NULL, *inv_out
-// (old -> new) allocated as `async` says, the caller's to free.
-sls_status group_adjacency(int64_t n, uint32_t **node_off, uint32_t *adj, bool async, cudaStream_t s,
-                           uint32_t **perm_out, uint32_t **inv_out);
-// Whether options o group the nodes of a mesh of n nodes by loop length
-// (FP64 only: the binary32 pass's loops are per lane, and there the grouping
-// only costs locality).
-inline bool groups_by_length(const sls_options &o, int64_t n)
-{
-    return o.precision != 32 && !o.skip_unchanged && (o.numbering == 2 || (o.numbering == 0 && n >= (int64_t(1) << 20)));
-}
-// Whether options o renumber a Form-A mesh of n nodes (grouped numbering).
-inline bool groups_nodes(const sls_options &o, int64_t n) { return o.form == 0 && groups_by_length(o, n); }
+// The window stream of a built adjacency (window_build.cu); segments: the id
+// ranges to cover one after another (Form B: the colour classes' bounds),
+// empty = one segment of all n nodes.  group: nodes dealt to the lanes by ring
+// length inside a window.  Synchronises s.
+sls_status build_windows(int64_t n, const std::vector<int64_t> &segments, const uint32_t *node_off,
+                         const uint32_t *adj, bool group, cudaStream_t s, WindowStream &out);
+// Whether options o deal a window's nodes to the lanes by ring length: not
+// where the caller's order is asked for, nor with skip_unchanged, whose
+// 32-node tiles are the subtiles.
+inline bool groups_lanes(const sls_options &o) { return !o.skip_unchanged && o.numbering != 1; }
 // Device adjacency build of a mesh handle; SLS_ERR_NOT_FOUND = use the host build.
-sls_status build_device_mesh(sls_mesh *M, const double *d_xy, const int32_t *d_tri, const uint8_t *h_boundary,
-                             cudaStream_t s);
+sls_status build_device_mesh(sls_mesh *M, double *d_xy, int32_t *d_tri, const uint8_t *h_boundary, cudaStream_t s);
 // The processing order of the free nodes, from the adjacency on the device
 // (mesh_build_gpu.cu): fills M->node_order.
 sls_status build_node_order(sls_mesh *M, cudaStream_t s);

@@ -1,8 +1,8 @@
 // batch.cu -- the batched form: many meshes of uneven size smoothed together.
 //
 // The meshes keep their own device buffers (from sls_mesh_create); the batch
-// adds a job table (one JobDesc per mesh), a list of warp tasks (32 nodes of
-// one mesh each) ordered by descending iteration count, and one statistics
+// adds a job table (one JobDesc per mesh), a list of window tasks (128 nodes
+// of one mesh each) ordered by descending iteration count, and one statistics
 // record per mesh and pass.  Round r runs pass r of every mesh that still
 // has passes left; the rounds of a whole sls_batch_smooth call are captured
 // once into a CUDA graph and replayed with a single cudaGraphLaunch.  Every
@@ -29,7 +29,7 @@ struct sls_batch {
     bool own_stream = false;
     JobDesc *d_jobs = nullptr;
     JobDesc *h_jobs = nullptr;         // pinned staging of the job table
-    WarpTask *d_tasks = nullptr;
+    WindowTask *d_tasks = nullptr;
     int64_t ntasks = 0;
     std::vector<int64_t> round_tasks;  // tasks taking part in round r
     PassStats *d_stats = nullptr;
@@ -38,7 +38,8 @@ struct sls_batch {
     std::vector<double *> d_start;     // per mesh: the packed starting coordinates
     int rounds = 0;
     int block = 128, grid = 0;
-    int64_t chunk = 0;                 // tasks per warp chunk (launch_batch_pass)
+    WindowShape shape;                 // covers every mesh's windows
+    int64_t chunk = 0;                 // tasks per block chunk (launch_batch_pass)
     unsigned long long *d_claim = nullptr;  // one chunk counter per round (dynamic chunks)
     cudaGraphExec_t exec = nullptr;
 };
@@ -76,7 +77,7 @@ sls_status build_graph(sls_batch *B)
     cudaError_t err = cudaSuccess;
     for (int r = 0; r < B->rounds && err == cudaSuccess; ++r)
         err = launch_batch_pass(B->d_jobs, B->d_tasks, B->round_tasks[r], r, B->layout, B->block, B->grid,
-                                B->stream, B->chunk, B->d_claim + r);
+                                B->shape, B->stream, B->chunk, B->d_claim + r);
     cudaError_t e2 = cudaStreamEndCapture(B->stream, &g);
     if (err != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
@@ -110,7 +111,10 @@ sls_status run(sls_batch *B, sls_info *infos)
         J.max_iter = B->iters[mi];
         J.base_round = 0;
         J.cur0 = M->cur;
-        J.pad = 0;
+        J.windows = (int32_t)M->windows.count;
+        J.bits = M->windows.shape.bits;
+        J.win_hdr = M->windows.hdr;
+        J.win_rows = M->windows.rows;
         J.accept = M->accept;
     }
     BATCH_TRY(cudaMemcpyAsync(B->d_jobs, B->h_jobs, sizeof(JobDesc) * k, cudaMemcpyHostToDevice, B->stream),
@@ -201,7 +205,7 @@ sls_status autotune(sls_batch *B, bool tune_block)
     for (size_t c = 0; c < cands.size() && st == SLS_OK; ++c) {
         B->block = cands[c].block;
         B->chunk = cands[c].chunk;
-        B->grid = device_sm_count() * batch_pass_occupancy(B->layout, B->block);
+        B->grid = device_sm_count() * batch_pass_occupancy(B->layout, B->block, B->shape);
         if (B->rounds > 0) st = build_graph(B);
         if (st != SLS_OK) break;
         cudaEventRecord(e0, B->stream);
@@ -225,7 +229,7 @@ sls_status autotune(sls_batch *B, bool tune_block)
     }
     B->block = best.block;
     B->chunk = best.chunk;
-    B->grid = device_sm_count() * batch_pass_occupancy(B->layout, B->block);
+    B->grid = device_sm_count() * batch_pass_occupancy(B->layout, B->block, B->shape);
     return SLS_OK;
 }
 
@@ -277,12 +281,21 @@ sls_status sls_batch_create(sls_mesh *const *meshes, int32_t k, const int32_t *i
     B->order.resize(k);
     std::iota(B->order.begin(), B->order.end(), 0);
     std::stable_sort(B->order.begin(), B->order.end(), [B](int a, int b) { return B->iters[a] > B->iters[b]; });
-    std::vector<WarpTask> tasks;
+    for (int j = 0; j < k; ++j) {
+        // a mesh made for the plain FP64 kernel has no window stream yet
+        sls_mesh *M = meshes[j];
+        if (M->windows.hdr) continue;
+        sls_status st = build_windows(M->n, {}, M->node_off, M->adj, groups_lanes(M->opt), M->stream, M->windows);
+        if (st == SLS_OK && cudaStreamSynchronize(M->stream) != cudaSuccess) st = fail(SLS_ERR_CUDA, "windows");
+        if (st != SLS_OK) return fail_free(st);
+    }
+    std::vector<WindowTask> tasks;
     std::vector<int64_t> tasks_upto(k + 1, 0);
     B->stats_off.resize(k);
     for (int slot = 0; slot < k; ++slot) {
         sls_mesh *M = B->meshes[B->order[slot]];
-        for (int64_t f = 0; f < M->n; f += 32) tasks.push_back(WarpTask{slot, (int32_t)f});
+        for (int64_t w = 0; w < M->windows.count; ++w) tasks.push_back(WindowTask{slot, (int32_t)w});
+        B->shape.cover(M->windows.shape);
         tasks_upto[slot + 1] = (int64_t)tasks.size();
         B->stats_off[slot] = B->nstats;
         B->nstats += std::max(1, B->iters[B->order[slot]]);
@@ -296,14 +309,14 @@ sls_status sls_batch_create(sls_mesh *const *meshes, int32_t k, const int32_t *i
         B->round_tasks[r] = tasks_upto[slots];
     }
     if (cudaMalloc(&B->d_jobs, sizeof(JobDesc) * k) != cudaSuccess ||
-        cudaMalloc(&B->d_tasks, sizeof(WarpTask) * std::max<int64_t>(1, B->ntasks)) != cudaSuccess ||
+        cudaMalloc(&B->d_tasks, sizeof(WindowTask) * std::max<int64_t>(1, B->ntasks)) != cudaSuccess ||
         cudaMalloc(&B->d_stats, sizeof(PassStats) * B->nstats) != cudaSuccess ||
         cudaMalloc(&B->d_claim, sizeof(unsigned long long) * std::max(1, B->rounds)) != cudaSuccess ||
         cudaMallocHost(&B->h_jobs, sizeof(JobDesc) * k) != cudaSuccess) {
         cudaGetLastError();
         return fail_free(fail(SLS_ERR_OOM, "batch allocation failed"));
     }
-    if (cudaMemcpy(B->d_tasks, tasks.data(), sizeof(WarpTask) * B->ntasks, cudaMemcpyHostToDevice) != cudaSuccess)
+    if (cudaMemcpy(B->d_tasks, tasks.data(), sizeof(WindowTask) * B->ntasks, cudaMemcpyHostToDevice) != cudaSuccess)
         return fail_free(fail(SLS_ERR_CUDA, "upload warp tasks"));
     B->d_start.assign(k, nullptr);
     for (int j = 0; j < k; ++j) {
@@ -322,7 +335,7 @@ sls_status sls_batch_create(sls_mesh *const *meshes, int32_t k, const int32_t *i
             return fail_free(fail(SLS_ERR_INVALID, "batch block_size must be 32, 64, 96 or 128"));
         B->block = opt->block_size;
     }
-    B->grid = device_sm_count() * batch_pass_occupancy(B->layout, B->block);
+    B->grid = device_sm_count() * batch_pass_occupancy(B->layout, B->block, B->shape);
     {
         // autotune on the packed meshes (the block size too unless it was
         // given), then restore their coordinates
@@ -372,7 +385,7 @@ sls_status sls_batch_set_shape(sls_batch *B, int32_t block, int64_t chunk)
     }
     B->block = block;
     B->chunk = chunk;
-    B->grid = device_sm_count() * batch_pass_occupancy(B->layout, B->block);
+    B->grid = device_sm_count() * batch_pass_occupancy(B->layout, B->block, B->shape);
     return SLS_OK;
 }
 

@@ -16,6 +16,20 @@ struct PassStats {
     unsigned int nodes_skipped;     // node updates not recomputed (unchanged inputs)
 };
 
+// What the windows of a mesh need of a block's shared memory: the largest
+// number of staged entries, halo nodes and hot rows of any of them, and the
+// bits of a list entry (window.cuh).
+struct WindowShape {
+    int entries = 0, halo = 0, hot = 0, bits = 8;
+    void cover(const WindowShape &o)
+    {
+        entries = entries > o.entries ? entries : o.entries;
+        halo = halo > o.halo ? halo : o.halo;
+        hot = hot > o.hot ? hot : o.hot;
+        bits = bits > o.bits ? bits : o.bits;
+    }
+};
+
 // Arguments of one Jacobi pass over one mesh.
 struct PassArgs {
     const double *in;          // coordinates X^q   (AoS: x0 y0 x1 y1 ...; SoA: x[n] then y[n])
@@ -23,10 +37,11 @@ struct PassArgs {
     const uint32_t *node_off;  // n+1 word offsets into adj
     const uint32_t *adj;       // per-node words: meta, neighbours, triangle codes
     int64_t n;
-    const uint32_t *order;     // nullptr: every node in index order; else the nodes to update
-    int64_t norder;            // (one colour class of Form B) and their number
-    int ranged;                // 1 (order null): only the nodes first .. first + count - 1
-    int64_t first, count;      // (a contiguous colour class of a renumbered Form-B mesh)
+    int ranged;                // 1: only the nodes first .. first + count - 1 (a contiguous
+    int64_t first, count;      // colour class of a renumbered Form-B mesh); 0: every node
+    const uint32_t *win_hdr;   // screened pass: the window stream (window.cuh) and the
+    const uint32_t *win_rows;  // windows win_first .. win_first + win_count - 1 of it
+    int64_t win_first, win_count;
     PassStats *stats;          // stats[q] receives this pass
     int q;                     // pass index within the call
     int strict;                // 1: accept iff q_new > q_old
@@ -63,14 +78,15 @@ struct JobDesc {
     int32_t max_iter;          // passes to run at most
     int32_t base_round;        // the job's pass q runs in round base_round + q
     int32_t cur0;              // which array holds the job's starting coordinates
-    int32_t pad;
+    int32_t windows, bits;     // window stream
+    const uint32_t *win_hdr, *win_rows;
     uint8_t *accept;           // n decisions, or nullptr
 };
 
-// 32 consecutive nodes [first, first + 32) of one job.
-struct WarpTask {
+// One window of one job.
+struct WindowTask {
     int32_t job;
-    int32_t first;
+    int32_t window;
 };
 
 constexpr uint32_t kMetaFixed = 0x80000000u;
@@ -170,6 +186,33 @@ __device__ __forceinline__ double alpha_fp64(double ax, double ay, double bx, do
     double l2 = __dadd_rn(__dmul_rn(e2x, e2x), __dmul_rn(e2y, e2y));
     double l3 = __dadd_rn(__dmul_rn(e3x, e3x), __dmul_rn(e3y, e3y));
     double s = __dadd_rn(__dadd_rn(l1, l2), l3);
+    return s > 0.0 ? __ddiv_rn(__dmul_rn(kTwoSqrt3, cross), s) : 0.0;
+}
+
+// alpha_fp64 of an incident triangle with the node at x in slot `slot` and
+// the other two vertices A before B in the stored order.  With u = x - A,
+// w = x - B, v = B - A every edge of the stored order is one of +-u, +-w, +-v,
+// and negation commutes with rounding, so
+//   slot 0: cross = u x w,     s = (|u|^2 + |w|^2) + |v|^2
+//   slot 1: cross = u x v,     s = (|u|^2 + |v|^2) + |w|^2
+//   slot 2: cross = -(u x v),  s = (|v|^2 + |u|^2) + |w|^2 (the same sum)
+// give bit for bit alpha_fp64 of the reordered points, and lanes with
+// different slots run the same instructions.
+__device__ __forceinline__ double alpha_at_slot(uint32_t slot, double x, double y, double ax, double ay, double bx,
+                                                double by)
+{
+    const double kTwoSqrt3 = 3.4641016151377544;  // nearest double to 2*sqrt(3)
+    const double ux = __dsub_rn(x, ax), uy = __dsub_rn(y, ay);
+    const double wx = __dsub_rn(x, bx), wy = __dsub_rn(y, by);
+    const double vx = __dsub_rn(bx, ax), vy = __dsub_rn(by, ay);
+    const double lu = __dadd_rn(__dmul_rn(ux, ux), __dmul_rn(uy, uy));
+    const double lw = __dadd_rn(__dmul_rn(wx, wx), __dmul_rn(wy, wy));
+    const double lv = __dadd_rn(__dmul_rn(vx, vx), __dmul_rn(vy, vy));
+    const bool s0 = slot == 0u;
+    const double zx = s0 ? wx : vx, zy = s0 ? wy : vy;
+    double cross = __dsub_rn(__dmul_rn(ux, zy), __dmul_rn(uy, zx));
+    cross = slot == 2u ? -cross : cross;
+    const double s = __dadd_rn(__dadd_rn(lu, s0 ? lw : lv), s0 ? lv : lw);
     return s > 0.0 ? __ddiv_rn(__dmul_rn(kTwoSqrt3, cross), s) : 0.0;
 }
 

@@ -8,10 +8,9 @@
 //   s - q0 N = (Ms 2^(Es - Eq) - Mq N) 2^Eq = r 2^Eq,
 // so s/N = (Mq + r/N) 2^Eq and the rounded quotient is Mq + k with k the
 // integer nearest to r/N, |k| <= 2.  Adding k to
-// the bit pattern of q0 steps through the representable values, also onto
-// the top of the binade (Mq + k = 2^53).  Where Mq + k leaves [2^52, 2^53]
-// the candidates are spaced differently; that case, and operands where
-// anything could under- or overflow, take the IEEE division.
+// the bit pattern of q0 steps through the representable values.  Where Mq + k
+// leaves the binade the candidates are spaced differently; that case, and
+// operands where anything could under- or overflow, take the IEEE division.
 //
 // Compiles for the host too, so the CPU tests run this code against the
 // host's IEEE division.
@@ -78,22 +77,21 @@ SLS_DS_HD uint64_t div_small_bits(uint64_t sb, uint32_t N, double y, double fN)
     if (es - 63u > 1937u) return bits_of(div_rn(of_bits(sb), fN));
     const uint64_t qb = bits_of(mul_rn(of_bits(sb), y));
     const uint32_t eq = (uint32_t)(qb >> 52) & 0x7ffu;
-    const uint64_t ms = (sb & 0x000fffffffffffffull) | 0x0010000000000000ull;
-    const uint64_t mq = (qb & 0x000fffffffffffffull) | 0x0010000000000000ull;
-    // s/N < s, so eq <= es; s/N >= s/16, so es - eq <= 5
-    const uint32_t de = es - eq;
-    const int64_t r = (int64_t)(ms << de) - (int64_t)(mq * N);
+    // s/N < s, so eq <= es; s/N >= s/16, so es - eq <= 5.  The remainder is
+    // small, |r| <= 2 N, so its low 32 bits are all of it (the leading bits of
+    // both significands lie above them).
+    const int32_t n = (int32_t)N;
+    const int32_t r = (int32_t)(((uint32_t)sb << ((es - eq) & 31u)) - (uint32_t)qb * N);
     // |r/N| against 1/2 and 3/2.  A quotient of two doubles is never exactly
     // halfway between two doubles (s = N (2M + 1) 2^(E-1) would need more than
     // 53 significant bits), so no tie can occur.
-    const int64_t n = (int64_t)N, a2 = r < 0 ? -2 * r : 2 * r;
-    if (a2 > 5 * n) return bits_of(div_rn(of_bits(sb), fN));
-    int64_t k = (int64_t)(a2 > n) + (int64_t)(a2 > 3 * n);
-    if (r < 0) k = -k;
-    const int64_t mk = (int64_t)mq + k;
-    if (mk < (int64_t)0x0010000000000000ll || mk > (int64_t)0x0020000000000000ll)
-        return bits_of(div_rn(of_bits(sb), fN));
-    return qb + (uint64_t)k;
+    const int32_t a2 = r < 0 ? -2 * r : 2 * r;
+    const int32_t k = (a2 > n ? 1 : 0) + (a2 > 3 * n ? 1 : 0);
+    const uint64_t qk = qb + (uint64_t)(int64_t)(r < 0 ? -k : k);
+    // a step out of the binade (also onto its top, which is rare) is left to
+    // the division
+    if (((uint32_t)((qk ^ qb) >> 32) & 0xfff00000u) != 0u || a2 > 5 * n) return bits_of(div_rn(of_bits(sb), fN));
+    return qk;
 }
 
 }  // namespace divs

@@ -17,19 +17,31 @@ int pass_fp64_occupancy(int layout, int block);
 // division by the degree as one FP64 multiplication plus an exact integer
 // correction, FP32 screening of the accept test, FP64 quality only where the
 // screen cannot decide (bit-identical results).
-cudaError_t launch_pass_screened(const PassArgs &a, int layout, int block, int grid, cudaStream_t s);
-int pass_screened_occupancy(int layout, int block);
+// shape: of the mesh's windows (WindowStream::shape).
+cudaError_t launch_pass_screened(const PassArgs &a, int layout, int block, int grid, const WindowShape &shape, cudaStream_t s);
+int pass_screened_occupancy(int layout, int block, const WindowShape &shape);
+
+// Passes a.q .. a.q + passes - 1 of a mesh with at most one window per resident
+// block (resident_fits), in one cooperative launch that stops at the
+// tolerance like separate ones; the passes ping-pong between a.in and a.out.
+// barrier: kBarrierWords device words, zero at the launch; word 1 is set when a
+// wait between the blocks ran out, and the passes are then incomplete.
+constexpr int kBarrierWords = 2;
+bool resident_fits(const PassArgs &a, int layout, int block, const WindowShape &shape);
+cudaError_t launch_resident(const PassArgs &a, int layout, int block, const WindowShape &shape, int passes,
+                            unsigned *barrier, cudaStream_t s);
 
 // One round of the batched / served form over all active jobs' tasks.
-// chunk > 0: tasks per warp chunk, taken in a grid stride; chunk < 0: chunks
+// chunk > 0: tasks per block chunk, taken in a grid stride; chunk < 0: chunks
 // of -chunk tasks claimed in order from *claim (zero at the launch); 0 = one
-// contiguous share of the task list per warp.
-cudaError_t launch_batch_pass(const JobDesc *jobs, const WarpTask *tasks, int64_t ntasks, int round,
-                              int layout, int block, int grid, cudaStream_t s, int64_t chunk,
+// contiguous share of the task list per block.  shape covers every job's
+// windows.
+cudaError_t launch_batch_pass(const JobDesc *jobs, const WindowTask *tasks, int64_t ntasks, int round, int layout,
+                              int block, int grid, const WindowShape &shape, cudaStream_t s, int64_t chunk,
                               unsigned long long *claim);
-int batch_pass_occupancy(int layout, int block);
-// The warp tasks of the na jobs of a table (job j's tasks from task_off[j]).
-cudaError_t launch_expand_tasks(const JobDesc *jobs, const int64_t *task_off, int na, WarpTask *tasks,
+int batch_pass_occupancy(int layout, int block, const WindowShape &shape);
+// The window tasks of the na jobs of a table (job j's tasks from task_off[j]).
+cudaError_t launch_expand_tasks(const JobDesc *jobs, const int64_t *task_off, int na, WindowTask *tasks,
                                 cudaStream_t s);
 // Record of round `round` of each of the na jobs (pass round - base_round,
 // clamped to the job's last pass) into out[0 .. na).
@@ -66,8 +78,7 @@ cudaError_t launch_gather_nodes(const double *xy, int layout, int64_t n, const i
 cudaError_t launch_scatter_nodes(double *xy0, double *xy1, int layout, int64_t n, const int32_t *idx, int64_t k,
                                  const uint32_t *inv, const double *in, unsigned *bad, int grid, cudaStream_t s);
 
-// A renumbered mesh (Form B: colour classes contiguous; Form A: nodes grouped
-// by loop length inside windows of ids).  Coordinates are
+// A renumbered mesh (Form B: colour classes contiguous).  Coordinates are
 // doubles or, with f32, floats, in the layout; perm maps a new id to the
 // caller's.
 // dst[k] = src[perm[k]]

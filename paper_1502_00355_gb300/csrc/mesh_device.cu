@@ -36,6 +36,22 @@ static void to_soa(const double *xy, int64_t n, std::vector<double> &tmp)
     }
 }
 
+// M->stats for `cap` passes, with one record in front of them.
+static sls_status alloc_stats(sls_mesh *M, int cap)
+{
+    PassStats *base = nullptr;
+    sls_status st = dev_alloc(M, (void **)&base, sizeof(PassStats) * ((size_t)cap + 1), "pass statistics");
+    M->stats = st == SLS_OK ? base + 1 : nullptr;
+    M->stats_cap = st == SLS_OK ? cap : 0;
+    return st;
+}
+
+static void free_stats(sls_mesh *M)
+{
+    if (M->stats) pool_free(M->stats - 1, M->stream);
+    M->stats = nullptr;
+}
+
 // Common set-up of a handle: stream, statistics, accept mask, launch shape.
 static sls_status mesh_setup(sls_mesh *M, const sls_options &o)
 {
@@ -48,8 +64,7 @@ static sls_status mesh_setup(sls_mesh *M, const sls_options &o)
         M->own_stream = true;
     }
     sls_status st;
-    M->stats_cap = 256;
-    if ((st = dev_alloc(M, (void **)&M->stats, sizeof(PassStats) * M->stats_cap, "pass statistics")) != SLS_OK) return st;
+    if ((st = alloc_stats(M, 256)) != SLS_OK) return st;
     SLS_CUDA_TRY(cudaMallocHost((void **)&M->h_stats, sizeof(PassStats)), "cudaMallocHost");
     if (o.record_accept) {
         if ((st = dev_alloc(M, (void **)&M->accept, (size_t)M->n, "accept mask")) != SLS_OK) return st;
@@ -77,9 +92,32 @@ static sls_status mesh_setup(sls_mesh *M, const sls_options &o)
     }
     sls_status pst = noalloc_prepare();
     if (pst != SLS_OK) return pst;
-    M->grid = device_sm_count() * (M->f32        ? pass_f32_occupancy(o.layout, M->block)
-                                   : M->screened ? pass_screened_occupancy(o.layout, M->block)
-                                                 : pass_fp64_occupancy(o.layout, M->block));
+    if (!M->screened)
+        M->grid = device_sm_count() * (M->f32 ? pass_f32_occupancy(o.layout, M->block)
+                                              : pass_fp64_occupancy(o.layout, M->block));
+    return SLS_OK;
+}
+
+// The last steps of a creation, once the adjacency stands: Form B's colouring
+// and renumbering, the window stream and launch shape of the screened pass,
+// the tile lists of skip_unchanged.
+static sls_status finish_creation(sls_mesh *M)
+{
+    sls_status st = build_node_order(M, M->stream);
+    if (st != SLS_OK) return st;
+    if (M->screened) {
+        st = build_windows(M->n, M->opt.form == 1 ? M->colour_off : std::vector<int64_t>(), M->node_off, M->adj,
+                           groups_lanes(M->opt), M->stream, M->windows);
+        if (st != SLS_OK) return st;
+        M->grid = device_sm_count() * pass_screened_occupancy(M->opt.layout, M->block, M->windows.shape);
+        PassArgs a{};
+        a.win_count = M->windows.count;
+        M->resident = M->opt.form == 0 && !M->opt.copy_back && !M->opt.skip_unchanged && !M->opt.l2_window &&
+                      resident_fits(a, M->opt.layout, M->block, M->windows.shape);
+    }
+    if ((st = build_tile_halo(M, M->stream)) != SLS_OK) return st;
+    // a batch or the allocation-free form runs the mesh on other streams
+    SLS_CUDA_TRY(cudaStreamSynchronize(M->stream), "mesh create");
     return SLS_OK;
 }
 
@@ -146,8 +184,7 @@ sls_status mesh_upload(sls_mesh *M, const HostMesh &hm, const double *xy, const 
                                  cudaMemcpyHostToDevice, M->stream), "upload triangles");
     SLS_CUDA_TRY(cudaStreamSynchronize(M->stream), "upload");
     if ((st = narrow_coordinates(M)) != SLS_OK) return st;
-    if ((st = build_node_order(M, M->stream)) != SLS_OK) return st;
-    return build_tile_halo(M, M->stream);
+    return finish_creation(M);
 }
 
 sls_status mesh_create_on_device(sls_mesh *M, const double *xy, int64_t n, const int32_t *tri, int64_t m,
@@ -172,10 +209,10 @@ sls_status mesh_create_on_device(sls_mesh *M, const double *xy, int64_t n, const
         HostMesh hm;
         st = build_host_mesh(xy, n, tri, m, boundary, hm);
         if (st != SLS_OK) return st;
-        pool_free(M->node_off, M->stream);
-        pool_free(M->adj, M->stream);
-        M->node_off = nullptr;
-        M->adj = nullptr;
+        // (the device build may have renumbered what was uploaded)
+        SLS_CUDA_TRY(cudaMemcpyAsync(aos, xy, cbytes, cudaMemcpyHostToDevice, M->stream), "upload coordinates");
+        SLS_CUDA_TRY(cudaMemcpyAsync(M->tri, tri, sizeof(int32_t) * 3 * (size_t)m, cudaMemcpyHostToDevice, M->stream),
+                     "upload triangles");
         M->n_free = hm.n_free;
         M->diag = hm.diag;
         M->adj_words = hm.node_off[hm.n];
@@ -193,8 +230,7 @@ sls_status mesh_create_on_device(sls_mesh *M, const double *xy, int64_t n, const
     SLS_CUDA_TRY(cudaMemcpyAsync(M->xy[1], M->xy[0], cbytes, cudaMemcpyDeviceToDevice, M->stream), "copy coordinates");
     SLS_CUDA_TRY(cudaStreamSynchronize(M->stream), "mesh create");
     if ((st = narrow_coordinates(M)) != SLS_OK) return st;
-    if ((st = build_node_order(M, M->stream)) != SLS_OK) return st;
-    return build_tile_halo(M, M->stream);
+    return finish_creation(M);
 }
 
 void mesh_release(sls_mesh *M)
@@ -205,10 +241,11 @@ void mesh_release(sls_mesh *M)
     pool_free(M->node_off, M->stream);
     pool_free(M->adj, M->stream);
     pool_free(M->node_order, M->stream);
+    M->windows.release(M->stream);
     pool_free(M->perm, M->stream);
     pool_free(M->inv, M->stream);
     pool_free(M->tri, M->stream);
-    pool_free(M->stats, M->stream);
+    free_stats(M);
     pool_free(M->accept, M->stream);
     pool_free(M->halo, M->stream);
     pool_free(M->chg[0], M->stream);
@@ -240,9 +277,12 @@ static cudaError_t launch_pass(const sls_mesh *M, const PassArgs &a)
 {
     if (M->opt.l2_window) set_l2_window(M, a.in, (M->f32 ? sizeof(float) : sizeof(double)) * 2 * (size_t)M->n);
     if (M->f32) return launch_pass_f32(a, M->opt.layout, M->block, M->grid, M->stream);
-    return M->screened ? launch_pass_screened(a, M->opt.layout, M->block, M->grid, M->stream)
+    return M->screened ? launch_pass_screened(a, M->opt.layout, M->block, M->grid, M->windows.shape, M->stream)
                        : launch_pass_fp64(a, M->opt.layout, M->block, M->grid, M->stream);
 }
+
+// Passes of one launch of the resident form.
+constexpr int kResidentPasses = 4096;
 
 sls_status mesh_run(sls_mesh *M, int32_t max_iter, double tol_rel, sls_info &info)
 {
@@ -250,17 +290,12 @@ sls_status mesh_run(sls_mesh *M, int32_t max_iter, double tol_rel, sls_info &inf
     if (max_iter == 0) return SLS_OK;
     if (M->stats_cap < max_iter) {
         cudaStreamSynchronize(M->stream);
-        pool_free(M->stats, M->stream);
-        M->stats = nullptr;
-        int cap = std::max(max_iter, 2 * M->stats_cap);
-        sls_status st = dev_alloc(M, (void **)&M->stats, sizeof(PassStats) * cap, "pass statistics");
-        if (st != SLS_OK) {
-            M->stats_cap = 0;
-            return st;
-        }
-        M->stats_cap = cap;
+        const int cap = std::max(max_iter, 2 * M->stats_cap);
+        free_stats(M);
+        sls_status st = alloc_stats(M, cap);
+        if (st != SLS_OK) return st;
     }
-    SLS_CUDA_TRY(cudaMemsetAsync(M->stats, 0, sizeof(PassStats) * max_iter, M->stream), "cudaMemset");
+    SLS_CUDA_TRY(cudaMemsetAsync(M->stats - 1, 0, sizeof(PassStats) * ((size_t)max_iter + 1), M->stream), "cudaMemset");
     const bool tol_active = tol_rel > 0.0;
     const double thr = tolerance_threshold(tol_rel, M->diag);
     unsigned long long thr_bits;
@@ -270,8 +305,9 @@ sls_status mesh_run(sls_mesh *M, int32_t max_iter, double tol_rel, sls_info &inf
     a.node_off = M->node_off;
     a.adj = M->adj;
     a.n = M->n;
-    a.order = M->node_order;
-    a.norder = M->n_free;
+    a.win_hdr = M->windows.hdr;
+    a.win_rows = M->windows.rows;
+    a.win_count = M->windows.count;
     a.stats = M->stats;
     a.strict = M->opt.accept_strict;
     a.tol_active = tol_active ? 1 : 0;
@@ -279,13 +315,26 @@ sls_status mesh_run(sls_mesh *M, int32_t max_iter, double tol_rel, sls_info &inf
     a.accept = M->accept;
     const bool form_b = M->opt.form == 1;
     const int cb = form_b ? 0 : M->opt.copy_back;
-    const int chunk = M->opt.passes_per_check;
+    unsigned *const barrier = reinterpret_cast<unsigned *>(M->stats - 1);
+    // the resident form stops at the tolerance by itself; between its launches
+    // other work gets its turn
+    const int chunk = M->resident ? kResidentPasses : M->opt.passes_per_check;
     const int nseg = (int)M->colour_off.size() - 1;
     int launched = 0;
     int64_t kernels = 0;
     while (launched < max_iter) {
         const int end = std::min(launched + chunk, (int)max_iter);
-        for (int q = launched; q < end; ++q) {
+        if (M->resident) {
+            a.q = launched;
+            a.in = M->xy[M->cur ^ (launched & 1)];
+            a.out = M->xy[M->cur ^ (launched & 1) ^ 1];
+            if (launched > 0)
+                SLS_CUDA_TRY(cudaMemsetAsync(barrier, 0, sizeof(unsigned) * kBarrierWords, M->stream), "cudaMemset");
+            SLS_CUDA_TRY(launch_resident(a, M->opt.layout, M->block, M->windows.shape, end - launched, barrier, M->stream),
+                         "pass kernel");
+            ++kernels;
+        }
+        for (int q = launched; q < end && !M->resident; ++q) {
             a.q = q;
             if (form_b) {
                 // Form B: the colour classes in turn, in place (Eq. 3).  A
@@ -294,10 +343,13 @@ sls_status mesh_run(sls_mesh *M, int32_t max_iter, double tol_rel, sls_info &inf
                 // the mesh is renumbered: class c is the id range colour_off[c] ..
                 a.in = a.out = M->xy[M->cur];
                 for (int c = 0; c < std::max(nseg, 1); ++c) {
-                    a.order = nullptr;
                     a.ranged = 1;
                     a.first = nseg > 0 ? M->colour_off[c] : 0;
                     a.count = nseg > 0 ? M->colour_off[c + 1] - M->colour_off[c] : 0;
+                    if (M->screened) {
+                        a.win_first = nseg > 0 ? M->windows.first_window[c] : 0;
+                        a.win_count = nseg > 0 ? M->windows.first_window[c + 1] - a.win_first : 0;
+                    }
                     SLS_CUDA_TRY(launch_pass(M, a), "pass kernel");
                     ++kernels;
                 }
@@ -306,8 +358,6 @@ sls_status mesh_run(sls_mesh *M, int32_t max_iter, double tol_rel, sls_info &inf
             const int src = cb ? M->cur : (M->cur ^ (q & 1));
             a.in = M->xy[src];
             a.out = M->xy[src ^ 1];
-            a.order = nullptr;
-            a.norder = 0;
             if (M->halo) {  // unchanged-tile skipping from the second pass of a call on
                 a.halo = M->halo;
                 a.chg_prev = M->chg[(q + 1) & 1];
@@ -340,10 +390,13 @@ sls_status mesh_run(sls_mesh *M, int32_t max_iter, double tol_rel, sls_info &inf
         SLS_CUDA_TRY(cudaStreamSynchronize(M->stream), "pass");
         if (cudaCtxResetPersistingL2Cache() != cudaSuccess) cudaGetLastError();
     }
-    std::vector<PassStats> hs(launched);
-    SLS_CUDA_TRY(cudaMemcpyAsync(hs.data(), M->stats, sizeof(PassStats) * launched,
+    std::vector<PassStats> all((size_t)launched + 1);
+    SLS_CUDA_TRY(cudaMemcpyAsync(all.data(), M->stats - 1, sizeof(PassStats) * all.size(),
                                  cudaMemcpyDeviceToHost, M->stream), "read pass statistics");
     SLS_CUDA_TRY(cudaStreamSynchronize(M->stream), "passes");
+    const PassStats *hs = all.data() + 1;
+    if (reinterpret_cast<const unsigned *>(all.data())[1])
+        return fail(SLS_ERR_TIMEOUT, "a wait between the blocks of a launch ran out");
     int it = 0;
     long long fb = 0, sk = 0;
     for (; it < launched && hs[it].executed; ++it) {

@@ -115,8 +115,9 @@ extern "C" sls_status sls_smooth_noalloc(const sls_mesh *M, double *xy_in, doubl
     a.node_off = M->node_off;
     a.adj = M->adj;
     a.n = M->n;
-    a.order = nullptr;
-    a.norder = 0;
+    a.win_hdr = M->windows.hdr;
+    a.win_rows = M->windows.rows;
+    a.win_count = M->windows.count;
     a.stats = stats;
     a.strict = M->opt.accept_strict;
     a.tol_active = tol_active ? 1 : 0;
@@ -132,7 +133,7 @@ extern "C" sls_status sls_smooth_noalloc(const sls_mesh *M, double *xy_in, doubl
             a.in = buf[q & 1];
             a.out = buf[(q + 1) & 1];
             a.q = q;
-            e = M->screened ? launch_pass_screened(a, 0, M->block, M->grid, s)
+            e = M->screened ? launch_pass_screened(a, 0, M->block, M->grid, M->windows.shape, s)
                             : launch_pass_fp64(a, 0, M->block, M->grid, s);
             if (e != cudaSuccess) return cuda_fail(e, "pass kernel");
         }

@@ -105,8 +105,8 @@ __device__ __forceinline__ float alpha_at(const float *in, int64_t n, const uint
 // has about 1.4 nodes in 10,000 above 12).
 constexpr int kRingMax = 12;
 
-// One pass over every node (a.order null) or over the listed nodes (one
-// colour class of Form B, in place).  a.in / a.out hold floats.  Each thread
+// One pass over every node, or over the ids of one colour class of Form B
+// (in place).  a.in / a.out hold floats.  Each thread
 // keeps its node's ring in its own column of a shared buffer (stride: block);
 // nodes with larger rings read their neighbours from global memory.
 template <int LAYOUT>
@@ -122,10 +122,10 @@ __global__ void __launch_bounds__(256) pass_f32_kernel(PassArgs a)
 
     unsigned best = 0u;  // bits of the largest squared move (non-negative floats order as integers)
     unsigned long long nacc = 0ull;
-    const int64_t cnt = a.order ? a.norder : (a.ranged ? a.count : a.n);
+    const int64_t cnt = a.ranged ? a.count : a.n;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < cnt; j += stride) {
-        const int64_t i = a.order ? (int64_t)__ldg(a.order + j) : a.first + j;
+        const int64_t i = a.first + j;
         const uint32_t off = __ldg(a.node_off + i);
         const uint32_t meta = __ldg(a.adj + off);
         if (meta & kMetaFixed) {

@@ -26,10 +26,10 @@ __global__ void __launch_bounds__(1024) pass_fp64_kernel(PassArgs a)
 
     unsigned long long best = 0ull, nacc = 0ull;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    // every node, or (a colour class of Form B) the listed free nodes
-    const int64_t cnt = a.order ? a.norder : (a.ranged ? a.count : a.n);
+    // every node, or (a colour class of Form B) a range of ids
+    const int64_t cnt = a.ranged ? a.count : a.n;
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < cnt; j += stride) {
-        const int64_t i = a.order ? (int64_t)__ldg(a.order + j) : a.first + j;
+        const int64_t i = a.first + j;
         const uint32_t meta = __ldg(a.adj + __ldg(a.node_off + i));
         if (meta & kMetaFixed) {
             if (a.accept) a.accept[i] = 0;
@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(1024) pass_fp64_kernel(PassArgs a)
         }
         unsigned long long bits;
         bool ok, moved;
-        exact_update<LAYOUT>(a, i, 0u, 0u, 0ull, 0ull, bits, ok, moved);
+        exact_update<LAYOUT>(a, i, bits, ok, moved);
         best = bits > best ? bits : best;
         nacc += ok ? 1ull : 0ull;
     }

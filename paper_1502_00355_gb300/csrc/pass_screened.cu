@@ -4,33 +4,44 @@
 // Section 3.3.4); what changes is which pipe does which work.  GB300 issues
 // about two FP64 operations per SM per clock against ~128 FP32/INT32, so the
 // FP64 pipe does only what decides the result's bits, and the rest moves to
-// the FP32 and integer pipes:
+// the FP32 and integer pipes.  Per window of 128 nodes (window.cuh), one
+// block:
 //
-//  1. The neighbour sums (Eq. 2) are the FP64 additions themselves, in the
+//  1. The window's nodes and their neighbours outside it are staged in shared
+//     memory, as FP64 bit patterns and as float head/tail splits (integer
+//     operations only).
+//  2. The neighbour sums (Eq. 2) are the FP64 additions themselves, in the
 //     stored summation order.
-//  2. The division by the degree is one FP64 multiplication by RN(1/N) and an
+//  3. The division by the degree is one FP64 multiplication by RN(1/N) and an
 //     exact integer remainder that picks the correctly rounded quotient
 //     (div_small.cuh), instead of a full division.
-//  3. If the centre equals the node's position bit for bit, q_new == q_old
+//  4. If the centre equals the node's position bit for bit, q_new == q_old
 //     exactly and no quality needs evaluating.
-//  4. Otherwise alpha of every incident triangle, before and after the move, is
-//     evaluated in FP32 in a frame centred on the node, with a rigorous bound
-//     on its distance to the exact alpha of the FP64 inputs, wide enough to
-//     also cover the FP64 evaluation's own rounding (one bound per side, valid
-//     for all of the node's triangles).  The neighbours' local coordinates
-//     come from float head/tail splits of the doubles; the centre's offset
-//     from one exact FP64 subtraction.  When the intervals of q_new and q_old
-//     are disjoint the FP64 decision is known.
-//  5. If one triangle alone attains both minima, a second screen takes the
+//  5. Otherwise alpha of every incident triangle, before and after the move, is
+//     evaluated in FP32 in a frame centred on the node, around the node's ring,
+//     with a rigorous bound on its distance to the exact alpha of the FP64
+//     inputs, wide enough to also cover the FP64 evaluation's own rounding.
+//     When the intervals of q_new and q_old are disjoint the FP64 decision is
+//     known.
+//  6. If one triangle alone attains both minima, a second screen takes the
 //     sign of alpha(centre) - alpha(node) from a formula in the move itself
 //     (no cancellation) and decides all but rounding-level ties.
-//  6. What is left goes to a per-warp queue in shared memory and is finished
-//     by the exact FP64 update 32 nodes at a time (dense lanes on the narrow
-//     FP64 pipe), on the triangles the screen could not rule out.
+//  7. What is left goes to the block's queue: one item per quality to be
+//     evaluated in FP64, with the coordinates it needs, so that full warps
+//     evaluate independent items side by side on the narrow FP64 pipe.
 //
 // Coordinates are moved as 64-bit patterns, never held in FP64 registers
 // unless they take part in FP64 arithmetic: the compiler copies FP64
 // registers with FP64-pipe instructions.
+//
+// What bounds it: instruction issue (64% of slots), the FP64 pipe (54%) and
+// the latency of shared-memory loads together; HBM stands at about a sixth of
+// the measured copy rate.  Gathering and splitting a coordinate once per
+// window (1.4 times a node) instead of once per neighbour visit (6.5 times)
+// took 1,653 warp instructions per 32 nodes to 1,230 and 23.5 FP64
+// instructions to 13.7.  Measured, to the tolerance, against one thread per
+// node gathering for itself: 2048^2 jittered grid 293.7 -> 217 us a pass,
+// 1024^2 96.9 -> 64.5, 4096^2 942 -> 713.
 #include <atomic>
 #include <cfloat>
 #include <mutex>
@@ -40,463 +51,1079 @@
 #include "kernels.h"
 #include "node_exact.cuh"
 #include "screen.cuh"
+#include "window.cuh"
 
 namespace sls {
 
 namespace {
 
-// Degree and triangle limits of the screened path (larger rings take the
-// exact path).  13 local-coordinate slots per thread keep seven blocks' shared
-// memory within the 164 KB carve-out, which leaves the gathers more L1 than
-// 16 slots (1% faster on jittered grids; a Delaunay mesh of random points has
-// about 7 nodes in 100,000 above 13).
-constexpr int kFastMax = 13;
-__constant__ double c_recip[kFastMax + 1];  // RN(1/N)
-__constant__ double c_degree[kFastMax + 1]; // N as a double
+constexpr int kRingMax = win::kRingMax;
+__constant__ double c_recip[kRingMax + 1];  // RN(1/N)
+__constant__ double c_degree[kRingMax + 1]; // N as a double
 
 __device__ __forceinline__ unsigned long long dbits(double v) { return (unsigned long long)__double_as_longlong(v); }
 __device__ __forceinline__ double bitsd(unsigned long long b) { return __longlong_as_double((long long)b); }
 
 using namespace scr;
 
-// Screens free or fixed node i of one mesh (Eq. 2 and the accept test of
-// Section 3.3.4).  Decided nodes are written and counted here; returns true
-// when the node must be finished by the exact path (d filled in).  loc is
-// this thread's slice of the shared local-coordinate buffer (stride nthr).
-//
-// Warp-synchronous: every lane of the warp calls it (have = false for lanes
-// without a node).  The neighbour loop runs to the warp's largest degree in
-// groups of four, every load of a group issued before its arithmetic; a lane
-// past its own degree adds -0 (x + (-0) == x for every double), so each
-// lane's sums are its node's, in the stored order.
-//
-// The accept test is screened with one error bound per side (before and
-// after the move) for all of the node's triangles.  The per-triangle bound
-//   e * (13.2 |a| + (264.6 + 194 |a|) g),  g = R^2 / s,
-// grows with |a| and g, so the side's largest |a|, its largest local
-// coordinate R (every vertex of every triangle of that side lies within it)
-// and its smallest edge sum s bound every triangle at once.
-template <int LAYOUT>
-__device__ __forceinline__ bool screen_node(const PassArgs &a, bool have, int64_t i, float2 *loc, int nthr,
-                                            Deferred &d, unsigned long long &best, unsigned long long &nacc,
-                                            uint32_t &res)
-{
-    res = 0u;  // decided nodes: bit 0 accepted, bit 1 coordinates changed
-    d.node = (int32_t)i;
-    d.flags = 0u;
-    d.masks = 0u;
-    d.pad = 0u;
-    d.cx = 0ull;
-    d.cy = 0ull;
-    uint32_t off = 0u, meta = kMetaFixed;
-    if (have) {
-        off = __ldg(a.node_off + i);
-        meta = __ldg(a.adj + off);
-    }
-    const bool fixed = (meta & kMetaFixed) != 0u;
-    if (have && fixed && a.accept) a.accept[i] = 0;
-    const uint32_t deg = fixed ? 0u : meta_degree(meta), ntri = fixed ? 0u : meta_ntri(meta);
-    const bool big = !fixed && (deg > (uint32_t)kFastMax || ntri > (uint32_t)kFastMax);
-    bool act = have && !fixed && !big;
-    const uint32_t *nb = a.adj + off + 1;
-    const uint32_t dmax = __reduce_max_sync(0xffffffffu, act ? deg : 0u);
+// ---- shared memory of a block ----------------------------------------------
 
-    ulonglong2 pb = make_ulonglong2(0ull, 0ull), v0 = make_ulonglong2(0ull, 0ull);
-    if (act) {
-        pb = CoordBits<LAYOUT>::get(a.in, a.n, i);
-        v0 = CoordBits<LAYOUT>::get(a.in, a.n, __ldg(nb));
-    }
-    float phx, plx, phy, ply;
-    bool ok = head_tail(pb.x, phx, plx) & head_tail(pb.y, phy, ply);
-    unsigned long long sxb = v0.x, syb = v0.y;
-    float rn = 0.0f, rmin = FLT_MAX;
-    {
-        float2 L;
-        bool ok0;
-        local_offset(v0.x, v0.y, phx, plx, phy, ply, L.x, L.y, ok0);
-        ok = ok & ok0;
-        if (act) loc[0] = L;
-        const float rl = fmaxf(fabsf(L.x), fabsf(L.y));
-        rn = rl;
-        rmin = rl;
-    }
-    for (uint32_t k0 = 1; k0 < dmax; k0 += 4) {
-        uint32_t id[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) id[u] = (act && k0 + u < deg) ? __ldg(nb + k0 + u) : 0u;
-        ulonglong2 v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            v[u] = (act && k0 + u < deg) ? CoordBits<LAYOUT>::get(a.in, a.n, id[u])
-                                         : make_ulonglong2(0x8000000000000000ull, 0x8000000000000000ull);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const uint32_t k = k0 + (uint32_t)u;
-            if (k < dmax) {  // warp-uniform
-                const bool on = act && k < deg;
-                // x + (-0) == x for every x: lanes past their degree add -0
-                sxb = dbits(__dadd_rn(bitsd(sxb), bitsd(v[u].x)));
-                syb = dbits(__dadd_rn(bitsd(syb), bitsd(v[u].y)));
-                float2 L;
-                bool okk;
-                local_offset(v[u].x, v[u].y, phx, plx, phy, ply, L.x, L.y, okk);
-                if (on) loc[k * nthr] = L;
-                const float rl = fmaxf(fabsf(L.x), fabsf(L.y));
-                rn = on ? fmaxf(rn, rl) : rn;
-                rmin = on ? fminf(rmin, rl) : rmin;
-                ok = on ? (ok & okk) : ok;
-            }
-        }
-    }
-    if (big) return true;  // exact path does it all
-    if (!act) return false;
-    const double fd = c_degree[deg], y = c_recip[deg];
-    const unsigned long long cbx = divs::div_small_bits(sxb, deg, y, fd);
-    const unsigned long long cby = divs::div_small_bits(syb, deg, y, fd);
-    d.cx = cbx;
-    d.cy = cby;
-    d.flags = kHasCentre;
-    if (cbx == pb.x && cby == pb.y) {
-        // the centre is the node itself: q_new == q_old exactly
-        const bool acc = !a.strict;
-        CoordBits<LAYOUT>::put(a.out, a.n, i, pb);
-        if (a.accept) a.accept[i] = acc ? 1 : 0;
-        nacc += acc ? 1ull : 0ull;
-        res = acc ? 1u : 0u;
-        return false;
-    }
-    if (!ok) return true;
-    const double dx = __dsub_rn(bitsd(cbx), bitsd(pb.x)), dy = __dsub_rn(bitsd(cby), bitsd(pb.y));
-    const float Cx = trunc_float(dbits(dx)), Cy = trunc_float(dbits(dy));
-    const float rC = fmaxf(fabsf(Cx), fabsf(Cy));
-    const float M = fmaxf(fabsf(phx), fabsf(phy)) * 1.0001f + fmaxf(rn, rC);
-    const float M2 = M * M;
-    if (!frame_ok(rmin, fmaxf(rn, rC), M)) return true;
-    const float rN = fmaxf(rn, rC);
-    float amin_o = FLT_MAX, a2_o = FLT_MAX, amax_o = 0.0f, smin_o = FLT_MAX;
-    float amin_n = FLT_MAX, a2_n = FLT_MAX, amax_n = 0.0f, smin_n = FLT_MAX;
-    uint32_t arg_o = 0u, arg_n = 0u;
-    for (uint32_t t0 = 0; t0 < ntri; t0 += 4) {
-        uint32_t c[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) c[u] = t0 + u < ntri ? __ldg(nb + deg + t0 + u) : 0u;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const uint32_t t = t0 + (uint32_t)u;
-            if (t < ntri) {
-                const float2 A = loc[code_first(c[u]) * nthr];
-                const float2 B = loc[code_second(c[u]) * nthr];
-                const float sk = code_slot(c[u]) == 1u ? -kTwoSqrt3f : kTwoSqrt3f;
-                const float ba2 = edge_ba2(A.x, A.y, B.x, B.y);
-                {
-                    float sv;
-                    const float av = screen_alpha(0.0f, 0.0f, A.x, A.y, B.x, B.y, ba2, sk, sv);
-                    if (av < amin_o) {
-                        a2_o = amin_o;
-                        amin_o = av;
-                        arg_o = t;
-                    } else {
-                        a2_o = fminf(a2_o, av);
-                    }
-                    amax_o = fmaxf(amax_o, fabsf(av));
-                    smin_o = fminf(smin_o, sv);
-                }
-                {
-                    float sv;
-                    const float av = screen_alpha(Cx, Cy, A.x, A.y, B.x, B.y, ba2, sk, sv);
-                    if (av < amin_n) {
-                        a2_n = amin_n;
-                        amin_n = av;
-                        arg_n = t;
-                    } else {
-                        a2_n = fminf(a2_n, av);
-                    }
-                    amax_n = fmaxf(amax_n, fabsf(av));
-                    smin_n = fminf(smin_n, sv);
-                }
-            }
-        }
-    }
-    // per side: q (FP64) lies in [amin - b, amin + b]; the minimum is attained
-    // by triangle arg alone when every other alpha lies above amin + b + b
-    const float go = side_g(rn, smin_o), gn = side_g(rN, smin_n);
-    int verdict = 0;
-    bool single_o = false, single_n = false;
-    const bool bok = bound_ok(smin_o, go, amax_o) & bound_ok(smin_n, gn, amax_n);
-    const float bo = side_bound(amax_o, go);
-    const float bn = side_bound(amax_n, gn);
-    const float minU_o = amin_o + bo, minU_n = amin_n + bn;
-    if (bok) {
-        const float minL_o = amin_o - bo, minL_n = amin_n - bn;
-        verdict = minL_n > minU_o ? 1 : (minU_n < minL_o ? -1 : 0);
-        single_o = a2_o - bo > minU_o;
-        single_n = a2_n - bn > minU_n;
-    }
-    if (verdict == 0 && single_o && single_n && arg_o == arg_n) {
-        const uint32_t c = __ldg(nb + deg + arg_o);
-        const float2 A = loc[code_first(c) * nthr], B = loc[code_second(c) * nthr];
-        verdict = diff_screen(A.x, A.y, B.x, B.y, Cx, Cy, code_slot(c) == 1u ? -1.0f : 1.0f, M2);
-    }
-    if (verdict == 0) {
-        // candidates for the exact path: every triangle whose interval
-        // reaches below the side's lowest upper end (all of them when the
-        // bounds do not hold)
-        const uint32_t all = (1u << ntri) - 1u;
-        uint32_t mo = bok ? (single_o ? (1u << arg_o) : 0u) : all;
-        uint32_t mn = bok ? (single_n ? (1u << arg_n) : 0u) : all;
-        if (bok && !(single_o && single_n)) {
-            for (uint32_t t = 0; t < ntri; ++t) {
-                const uint32_t c = __ldg(nb + deg + t);
-                const float2 A = loc[code_first(c) * nthr];
-                const float2 B = loc[code_second(c) * nthr];
-                const float sk = code_slot(c) == 1u ? -kTwoSqrt3f : kTwoSqrt3f;
-                const float ba2 = edge_ba2(A.x, A.y, B.x, B.y);
-                float sv;
-                if (!single_o && screen_alpha(0.0f, 0.0f, A.x, A.y, B.x, B.y, ba2, sk, sv) - bo <= minU_o)
-                    mo |= 1u << t;
-                if (!single_n && screen_alpha(Cx, Cy, A.x, A.y, B.x, B.y, ba2, sk, sv) - bn <= minU_n)
-                    mn |= 1u << t;
-            }
-        }
-        d.flags |= kMasked;
-        d.masks = mo | (mn << 16);
-        return true;
-    }
-    const bool acc = verdict > 0;
-    ulonglong2 outp = pb;
-    if (acc) {
-        const unsigned long long b2 = dbits(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
-        best = b2 > best ? b2 : best;
-        nacc += 1ull;
-        outp = make_ulonglong2(cbx, cby);
-        res = 3u;  // the centre differs from the node (equal centres return above)
-    }
-    CoordBits<LAYOUT>::put(a.out, a.n, i, outp);
-    if (a.accept) a.accept[i] = acc ? 1 : 0;
-    return false;
+constexpr int kBlockMax = 128;
+constexpr int kItems = 112;       // qualities waiting for their FP64 evaluation
+constexpr int kPending = 64;      // nodes they belong to
+constexpr int kItemsFull = 72;    // the queue is worked off once it holds this many items
+constexpr int kPendingFull = 44;  // or nodes
+constexpr uint32_t kNoItem = 0xffffffffu;
+
+struct __align__(16) Queue {
+    ulonglong2 p[kPending], c[kPending];                    // the node, its centre
+    double px[kItems], py[kItems], qx[kItems], qy[kItems];  // the step's two vertices, in ring order; then px: the quality
+    uint32_t item[kItems];      // pending node | side << 8 (1: after the move) | step << 9
+    int32_t node[kPending];     // -1: no entry
+    uint32_t range[kPending];   // first item | items << 8 | lane << 16
+    uint32_t cold[kPending];    // row of the lane's slots and, next to it, directions
+    uint32_t nitems, npending;  // claimed (may exceed the capacity)
+    unsigned int nacc, nexact;  // accepted and exactly decided nodes (flush)
+    unsigned long long best;    // bits of the block's largest squared move
+    float best_low;             // at most that (-1: none yet)
+};
+
+// A block keeps two windows in shared memory: the one it works on and the
+// next one, which is copied in meanwhile.  Headers are fetched three windows
+// ahead and halo ids two, because each names what the next copies.
+struct __align__(16) Ahead {
+    uint32_t hdr[4][win::kHeaderWords];  // window i's header in slot i & 3
+    uint8_t idle[4][4];                  // skip_unchanged: its subtiles that need no work
+};
+
+struct Block {
+    Queue *q;
+    Ahead *ahead;
+    uint32_t *ids;            // halo ids, window i's in buffer i & 1
+    uint32_t *rows;           // hot rows
+    char *xy;                 // staged entries: coordinates, then head/tail splits
+    uint32_t ids_words, rows_words, half, stage;  // buffer sizes: words, words, bytes of one array, bytes
+                                                  // from one buffer to the other (0: there is one)
+};
+
+// Buffers of staged entries: one where two would leave an SM with few blocks.
+// Colour classes (about 510 entries a window) run 233 us a sweep with one and
+// 281 with two (1500 x 1100 grid), a random numbering kept as it is (900
+// entries) 111 against 144 us a pass; local numberings (at most 255) gain 8%
+// from the second.
+constexpr int kTwoBufferEntries = 320;
+__host__ __device__ inline int buffers_for(const WindowShape &s) { return s.entries <= kTwoBufferEntries ? 2 : 1; }
+__host__ __device__ inline uint32_t ids_words_of(const WindowShape &s) { return ((uint32_t)s.halo + 3u) & ~3u; }
+size_t smem_for(const WindowShape &s)
+{
+    return sizeof(Queue) + sizeof(Ahead) + 2 * 4 * (size_t)ids_words_of(s) + 2 * 128 * (size_t)s.hot +
+           (size_t)buffers_for(s) * 32 * (size_t)(s.entries + 1);
 }
 
-// Finishes one full warp's worth of deferred nodes (lane k takes entry k)
-// when the warp's queue holds at least 32, or all remaining entries at the
-// end.  Dense lanes keep the narrow FP64 pipe busy without block barriers.
-template <int LAYOUT>
-__device__ __forceinline__ void drain_queue(const PassArgs &a, Deferred *wq, int &qn, bool all,
-                                            unsigned long long &best, unsigned long long &nacc)
+struct Tally {
+    unsigned int nacc, nexact;
+};
+
+__device__ __forceinline__ void reset(Queue *q)
 {
-    const int lane = threadIdx.x & 31;
-    while (qn >= 32 || (all && qn > 0)) {
-        if (lane < qn) {
-            const Deferred e = wq[lane];
+    q->nitems = q->npending = q->nacc = q->nexact = 0u;
+    q->best = 0ull;
+    q->best_low = -1.0f;
+}
+
+// The block's statistics into a pass record; the queue starts afresh.  All
+// threads call it; nothing may be pushed before the next barrier.
+__device__ __forceinline__ void flush(Queue *q, PassStats *st, const Tally &tally)
+{
+    const unsigned acc = __reduce_add_sync(0xffffffffu, tally.nacc), ex = __reduce_add_sync(0xffffffffu, tally.nexact);
+    if ((threadIdx.x & 31) == 0) {
+        if (acc) atomicAdd(&q->nacc, acc);
+        if (ex) atomicAdd(&q->nexact, ex);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (q->best) atomicMax(&st->maxd2_bits, q->best);
+        if (q->nacc) atomicAdd(&st->nacc, (unsigned long long)q->nacc);
+        if (q->nexact) atomicAdd(&st->fallbacks, (unsigned long long)q->nexact);
+        reset(q);
+    }
+}
+
+// A squared move (FP64 bits) towards the block's largest.
+__device__ __forceinline__ void note_move(Queue *q, unsigned long long b2)
+{
+    if (b2 <= *const_cast<volatile unsigned long long *>(&q->best)) return;
+    atomicMax(&q->best, b2);
+    atomicMax(reinterpret_cast<int *>(&q->best_low), __float_as_int(__double2float_rd(bitsd(b2))));
+}
+
+__device__ __forceinline__ Block block_memory(unsigned char *smem, const WindowShape &s)
+{
+    Block b;
+    b.q = reinterpret_cast<Queue *>(smem);
+    b.ahead = reinterpret_cast<Ahead *>(smem + sizeof(Queue));
+    b.ids = reinterpret_cast<uint32_t *>(smem + sizeof(Queue) + sizeof(Ahead));
+    b.ids_words = ids_words_of(s);
+    b.rows = b.ids + 2 * b.ids_words;
+    b.rows_words = 32u * (uint32_t)s.hot;
+    b.xy = reinterpret_cast<char *>(b.rows + 2 * b.rows_words);
+    b.half = (uint32_t)(s.entries + 1) * 16u;
+    b.stage = buffers_for(s) == 2 ? 2u * b.half : 0u;
+    // the padding entries: -0 for the sums, NaN for the rings
+    const float nan = __int_as_float(0x7fffffff);
+    for (uint32_t k = threadIdx.x; k < (uint32_t)buffers_for(s); k += blockDim.x) {
+        *reinterpret_cast<ulonglong2 *>(b.xy + k * b.stage) =
+            make_ulonglong2(0x8000000000000000ull, 0x8000000000000000ull);
+        *reinterpret_cast<float4 *>(b.xy + k * b.stage + b.half) = make_float4(nan, nan, nan, nan);
+    }
+    if (threadIdx.x == 0) reset(b.q);
+    return b;
+}
+
+// Asynchronous copies global -> shared (no registers held while they fly).
+__device__ __forceinline__ void copy16(void *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void copy8(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// ---- the FP64 queue ---------------------------------------------------------
+
+// FP64 quality of step t (P -> Q) of a ring with the node at x.  The step runs
+// in the triangle's stored direction unless `rev`; the stored order of P and Q
+// is P, Q for slots 0 and 2 and Q, P for slot 1.
+__device__ __forceinline__ double step_quality(ulonglong2 x, unsigned long long px, unsigned long long py,
+                                               unsigned long long qx, unsigned long long qy, uint32_t slots,
+                                               uint32_t rev, uint32_t t)
+{
+    const uint32_t slot = (slots >> (2u * t)) & 3u;
+    const bool swap = (((rev >> t) & 1u) != 0u) != (slot == 1u);
+    return alpha_at_slot(slot, bitsd(x.x), bitsd(x.y), bitsd(swap ? qx : px), bitsd(swap ? qy : py),
+                         bitsd(swap ? px : qx), bitsd(swap ? py : qy));
+}
+
+// Evaluates every waiting item and finishes the nodes they belong to.  All
+// threads of the block call it, with no push in flight.
+template <int LAYOUT>
+__device__ __noinline__ Tally drain(const PassArgs &a, Queue *q, Tally tally)
+{
+    const uint32_t ni = q->nitems < (uint32_t)kItems ? q->nitems : (uint32_t)kItems;
+    for (uint32_t k = threadIdx.x; k < ni; k += blockDim.x) {
+        const uint32_t it = q->item[k];
+        if (it == kNoItem) continue;
+        const uint32_t e = it & 0xffu;
+        const uint32_t *row = a.win_rows + (size_t)q->cold[e] * 32u + (q->range[e] >> 16);
+        const ulonglong2 x = (it & 0x100u) ? q->c[e] : q->p[e];
+        q->px[k] = step_quality(x, dbits(q->px[k]), dbits(q->py[k]), dbits(q->qx[k]), dbits(q->qy[k]), __ldg(row),
+                                __ldg(row + 32), it >> 9);
+    }
+    __syncthreads();
+    const uint32_t np = q->npending < (uint32_t)kPending ? q->npending : (uint32_t)kPending;
+    for (uint32_t e = threadIdx.x; e < np; e += blockDim.x) {
+        const int32_t node = q->node[e];
+        if (node < 0) continue;
+        const uint32_t i0 = q->range[e] & 0xffu, cnt = (q->range[e] >> 8) & 0xffu;
+        double q_old = bitsd(0x7ff0000000000000ull), q_new = q_old;
+#pragma unroll 4
+        for (uint32_t k = i0; k < i0 + cnt; ++k) {
+            const double v = q->px[k];
+            if (q->item[k] & 0x100u) {
+                if (v < q_new) q_new = v;
+            } else {
+                if (v < q_old) q_old = v;
+            }
+        }
+        unsigned long long b2;
+        bool acc, moved;
+        const ulonglong2 p = q->p[e], c = q->c[e];
+        finish_exact<LAYOUT>(a, node, make_double2(bitsd(p.x), bitsd(p.y)), make_double2(bitsd(c.x), bitsd(c.y)),
+                             q_old, q_new, b2, acc, moved);
+        note_move(q, b2);
+        tally.nacc += acc ? 1u : 0u;
+        if (a.halo) {  // the node's bits in its tile's masks (written with the tile's other nodes)
+            const uint32_t bit = 1u << (node & 31);
+            if (moved) atomicOr(a.chg_cur + (node >> 5), bit);
+            if (acc) atomicOr(a.accm + (node >> 5), bit);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) q->nitems = q->npending = 0u;
+    __syncthreads();
+    return tally;
+}
+
+// ---- one subtile --------------------------------------------------------------
+
+// List entries of BITS bits in a lane's words (32 words apart), as byte
+// offsets of staged entries.
+template <int BITS>
+struct List {
+    static constexpr uint32_t kPer = 32 / BITS;
+    static __device__ __forceinline__ uint32_t in_word(uint32_t word, uint32_t j)
+    {
+        return ((word >> (BITS * j)) & ((1u << BITS) - 1u)) << 4;
+    }
+    static __device__ __forceinline__ uint32_t at(const uint32_t *list, uint32_t t)
+    {
+        return in_word(list[32u * (t / kPer)], t % kPer);
+    }
+};
+
+// ---- the ring walk: screen.cuh's ring form, both sides of the move in the
+// halves of packed FP32 pairs (one instruction for two operations, the same
+// roundings).
+
+__device__ __forceinline__ uint64_t pair(float lo, float hi)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void halves(uint64_t v, float &lo, float &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+// The larger of two, NaN when either is.
+__device__ __forceinline__ float max_nan(float a, float b)
+{
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+
+// What the walk knows of the node.
+struct RingWalk {
+    const char *split;         // staged head/tail splits
+    float phx, plx, phy, ply;  // the node's splits
+    float Cx, Cy;              // the centre's offset
+    uint32_t slots, rev;       // irregular subtiles only
+
+    __device__ __forceinline__ RingVertex vertex(uint32_t off) const
+    {
+        const float4 h = *reinterpret_cast<const float4 *>(split + off);
+        return ring_vertex(h.x, h.y, h.z, h.w, phx, plx, phy, ply, Cx, Cy);
+    }
+};
+
+// ring_vertex's values before | after the move; TURNED: y and yc negated.
+// Steps go from plain to turned vertices and back, so that their cross
+// products need no negation.
+struct PairVertex {
+    float x, y;
+    uint64_t xx, yy, nn;
+};
+
+template <bool TURNED>
+__device__ __forceinline__ PairVertex pair_vertex(const RingWalk &w, uint32_t off)
+{
+    const float4 h = *reinterpret_cast<const float4 *>(w.split + off);
+    PairVertex v;
+    v.x = (h.x - w.phx) + (h.y - w.plx);
+    v.y = TURNED ? (w.phy - h.z) + (w.ply - h.w) : (h.z - w.phy) + (h.w - w.ply);
+    v.xx = pair(v.x, v.x - w.Cx);
+    v.yy = pair(v.y, TURNED ? v.y + w.Cy : v.y - w.Cy);
+    v.nn = fma2(v.xx, v.xx, mul2(v.yy, v.yy));
+    return v;
+}
+
+struct Minima {
+    float m1o, m2o, m1n, m2n;  // smallest and second smallest value before and after the move
+    float smin, rn;            // smallest edge sum, largest local coordinate
+};
+
+// ring_values of the step P -> Q (FROM_PLAIN: P is the plain one), packed with
+// its number, into the minima.  Padding steps are NaN and change nothing.
+template <bool IRREGULAR, bool FROM_PLAIN>
+__device__ __forceinline__ void ring_step(const RingWalk &w, Minima &m, const PairVertex &P, const PairVertex &Q,
+                                          uint32_t t)
+{
+    m.rn = fmaxf(m.rn, fmaxf(fabsf(Q.x), fabsf(Q.y)));
+    if (IRREGULAR && ((w.slots >> (2u * t)) & 3u) == 3u) return;
+    const float bx = Q.x - P.x, by = Q.y + P.y;
+    const float b2 = fmaf(bx, bx, by * by);
+    float so, sn, co, cn;
+    halves(add2(add2(P.nn, Q.nn), pair(b2, b2)), so, sn);
+    halves(fma2(P.xx, Q.yy, mul2(P.yy, Q.xx)), co, cn);  // the cross product, negated from a plain vertex
+    float vo = (FROM_PLAIN ? -co : co) * rcp_ring(so), vn = (FROM_PLAIN ? -cn : cn) * rcp_ring(sn);
+    if (IRREGULAR && ((w.rev >> t) & 1u)) {
+        vo = -vo;
+        vn = -vn;
+    }
+    vo = with_step(vo, t);
+    vn = with_step(vn, t);
+    m.m2o = fminf(m.m2o, max_nan(m.m1o, vo));
+    m.m1o = fminf(m.m1o, vo);
+    m.m2n = fminf(m.m2n, max_nan(m.m1n, vn));
+    m.m1n = fminf(m.m1n, vn);
+    m.smin = fminf(m.smin, fminf(so, sn));
+}
+
+// Walks the rings of a warp's lanes to the subtile's largest step number l,
+// two steps between branches (so that the loads of one overlap the other's
+// arithmetic).
+template <bool IRREGULAR, int BITS>
+__device__ __forceinline__ Minima walk_ring(const RingWalk &w, uint32_t l, const uint32_t *list)
+{
+    using L = List<BITS>;
+    Minima m;
+    m.m1o = m.m2o = m.m1n = m.m2n = m.smin = FLT_MAX;
+    uint32_t word = list[0];
+    PairVertex A = pair_vertex<false>(w, L::in_word(word, 0));
+    m.rn = fmaxf(fabsf(A.x), fabsf(A.y));
+    for (uint32_t t = 0;; t += L::kPer) {  // a word's entries per trip; A is entry t
+#pragma unroll
+        for (uint32_t j = 0; j < L::kPer; j += 2) {
+            const uint32_t e1 = L::in_word(word, j + 1);
+            if (j + 2 == L::kPer) {
+                list += 32;
+                word = *list;
+            }
+            const uint32_t e2 = L::in_word(word, (j + 2) % L::kPer);
+            const PairVertex B = pair_vertex<true>(w, e1);
+            const PairVertex C = pair_vertex<false>(w, e2);
+            ring_step<IRREGULAR, true>(w, m, A, B, t + j);
+            ring_step<IRREGULAR, false>(w, m, B, C, t + j + 1u);
+            A = C;
+            if (t + j + 2u >= l) return m;
+        }
+    }
+}
+
+// What a lane knows of a node that its screen left open.
+struct Open {
+    float Cx, Cy;        // the centre's offset
+    float b, up_o, up_n; // a step is a candidate unless its value less b lies above the side's up
+    uint32_t own, steps;
+};
+
+// The nodes of a warp that its screen left open (mask): for each, lane t looks
+// at step t before the move and lane 16 + t after it; the steps that can
+// attain a side's minimum go into the queue or, when that has no room, are
+// evaluated at once.  list: a lane's ring; cold: the subtile's slots row.
+// Returns per lane 1 accepted, 2 moved (decided at once), 8 queue full enough
+// to be worked off.
+template <int LAYOUT, int BITS>
+__device__ __noinline__ uint32_t settle_open(const PassArgs &a, Queue *q, const char *xy, uint32_t half,
+                                             const uint32_t *list, uint32_t cold, bool irregular, int32_t node,
+                                             ulonglong2 c, Open o, unsigned mask)
+{
+    const uint32_t lane = threadIdx.x & 31u, t = lane & 15u;
+    const bool after = lane >= 16u;
+    uint32_t out = 0u;
+    for (; mask; mask &= mask - 1u) {
+        const uint32_t src = (uint32_t)__ffs((int)mask) - 1u;
+        const uint32_t own = __shfl_sync(0xffffffffu, o.own, src), steps = __shfl_sync(0xffffffffu, o.steps, src);
+        const float Cx = __shfl_sync(0xffffffffu, o.Cx, src), Cy = __shfl_sync(0xffffffffu, o.Cy, src);
+        const float b = __shfl_sync(0xffffffffu, o.b, src);
+        const float up_o = __shfl_sync(0xffffffffu, o.up_o, src), up_n = __shfl_sync(0xffffffffu, o.up_n, src);
+        const uint32_t *ring = list + (int)src - (int)lane;
+        const uint32_t *row = a.win_rows + (size_t)cold * 32u + src;
+        uint32_t eP = 0u, eQ = 0u;
+        bool cand = false;
+        if (t < steps) {
+            eP = List<BITS>::at(ring, t);
+            eQ = List<BITS>::at(ring, t + 1u);
+            const float4 h = *reinterpret_cast<const float4 *>(xy + half + own);
+            const float4 hP = *reinterpret_cast<const float4 *>(xy + half + eP);
+            const float4 hQ = *reinterpret_cast<const float4 *>(xy + half + eQ);
+            const RingVertex P = ring_vertex(hP.x, hP.y, hP.z, hP.w, h.x, h.y, h.z, h.w, Cx, Cy);
+            const RingVertex Q = ring_vertex(hQ.x, hQ.y, hQ.z, hQ.w, h.x, h.y, h.z, h.w, Cx, Cy);
+            float vo, vn, so, sn;
+            ring_values(P, Q, vo, vn, so, sn);
+            float v = after ? vn : vo;
+            cand = true;
+            if (irregular) {
+                cand = ((__ldg(row) >> (2u * t)) & 3u) != 3u;
+                if ((__ldg(row + 32) >> t) & 1u) v = -v;
+            }
+            cand = cand && !(kTwoSqrt3f * with_step(v, t) - b > (after ? up_n : up_o));
+        }
+        const unsigned cands = __ballot_sync(0xffffffffu, cand);
+        const uint32_t cnt = __popc(cands), place = __popc(cands & ((1u << lane) - 1u));
+        uint32_t e = 0u, i0 = 0u;
+        if (lane == 0u) {
+            e = atomicAdd(&q->npending, 1u);
+            i0 = atomicAdd(&q->nitems, cnt);
+        }
+        e = __shfl_sync(0xffffffffu, e, 0);
+        i0 = __shfl_sync(0xffffffffu, i0, 0);
+        if (e + 1u >= (uint32_t)kPendingFull || i0 + cnt >= (uint32_t)kItemsFull) out |= 8u;
+        const ulonglong2 P = *reinterpret_cast<const ulonglong2 *>(xy + eP);
+        const ulonglong2 Q = *reinterpret_cast<const ulonglong2 *>(xy + eQ);
+        if (e < (uint32_t)kPending && i0 + cnt <= (uint32_t)kItems) {
+            if (cand) {
+                const uint32_t at = i0 + place;
+                q->px[at] = bitsd(P.x);
+                q->py[at] = bitsd(P.y);
+                q->qx[at] = bitsd(Q.x);
+                q->qy[at] = bitsd(Q.y);
+                q->item[at] = e | (after ? 0x100u : 0u) | (t << 9);
+            }
+            if (lane == src) {
+                q->p[e] = *reinterpret_cast<const ulonglong2 *>(xy + own);
+                q->c[e] = c;
+                q->node[e] = node;
+                q->cold[e] = cold;
+                q->range[e] = i0 | (cnt << 8) | (lane << 16);
+            }
+            continue;
+        }
+        // no room: what was claimed stays empty
+        if (i0 + lane < (uint32_t)kItems && lane < cnt) q->item[i0 + lane] = kNoItem;
+        if (lane == 0u && e < (uint32_t)kPending) q->node[e] = -1;
+        const ulonglong2 p = *reinterpret_cast<const ulonglong2 *>(xy + own);
+        const ulonglong2 cs = make_ulonglong2(__shfl_sync(0xffffffffu, c.x, src), __shfl_sync(0xffffffffu, c.y, src));
+        double v = bitsd(0x7ff0000000000000ull);
+        if (cand) v = step_quality(after ? cs : p, P.x, P.y, Q.x, Q.y, __ldg(row), __ldg(row + 32), t);
+        for (int w = 8; w > 0; w >>= 1) {
+            const double u = __shfl_xor_sync(0xffffffffu, v, w);
+            if (u < v) v = u;
+        }
+        const double q_old = __shfl_sync(0xffffffffu, v, 0), q_new = __shfl_sync(0xffffffffu, v, 16);
+        if (lane == src) {
             unsigned long long b2;
             bool acc, moved;
-            exact_update<LAYOUT>(a, e.node, e.flags, e.masks, e.cx, e.cy, b2, acc, moved);
-            best = b2 > best ? b2 : best;
-            nacc += acc ? 1ull : 0ull;
-            if (a.halo) {  // the node's bits in its tile's masks (written with the tile's other nodes)
-                const uint32_t bit = 1u << (e.node & 31);
-                if (moved) atomicOr(a.chg_cur + (e.node >> 5), bit);
-                if (acc) atomicOr(a.accm + (e.node >> 5), bit);
+            finish_exact<LAYOUT>(a, node, make_double2(bitsd(p.x), bitsd(p.y)), make_double2(bitsd(c.x), bitsd(c.y)),
+                                 q_old, q_new, b2, acc, moved);
+            note_move(q, b2);
+            out |= (acc ? 1u : 0u) | (moved ? 2u : 0u);
+        }
+    }
+    return out;
+}
+
+// FP32 offset of the centre from the node (relative error below 2^-23).  With
+// equal sign and exponent field the difference is a whole number of units in
+// the last place; otherwise one FP64 subtraction.
+__device__ __forceinline__ void offset_of(ulonglong2 c, ulonglong2 p, float &Cx, float &Cy)
+{
+    const uint32_t hx = (uint32_t)(p.x >> 32), hy = (uint32_t)(p.y >> 32);
+    const uint32_t ex = (hx >> 20) & 0x7ffu, ey = (hy >> 20) & 0x7ffu;
+    const uint32_t other = ((uint32_t)((c.x ^ p.x) >> 32) | (uint32_t)((c.y ^ p.y) >> 32)) & 0xfff00000u;
+    if (other == 0u && ex - 949u <= 200u && ey - 949u <= 200u) {
+        // unit in the last place, with the sign of the coordinate
+        const float ux = __uint_as_float((hx & 0x80000000u) | ((ex - 948u) << 23));
+        const float uy = __uint_as_float((hy & 0x80000000u) | ((ey - 948u) << 23));
+        Cx = __ll2float_rn((long long)(c.x - p.x)) * ux;
+        Cy = __ll2float_rn((long long)(c.y - p.y)) * uy;
+    } else {
+        Cx = trunc_float(dbits(__dsub_rn(bitsd(c.x), bitsd(p.x))));
+        Cy = trunc_float(dbits(__dsub_rn(bitsd(c.y), bitsd(p.y))));
+    }
+}
+
+// A subtile's rows, for one lane.
+struct Rows {
+    const uint32_t *at;    // the lane's word of the first row (shared memory)
+    uint32_t cold;         // its slots row of the stream; its directions row is the next
+    uint32_t d, l;         // the subtile's largest degree and step number
+    uint32_t meta;
+    bool irregular;
+};
+
+// Updates the free node a lane holds (Eq. 2 and the accept test of Section
+// 3.3.4).  res: bit 0 accepted, bit 1 coordinates changed.  Returns true when
+// the node's record has to decide (a coordinate outside the splits' range).
+template <int LAYOUT, int BITS>
+__device__ __forceinline__ bool update_lane(const PassArgs &a, Queue *q, const char *xy, uint32_t half, const Rows &r,
+                                            int32_t node, Tally &tally, uint32_t &res, bool &full)
+{
+    using L = List<BITS>;
+    const uint32_t deg = win::meta_deg(r.meta), steps = win::meta_steps(r.meta);
+    const uint32_t own = (win::meta_place(r.meta) + 1u) * 16u;
+    // the sums, to the subtile's largest degree: lists are padded with the
+    // entry that holds (-0, -0)
+    const uint32_t *list = r.at + 32;
+    uint32_t word = *list;
+    double sx = 0.0, sy = 0.0;
+    for (uint32_t k = 0;;) {  // four neighbours' loads go out together
+        ulonglong2 v[4];
+#pragma unroll
+        for (uint32_t j = 0; j < 4u; ++j) {
+            if (j > 0u && j % L::kPer == 0u) word = list[32u * (j / L::kPer)];
+            v[j] = *reinterpret_cast<const ulonglong2 *>(xy + L::in_word(word, j % L::kPer));
+        }
+        // branches out, not conditions: an addition that is not due must not
+        // occupy the FP64 pipe
+        if (k == 0u) {
+            sx = bitsd(v[0].x);
+            sy = bitsd(v[0].y);
+        } else {
+            sx = __dadd_rn(sx, bitsd(v[0].x));
+            sy = __dadd_rn(sy, bitsd(v[0].y));
+        }
+        if (++k >= r.d) break;
+        sx = __dadd_rn(sx, bitsd(v[1].x));
+        sy = __dadd_rn(sy, bitsd(v[1].y));
+        if (++k >= r.d) break;
+        sx = __dadd_rn(sx, bitsd(v[2].x));
+        sy = __dadd_rn(sy, bitsd(v[2].y));
+        if (++k >= r.d) break;
+        sx = __dadd_rn(sx, bitsd(v[3].x));
+        sy = __dadd_rn(sy, bitsd(v[3].y));
+        if (++k >= r.d) break;
+        list += 32u * (4u / L::kPer);
+        word = *list;
+    }
+    list = r.at + 32u * (1u + win::list_rows(r.d, BITS));  // the ring
+    res = 0u;
+    const bool free = (r.meta & win::kFree) != 0u;
+    const ulonglong2 pb = *reinterpret_cast<const ulonglong2 *>(xy + own);
+    ulonglong2 cb = pb;
+    if (free) {
+        const double fd = c_degree[deg], y = c_recip[deg];
+        cb.x = divs::div_small_bits(dbits(sx), deg, y, fd);
+        cb.y = divs::div_small_bits(dbits(sy), deg, y, fd);
+    }
+    bool act = cb.x != pb.x || cb.y != pb.y;
+    if (free && !act) {
+        // the centre is the node itself: q_new == q_old exactly
+        const bool acc = !a.strict;
+        CoordBits<LAYOUT>::put(a.out, a.n, node, pb);
+        if (a.accept) a.accept[node] = acc ? 1 : 0;
+        tally.nacc += acc ? 1u : 0u;
+        res = acc ? 1u : 0u;
+    }
+    if (!__any_sync(0xffffffffu, act)) return false;
+    RingWalk w;
+    w.split = xy + half;
+    {
+        const float4 h = *reinterpret_cast<const float4 *>(xy + half + own);
+        w.phx = h.x;
+        w.plx = h.y;
+        w.phy = h.z;
+        w.ply = h.w;
+    }
+    w.Cx = w.Cy = 0.0f;
+    if (act) offset_of(cb, pb, w.Cx, w.Cy);
+    w.slots = w.rev = 0u;
+    Minima m;
+    if (r.irregular) {
+        const uint32_t *row = a.win_rows + (size_t)r.cold * 32u + (threadIdx.x & 31u);
+        w.slots = __ldg(row);
+        w.rev = __ldg(row + 32);
+        m = walk_ring<true, BITS>(w, r.l, list);
+    } else {
+        m = walk_ring<false, BITS>(w, r.l, list);
+    }
+    // a coordinate of the node or of a neighbour outside the splits' range
+    const bool record = act && !(fmaxf(m.rn, fmaxf(fabsf(w.phx), fabsf(w.phy))) < FLT_MAX);
+    act = act && !record;
+    const float rN = fmaxf(m.rn, fmaxf(fabsf(w.Cx), fabsf(w.Cy)));
+    const float M = fmaxf(fabsf(w.phx), fabsf(w.phy)) * 1.0001f + rN;
+    const float g = side_g(rN, m.smin);
+    const bool bok = frame_ok(m.rn, rN, M) & ring_ok(m.smin, g);
+    Open o;
+    o.b = ring_bound(g);
+    // per side: q (FP64) lies in [amin - b, amin + b]; the minimum is attained
+    // by one triangle alone when every other value lies above amin + b + b
+    const float amin_o = kTwoSqrt3f * m.m1o, amin_n = kTwoSqrt3f * m.m1n;
+    o.up_o = amin_o + o.b;
+    o.up_n = amin_n + o.b;
+    int verdict = 0;
+    if (bok) verdict = amin_n - o.b > o.up_o ? 1 : (o.up_n < amin_o - o.b ? -1 : 0);
+    const uint32_t to = step_of(m.m1o);
+    if (act && verdict == 0 && bok && to == step_of(m.m1n) && kTwoSqrt3f * m.m2o - o.b > o.up_o &&
+        kTwoSqrt3f * m.m2n - o.b > o.up_n) {
+        const RingVertex P = w.vertex(L::at(list, to)), Q = w.vertex(L::at(list, to + 1u));
+        verdict = diff_screen(P.x, P.y, Q.x, Q.y, w.Cx, w.Cy, ((w.rev >> to) & 1u) ? -1.0f : 1.0f, M * M);
+    }
+    const unsigned open = __ballot_sync(0xffffffffu, act && verdict == 0);
+    if (act && verdict != 0) {
+        const bool acc = verdict > 0;
+        if (acc) {
+            // the exact squared move is needed only where it can be the block's
+            // largest: the screen's offset gives it to within a few units of 2^-24
+            const float about = fmaf(w.Cx, w.Cx, w.Cy * w.Cy) * 1.000001f + 1e-37f;
+            if (about >= *const_cast<volatile float *>(&q->best_low)) {
+                const ulonglong2 p = *reinterpret_cast<const ulonglong2 *>(xy + own);
+                const double dx = __dsub_rn(bitsd(cb.x), bitsd(p.x)), dy = __dsub_rn(bitsd(cb.y), bitsd(p.y));
+                note_move(q, dbits(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy))));
+            }
+            tally.nacc += 1u;
+            res = 3u;  // the centre differs from the node (equal centres are done above)
+        } else {
+            cb = *reinterpret_cast<const ulonglong2 *>(xy + own);
+        }
+        CoordBits<LAYOUT>::put(a.out, a.n, node, cb);
+        if (a.accept) a.accept[node] = acc ? 1 : 0;
+    }
+    if (open) {
+        if (act && verdict == 0) tally.nexact += 1u;
+        if (!bok) {  // every step is a candidate
+            o.b = 0.0f;
+            o.up_o = o.up_n = __int_as_float(0x7f800000);
+        }
+        o.Cx = w.Cx;
+        o.Cy = w.Cy;
+        o.own = own;
+        o.steps = steps;
+        const uint32_t done = settle_open<LAYOUT, BITS>(a, q, xy, half, list, r.cold, r.irregular, node, cb, o, open);
+        full = full || (done & 8u);
+        if (done & 3u) res = done & 3u;
+        tally.nacc += done & 1u;
+    }
+    return record;
+}
+
+// ---- a block's windows ----------------------------------------------------------
+
+// Nodes of a subtile that their records decide, a warp each.
+template <int LAYOUT, bool COHERENT>
+__device__ __noinline__ Tally by_record(const PassArgs &a, Queue *q, int32_t node, unsigned left, Tally tally)
+{
+    while (left) {
+        const int src = __ffs((int)left) - 1;
+        left &= left - 1u;
+        const int32_t nd = __shfl_sync(0xffffffffu, node, src);
+        unsigned long long b2;
+        bool acc, moved;
+        exact_update_warp<LAYOUT, COHERENT>(a, nd, b2, acc, moved);
+        if ((threadIdx.x & 31) == 0) {
+            note_move(q, b2);
+            tally.nacc += acc ? 1u : 0u;
+            tally.nexact += 1u;
+            if (a.halo) {
+                const uint32_t bit = 1u << (nd & 31);
+                if (moved) atomicOr(a.chg_cur + (nd >> 5), bit);
+                if (acc) atomicOr(a.accm + (nd >> 5), bit);
             }
         }
-        const int rest = qn > 32 ? qn - 32 : 0;
-        __syncwarp();
-        if (lane < rest) wq[lane] = wq[32 + lane];
-        __syncwarp();
-        qn = rest;
+    }
+    return tally;
+}
+
+// Splits the staged entries a thread copied itself (first, first + step, ...).
+__device__ __forceinline__ void split_staged(char *xy, uint32_t half, uint32_t staged, uint32_t first, uint32_t step)
+{
+    for (uint32_t e = first; e < staged; e += step) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(xy + (e + 1u) * 16u);
+        float4 s;
+        const bool okx = head_tail(v.x, s.x, s.y), oky = head_tail(v.y, s.z, s.w);
+        // no split: the rings it is on then fail their range check
+        if (!(okx & oky)) s = make_float4(__int_as_float(0x7f800000), 0.f, __int_as_float(0x7f800000), 0.f);
+        *reinterpret_cast<float4 *>(xy + half + (e + 1u) * 16u) = s;
     }
 }
 
-// Warp-wide reduction of the statistics into one record (lane 0 writes).
-__device__ __forceinline__ void warp_flush_stats(PassStats *st, unsigned long long best,
-                                                 unsigned long long nacc, unsigned long long nfb)
+// Updates the nodes of subtile `sub` of a staged window (h: its header, rows:
+// its hot rows in shared memory).
+template <int LAYOUT, int BITS, bool COHERENT>
+__device__ __forceinline__ void work_subtile(const PassArgs &a, Queue *q, const char *xy, uint32_t half,
+                                             const uint32_t *h, const uint32_t *rows, int sub, Tally &tally,
+                                             bool &full)
 {
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long m2 = __shfl_xor_sync(0xffffffffu, best, o);
-        best = m2 > best ? m2 : best;
-        nacc += __shfl_xor_sync(0xffffffffu, nacc, o);
-        nfb += __shfl_xor_sync(0xffffffffu, nfb, o);
+    const int lane = threadIdx.x & 31;
+    Rows r;
+    r.d = (h[3] >> (8 * sub)) & 15u;
+    r.l = (h[3] >> (8 * sub + 4)) & 15u;
+    r.at = rows + ((h[4] >> (8 * sub)) & 0xffu) * 32u + lane;
+    r.cold = h[0] + win::halo_rows(win::hdr_halo(h[2])) + h[5] + 2u * sub;
+    r.meta = *r.at;
+    r.irregular = win::hdr_irregular(h[2], (uint32_t)sub);
+    const int32_t node = (int32_t)(h[1] + win::meta_place(r.meta));
+    const bool have = (r.meta & win::kNode) != 0u;
+    if (have && !(r.meta & (win::kFree | win::kBig)) && a.accept) a.accept[node] = 0;
+    uint32_t res = 0u;
+    bool record = have && (r.meta & win::kBig);
+    if (r.d > 0u) record |= update_lane<LAYOUT, BITS>(a, q, xy, half, r, node, tally, res, full);
+    __syncwarp();
+    if (a.halo) {  // before any other write to the tile's masks
+        const int64_t wt = (int64_t)(h[1] >> 5) + sub;
+        const unsigned cb = __ballot_sync(0xffffffffu, (res & 2u) != 0u);
+        const unsigned ab = __ballot_sync(0xffffffffu, (res & 1u) != 0u);
+        if (lane == 0 && wt * 32 < (int64_t)h[1] + win::hdr_count(h[2])) {
+            a.chg_cur[wt] = cb;
+            a.accm[wt] = ab;
+        }
     }
-    if ((threadIdx.x & 31) == 0) {
-        if (best) atomicMax(&st->maxd2_bits, best);
-        if (nacc) atomicAdd(&st->nacc, nacc);
-        if (nfb) atomicAdd(&st->fallbacks, nfb);
-    }
+    const unsigned left = __ballot_sync(0xffffffffu, record);
+    if (left) tally = by_record<LAYOUT, COHERENT>(a, q, node, left, tally);
 }
 
-template <int LAYOUT>
-// 128 threads, 7 blocks per SM: 28 warps per SM (72 registers a thread).
-__global__ void __launch_bounds__(128, 7) pass_screened_kernel(PassArgs a)
+// Works windows w0, w0 + stride, ... (n of them).  Every thread of the block
+// calls it; `full` is this thread's note that the queue should be worked off,
+// which happens at the next window's barrier.
+//
+// Window i's data was copied in while window i - 1 was worked on; one barrier
+// per window says that it is there and that window i - 1, whose buffer the
+// next copies overwrite, is finished.  (With one buffer of staged entries the
+// copies wait for that barrier, and a second one says that they are there.)
+template <int LAYOUT, int BITS>
+__device__ __forceinline__ void run_windows(const PassArgs &a, const Block &blk, int64_t w0, int n, int64_t stride,
+                                            Tally &tally, unsigned &nskip, bool &full)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int nthr = blockDim.x;
-    float2 *s_loc = reinterpret_cast<float2 *>(smem_raw);                       // [kFastMax][nthr]
-    Deferred *s_q = reinterpret_cast<Deferred *>(s_loc + kFastMax * nthr);      // [64] per warp
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthr = blockDim.x, nwarps = nthr >> 5;
+    Ahead *ah = blk.ahead;
 
-    if (pass_is_skipped(a.stats, a.q, a.tol_active, a.thr_bits)) return;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (blockIdx.x == 0 && tid == 0) a.stats[a.q].executed = 1u;
-
-    unsigned long long best = 0ull, nacc = 0ull, nfb = 0ull;
-    unsigned nskip = 0u;  // node updates this warp left as they were (lane 0)
-    float2 *loc = s_loc + tid;
-    Deferred *wq = s_q + 64 * warp;
-    int qn = 0;  // warp-uniform queue length
-    // every node in index order, or (a colour class of Form B) the listed
-    // nodes or a range of ids
-    const int64_t cnt = a.order ? a.norder : (a.ranged ? a.count : a.n);
-    const int64_t nwtiles = (cnt + 31) / 32;
-    const int64_t wstride = (int64_t)gridDim.x * (nthr >> 5);
-    for (int64_t wt = (int64_t)blockIdx.x * (nthr >> 5) + warp; wt < nwtiles; wt += wstride) {
-        if (a.skip) {
-            // the tile's inputs: its own nodes and every neighbour, by tile
-            const uint2 h = lane < kHaloEntries ? __ldg(a.halo + wt * kHaloEntries + lane) : make_uint2(0u, 0u);
-            const bool never = __shfl_sync(0xffffffffu, h.x, 0) == kHaloNever;
-            const uint32_t c = h.y != 0u ? __ldg(a.chg_prev + h.x) & h.y : 0u;
-            if (!__any_sync(0xffffffffu, c != 0u) && !never) {
-                // all unchanged: the same inputs as in the previous pass, so the
-                // same results, which `out` and the masks already hold
-                if (lane == 0) {
+    auto fetch_header = [&](int i) {
+        if (i < n && tid < 2)
+            copy16(&ah->hdr[i & 3][4 * tid], a.win_hdr + (w0 + i * stride) * win::kHeaderWords + 4 * tid);
+    };
+    auto fetch_ids = [&](int i) {
+        if (i >= n) return;
+        const uint32_t *h = ah->hdr[i & 3];
+        const uint32_t *src = a.win_rows + (size_t)h[0] * 32u;
+        uint32_t *dst = blk.ids + (i & 1) * blk.ids_words;
+        for (uint32_t k = 4 * tid; k < win::hdr_halo(h[2]); k += 4 * nthr) copy16(dst + k, src + k);
+    };
+    auto all_idle = [&](int i) { return a.skip && *reinterpret_cast<const uint32_t *>(ah->idle[i & 3]) == 0x01010101u; };
+    auto fetch_data = [&](int i) {
+        if (i >= n || all_idle(i)) return;
+        const uint32_t *h = ah->hdr[i & 3];
+        const uint32_t count = win::hdr_count(h[2]), nhalo = win::hdr_halo(h[2]);
+        const uint32_t *src = a.win_rows + ((size_t)h[0] + win::halo_rows(nhalo)) * 32u;
+        uint32_t *rows = blk.rows + (i & 1) * blk.rows_words;
+        for (uint32_t k = 4 * tid; k < 32u * h[5]; k += 4 * nthr) copy16(rows + k, src + k);
+        const uint32_t *ids = blk.ids + (i & 1) * blk.ids_words;
+        char *xy = blk.xy + (i & 1) * blk.stage + 16;
+        for (uint32_t e = tid; e < count + nhalo; e += nthr) {
+            const int64_t id = e < count ? (int64_t)h[1] + e : (int64_t)ids[e - count];
+            if (LAYOUT == 0) {
+                copy16(xy + e * 16u, a.in + 2 * id);
+            } else {
+                copy8(xy + e * 16u, a.in + id);
+                copy8(xy + e * 16u + 8u, a.in + a.n + id);
+            }
+        }
+    };
+    // skip_unchanged: whether the subtiles of window i have only unchanged
+    // inputs; such a tile's results are those of the previous pass, which
+    // `out` and the masks already hold
+    auto check_idle = [&](int i) {
+        if (!a.skip || i >= n) return;
+        const uint32_t *h = ah->hdr[i & 3];
+        for (int sub = warp; sub < 4; sub += nwarps) {
+            const int64_t wt = (int64_t)(h[1] >> 5) + sub;
+            bool idle = true;
+            if (wt * 32 < (int64_t)h[1] + win::hdr_count(h[2])) {
+                // the tile's inputs: its own nodes and every neighbour, by tile
+                const uint2 e = lane < kHaloEntries ? __ldg(a.halo + wt * kHaloEntries + lane) : make_uint2(0u, 0u);
+                const bool never = __shfl_sync(0xffffffffu, e.x, 0) == kHaloNever;
+                const uint32_t c = e.y != 0u && !never ? __ldg(a.chg_prev + e.x) & e.y : 0u;
+                idle = !__any_sync(0xffffffffu, c != 0u) && !never;
+                if (idle && lane == 0) {
                     a.chg_cur[wt] = 0u;
-                    nacc += (unsigned long long)__popc(a.accm[wt]);
+                    tally.nacc += (unsigned)__popc(a.accm[wt]);
                     nskip += (unsigned)(a.n - wt * 32 < 32 ? a.n - wt * 32 : 32);
                 }
-                continue;
             }
+            if (lane == 0) ah->idle[i & 3][sub] = idle ? 1 : 0;
         }
-        const int64_t j = wt * 32 + lane;
-        Deferred d;
-        const bool have = j < cnt;
-        uint32_t res;
-        const bool defer = screen_node<LAYOUT>(a, have, have ? (a.order ? (int64_t)__ldg(a.order + j) : a.first + j) : 0,
-                                               loc, nthr, d, best, nacc, res);
-        const unsigned m = __ballot_sync(0xffffffffu, defer);
-        if (a.halo) {  // before any drain: deferred nodes add their bits there
-            const unsigned cb = __ballot_sync(0xffffffffu, (res & 2u) != 0u);
-            const unsigned ab = __ballot_sync(0xffffffffu, (res & 1u) != 0u);
-            if (lane == 0) {
-                a.chg_cur[wt] = cb;
-                a.accm[wt] = ab;
-            }
+    };
+
+    __syncthreads();  // whatever was worked on before is finished
+    fetch_header(0);
+    fetch_header(1);
+    fetch_header(2);
+    copies_done();
+    __syncthreads();
+    fetch_ids(0);
+    fetch_ids(1);
+    check_idle(0);
+    check_idle(1);
+    copies_done();
+    __syncthreads();
+    if (blk.stage) fetch_data(0);
+    for (int i = 0; i < n; ++i) {
+        if (!blk.stage) {  // one buffer: window i - 1 has to be finished first
+            copies_done();
+            __syncthreads();
+            fetch_data(i);
         }
-        if (defer) wq[qn + __popc(m & ((1u << lane) - 1u))] = d;
-        qn += __popc(m);
-        nfb += defer ? 1ull : 0ull;
-        if (qn >= 32) {  // warp-uniform; entries written by other lanes must be visible
-            __syncwarp();
-            drain_queue<LAYOUT>(a, wq, qn, false, best, nacc);
+        copies_done();
+        char *xy = blk.xy + (i & 1) * blk.stage;
+        const uint32_t *h = ah->hdr[i & 3];
+        const bool rest = all_idle(i);
+        if (!rest) {
+            split_staged(xy, blk.half, win::hdr_count(h[2]) + win::hdr_halo(h[2]), tid, nthr);
+        }
+        if (__syncthreads_or(full)) {
+            tally = drain<LAYOUT>(a, blk.q, tally);
+            full = false;
+        }
+        if (blk.stage) fetch_data(i + 1);
+        fetch_ids(i + 2);
+        fetch_header(i + 3);
+        check_idle(i + 2);
+        if (rest) continue;
+        for (int sub = warp; sub < 4; sub += nwarps) {
+            if (a.skip && ah->idle[i & 3][sub]) continue;
+            work_subtile<LAYOUT, BITS, false>(a, blk.q, xy, blk.half, h, blk.rows + (i & 1) * blk.rows_words, sub, tally,
+                                              full);
         }
     }
-    __syncwarp();
-    drain_queue<LAYOUT>(a, wq, qn, true, best, nacc);
+}
+
+// The kernels are compiled for 7 blocks of 128 threads per SM (72 registers):
+// 2048^2 runs 228 us a pass with 7, 233 with 6 and 239 with 8, whose 64
+// registers spill.
+constexpr int kBlocksPerSm = 7;
+
+template <int LAYOUT, int BITS>
+__global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
+    pass_screened_kernel(const __grid_constant__ PassArgs a, const __grid_constant__ WindowShape shape)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    if (pass_is_skipped(a.stats, a.q, a.tol_active, a.thr_bits)) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.stats[a.q].executed = 1u;
+    const Block blk = block_memory(smem_raw, shape);
+    Tally tally{0u, 0u};
+    unsigned nskip = 0u;  // node updates this warp left as they were (lane 0)
+    bool full = false;
+    if ((int64_t)blockIdx.x < a.win_count)
+        run_windows<LAYOUT, BITS>(a, blk, a.win_first + blockIdx.x,
+                                  (int)((a.win_count - blockIdx.x + gridDim.x - 1) / gridDim.x), gridDim.x, tally,
+                                  nskip, full);
+    __syncthreads();
+    if (blk.q->npending) tally = drain<LAYOUT>(a, blk.q, tally);
     if (nskip) atomicAdd(&a.stats[a.q].nodes_skipped, nskip);
-    block_reduce_stats(a.stats + a.q, best, nacc, nfb);
+    flush(blk.q, a.stats + a.q, tally);
+}
+
+// ---- all passes of a small mesh in one launch -----------------------------------
+// A mesh with at most one window per resident block: every block keeps its
+// window's lists in shared memory and runs pass after pass, with a grid-wide
+// barrier between passes instead of a launch.  What is left of a pass is its
+// own chain of dependent steps (coordinates from L2, the sums, the ring walk,
+// the queue, the barrier).  A 64^2 mesh runs 9.3 us a pass against 13.5 with a
+// launch each, 100,000 Delaunay points 19 against 23; past one window per
+// resident block (about 136,000 nodes) the blocks would have to fetch their
+// lists again every pass, as separate launches do.
+
+struct GridBarrier {
+    unsigned int arrived;  // blocks that arrived, over all passes of the launch
+    unsigned int lost;     // a wait ran out: nobody waits any more
+};
+
+// Polls before a waiting block gives up (a poll takes about a microsecond; a
+// pass of such a mesh some tens of them).
+constexpr unsigned kPollLimit = 1u << 22;
+
+// All threads call it; false when some block's wait ran out.  Writes to global
+// memory before it are visible after it to reads from L2.
+__device__ __forceinline__ bool grid_barrier(GridBarrier *b, unsigned target)
+{
+    __shared__ bool s_ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(&b->arrived, 1u);
+        unsigned seen = 0u, polls = 0u;
+        do {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&b->arrived) : "memory");
+        } while (seen < target && ++polls < kPollLimit);
+        s_ok = seen >= target;
+        if (!s_ok) atomicExch(&b->lost, 1u);
+    }
+    __syncthreads();
+    return s_ok;
+}
+
+template <int LAYOUT, int BITS>
+__global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
+    resident_kernel(const __grid_constant__ PassArgs a0, const __grid_constant__ WindowShape shape, int passes,
+                    GridBarrier *barrier)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ PassArgs s_args;
+    __shared__ bool s_stop;
+    const int tid = threadIdx.x, warp = tid >> 5, nthr = blockDim.x, nwarps = nthr >> 5;
+    const Block blk = block_memory(smem_raw, shape);
+    if (tid == 0) {
+        s_args = a0;
+        s_stop = pass_is_skipped(a0.stats, a0.q, a0.tol_active, a0.thr_bits);
+    }
+    // the window's header, halo ids and lists, once
+    uint32_t *h = blk.ahead->hdr[0];
+    if (tid < 2) copy16(h + 4 * tid, a0.win_hdr + (size_t)blockIdx.x * win::kHeaderWords + 4 * tid);
+    copies_done();
+    __syncthreads();
+    if (s_stop) return;
+    const uint32_t count = win::hdr_count(h[2]), nhalo = win::hdr_halo(h[2]), staged = count + nhalo;
+    const uint32_t *src = a0.win_rows + (size_t)h[0] * 32u;
+    for (uint32_t k = 4 * tid; k < nhalo; k += 4 * nthr) copy16(blk.ids + k, src + k);
+    src += win::halo_rows(nhalo) * 32u;
+    for (uint32_t k = 4 * tid; k < 32u * h[5]; k += 4 * nthr) copy16(blk.rows + k, src + k);
+    copies_done();
+    __syncthreads();
+    const PassArgs &a = s_args;
+    const double *in = a0.in;
+    for (int done = 1;; ++done) {
+        for (uint32_t e = tid; e < staged; e += nthr) {  // from L2: other blocks wrote them
+            const int64_t id = e < count ? (int64_t)h[1] + e : (int64_t)blk.ids[e - count];
+            char *dst = blk.xy + (e + 1u) * 16u;
+            if (LAYOUT == 0) {
+                copy16(dst, in + 2 * id);
+            } else {
+                *reinterpret_cast<double2 *>(dst) = make_double2(__ldcg(in + id), __ldcg(in + a0.n + id));
+            }
+        }
+        if (tid == 0 && done > 1 && a0.tol_active) {  // the pass before met the tolerance
+            unsigned long long moved;
+            asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(moved) : "l"(&a0.stats[a.q - 1].maxd2_bits));
+            s_stop = moved < a0.thr_bits;
+        }
+        copies_done();
+        split_staged(blk.xy, blk.half, staged, tid, nthr);
+        __syncthreads();
+        if (s_stop) return;
+        if (blockIdx.x == 0 && tid == 0) a.stats[a.q].executed = 1u;
+        Tally tally{0u, 0u};
+        bool full = false;  // (one window: the queue is worked off after it)
+        for (int sub = warp; sub < 4; sub += nwarps)
+            work_subtile<LAYOUT, BITS, true>(a, blk.q, blk.xy, blk.half, h, blk.rows, sub, tally, full);
+        __syncthreads();
+        if (blk.q->npending) tally = drain<LAYOUT>(a, blk.q, tally);
+        flush(blk.q, a.stats + a.q, tally);
+        if (done == passes) return;
+        in = (done & 1) ? a0.out : a0.in;
+        if (tid == 0) {
+            s_args.in = in;
+            s_args.out = (done & 1) ? const_cast<double *>(a0.in) : a0.out;
+            s_args.q += 1;
+        }
+        if (!grid_barrier(barrier, (unsigned)done * gridDim.x)) return;
+    }
 }
 
 // ---- batched / served form: many meshes, one launch per round -----------
-// Work is a list of warp tasks (32 consecutive nodes of one job).  With
-// chunk > 0 the warps take chunks of `chunk` consecutive tasks in a grid
-// stride (warp w: chunks w, w + W, w + 2W, ...), so that at any moment they
-// work on a window of neighbouring tasks and share its gathers in L1 and L2;
-// with chunk < 0 they claim chunks of -chunk tasks in list order from the
-// round's counter (*claim, zero at the launch), which keeps that window and
-// lets a warp that drew cheap tasks take more; chunk = 0 gives each warp one
-// contiguous share of the list.  A job takes part in
-// round r as its pass q = r - base_round while q < max_iter and its
-// tolerance is not met.  The deferred queue is drained and the statistics
-// flushed whenever the warp moves to another job, so every record gets
-// exactly its own job's counts.
-template <int LAYOUT>
-__global__ void __launch_bounds__(128, 6) batch_pass_kernel(const JobDesc *__restrict__ jobs,
-                                                          const WarpTask *__restrict__ tasks, int64_t ntasks,
-                                                          int round, int64_t chunk,
-                                                          unsigned long long *claim)
+// Work is a list of window tasks.  With chunk > 0 the blocks take chunks of
+// `chunk` consecutive tasks in a grid stride (block b: chunks b, b + B,
+// b + 2B, ...); with chunk < 0 they claim chunks of -chunk tasks in list order
+// from the round's counter (*claim, zero at the launch); chunk = 0 gives each
+// block one contiguous share of the list.  A job takes part in round r as its
+// pass q = r - base_round while q < max_iter and its tolerance is not met.
+// The queue is worked off and the statistics flushed whenever the block moves
+// to another job, so every record gets exactly its own job's counts.
+// WIDE: some job's lists may have 16-bit entries.
+template <int LAYOUT, bool WIDE>
+__global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
+    batch_pass_kernel(const JobDesc *__restrict__ jobs, const WindowTask *__restrict__ tasks, int64_t ntasks,
+                      int round, int64_t chunk, unsigned long long *claim, const __grid_constant__ WindowShape shape)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int nthr = blockDim.x;
-    float2 *s_loc = reinterpret_cast<float2 *>(smem_raw);
-    Deferred *s_q = reinterpret_cast<Deferred *>(s_loc + kFastMax * nthr);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    float2 *loc = s_loc + tid;
-    Deferred *wq = s_q + 64 * warp;
-
-    const int64_t nwarps = (int64_t)gridDim.x * (nthr >> 5);
-    const int64_t gw = (int64_t)blockIdx.x * (nthr >> 5) + warp;
+    __shared__ PassArgs s_args;
+    __shared__ int64_t s_claim;
+    __shared__ int s_active, s_wide, s_windows;
+    const Block blk = block_memory(smem_raw, shape);
     const bool dynamic = chunk < 0;
-    const int64_t per = chunk > 0 ? chunk : (dynamic ? -chunk : (ntasks + nwarps - 1) / nwarps);
-    const int64_t cstride = chunk > 0 ? nwarps * chunk : ntasks;  // one share per warp when chunk == 0
+    const int64_t nblocks = gridDim.x;
+    const int64_t per = chunk > 0 ? chunk : (dynamic ? -chunk : (ntasks + nblocks - 1) / nblocks);
+    const int64_t cstride = chunk > 0 ? nblocks * chunk : ntasks;  // one share per block when chunk == 0
     auto claim_next = [&]() -> int64_t {
-        unsigned long long v = 0ull;
-        if (lane == 0) v = atomicAdd(claim, (unsigned long long)per);
-        return (int64_t)__shfl_sync(0xffffffffu, v, 0);
+        __syncthreads();
+        if (threadIdx.x == 0) s_claim = (int64_t)atomicAdd(claim, (unsigned long long)per);
+        __syncthreads();
+        return s_claim;
     };
-    int64_t c0 = dynamic ? claim_next() : gw * per;  // first task of the current chunk
+    int64_t c0 = dynamic ? claim_next() : (int64_t)blockIdx.x * per;  // first task of the current chunk
     int64_t t = c0;
-
     int cur_job = -1;
-    bool active = false;
-    PassArgs a{};
-    unsigned long long best = 0ull, nacc = 0ull, nfb = 0ull;
-    int qn = 0;
+    Tally tally{0u, 0u};
+    unsigned nskip = 0u;
+    bool full = false, active = false;
     for (;;) {
-        if (t >= c0 + per || t >= ntasks) {  // next chunk of this warp
+        if (t >= c0 + per || t >= ntasks) {  // next chunk of this block
             c0 = dynamic ? (c0 < ntasks ? claim_next() : c0) : c0 + cstride;
             t = c0;
         }
         const bool more = t < ntasks && c0 < ntasks;
         const int job = more ? tasks[t].job : -2;
         if (job != cur_job) {
+            __syncthreads();
             if (cur_job >= 0 && active) {
-                __syncwarp();
-                drain_queue<LAYOUT>(a, wq, qn, true, best, nacc);
-                warp_flush_stats(a.stats + a.q, best, nacc, nfb);
+                if (blk.q->npending) tally = drain<LAYOUT>(s_args, blk.q, tally);
+                flush(blk.q, s_args.stats + s_args.q, tally);
+                __syncthreads();
             }
-            best = nacc = nfb = 0ull;
+            tally = Tally{0u, 0u};
+            full = false;
             cur_job = job;
             if (job < 0) break;
-            const JobDesc *J = jobs + job;
-            const int q = round - J->base_round;
-            PassStats *st = J->stats;
-            const int tol_active = J->tol_active;
-            const unsigned long long thr_bits = J->thr_bits;
-            active = q >= 0 && q < J->max_iter && !pass_is_skipped(st, q, tol_active, thr_bits);
-            if (active) {
-                double *x0 = J->xy[0], *x1 = J->xy[1];
+            if (threadIdx.x == 0) {
+                const JobDesc *J = jobs + job;
+                const int q = round - J->base_round;
+                PassArgs &a = s_args;
+                a = PassArgs{};
                 const bool odd = ((J->cur0 + q) & 1) != 0;
-                a.in = odd ? x1 : x0;
-                a.out = odd ? x0 : x1;
+                a.in = odd ? J->xy[1] : J->xy[0];
+                a.out = odd ? J->xy[0] : J->xy[1];
                 a.node_off = J->node_off;
                 a.adj = J->adj;
                 a.n = J->n;
-                a.order = nullptr;
-                a.norder = 0;
-                a.stats = st;
+                a.win_hdr = J->win_hdr;
+                a.win_rows = J->win_rows;
+                a.stats = J->stats;
                 a.q = q;
                 a.strict = J->strict;
-                a.tol_active = tol_active;
-                a.thr_bits = thr_bits;
+                a.tol_active = J->tol_active;
+                a.thr_bits = J->thr_bits;
                 a.accept = J->accept;
+                s_wide = J->bits != 8;
+                s_windows = J->windows;
+                s_active = q >= 0 && q < J->max_iter && !pass_is_skipped(J->stats, q, J->tol_active, J->thr_bits);
             }
+            __syncthreads();
+            active = s_active != 0;
         }
-        if (!active) {
-            ++t;
-            continue;
-        }
-        const int64_t first = tasks[t].first;
-        ++t;
-        if (first == 0 && lane == 0) a.stats[a.q].executed = 1u;
-        const int64_t i = first + lane;
-        Deferred d;
-        uint32_t res;
-        const bool defer = screen_node<LAYOUT>(a, i < a.n, i < a.n ? i : 0, loc, nthr, d, best, nacc, res);
-        const unsigned m = __ballot_sync(0xffffffffu, defer);
-        if (defer) wq[qn + __popc(m & ((1u << lane) - 1u))] = d;
-        qn += __popc(m);
-        nfb += defer ? 1ull : 0ull;
-        if (qn >= 32) {
-            __syncwarp();
-            drain_queue<LAYOUT>(a, wq, qn, false, best, nacc);
-        }
+        // the job's windows up to the end of the chunk
+        const int window = tasks[t].window;
+        int64_t run = s_windows - window;
+        if (run > c0 + per - t) run = c0 + per - t;
+        if (run > ntasks - t) run = ntasks - t;
+        t += run;
+        if (!active) continue;
+        if (window == 0 && threadIdx.x == 0) s_args.stats[s_args.q].executed = 1u;
+        if (WIDE && s_wide)
+            run_windows<LAYOUT, 16>(s_args, blk, window, (int)run, 1, tally, nskip, full);
+        else
+            run_windows<LAYOUT, 8>(s_args, blk, window, (int)run, 1, tally, nskip, full);
     }
+}
+
+const void *kernel_of(int layout, int bits)
+{
+    if (layout == 0)
+        return bits == 8 ? (const void *)pass_screened_kernel<0, 8> : (const void *)pass_screened_kernel<0, 16>;
+    return bits == 8 ? (const void *)pass_screened_kernel<1, 8> : (const void *)pass_screened_kernel<1, 16>;
+}
+
+const void *resident_kernel_of(int layout, int bits)
+{
+    if (layout == 0) return bits == 8 ? (const void *)resident_kernel<0, 8> : (const void *)resident_kernel<0, 16>;
+    return bits == 8 ? (const void *)resident_kernel<1, 8> : (const void *)resident_kernel<1, 16>;
+}
+
+const void *batch_kernel_of(int layout, int bits)
+{
+    if (layout == 0)
+        return bits == 8 ? (const void *)batch_pass_kernel<0, false> : (const void *)batch_pass_kernel<0, true>;
+    return bits == 8 ? (const void *)batch_pass_kernel<1, false> : (const void *)batch_pass_kernel<1, true>;
 }
 
 // Constant memory and function attributes belong to a context: they are set
@@ -517,19 +1144,21 @@ cudaError_t ensure_constants()
     if (g_consts_ctx[dev].load(std::memory_order_acquire) == key) return cudaSuccess;
     std::lock_guard<std::mutex> lock(g_consts_mu);
     if (g_consts_ctx[dev].load(std::memory_order_relaxed) == key) return cudaSuccess;
-    double r[kFastMax + 1];
-    double dg[kFastMax + 1];
+    double r[kRingMax + 1];
+    double dg[kRingMax + 1];
     r[0] = 0.0;
     dg[0] = 0.0;
-    for (int k = 1; k <= kFastMax; ++k) {
+    for (int k = 1; k <= kRingMax; ++k) {
         r[k] = 1.0 / (double)k;
         dg[k] = (double)k;
     }
     e = cudaMemcpyToSymbol(c_recip, r, sizeof r);
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_degree, dg, sizeof dg);
     if (e != cudaSuccess) return e;
-    const void *fns[4] = {(const void *)pass_screened_kernel<0>, (const void *)pass_screened_kernel<1>,
-                          (const void *)batch_pass_kernel<0>, (const void *)batch_pass_kernel<1>};
+    const void *fns[12] = {kernel_of(0, 8),       kernel_of(0, 16),      kernel_of(1, 8),
+                          kernel_of(1, 16),      batch_kernel_of(0, 8), batch_kernel_of(0, 16),
+                          batch_kernel_of(1, 8), batch_kernel_of(1, 16), resident_kernel_of(0, 8),
+                          resident_kernel_of(0, 16), resident_kernel_of(1, 8), resident_kernel_of(1, 16)};
     for (const void *f : fns) {
         e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         if (e != cudaSuccess) return e;
@@ -538,35 +1167,55 @@ cudaError_t ensure_constants()
     return cudaSuccess;
 }
 
-}  // namespace
-
-size_t screened_smem_bytes(int block)
+int occupancy(const void *f, int block, const WindowShape &shape)
 {
-    return (size_t)block * (kFastMax * sizeof(float2) + 2 * sizeof(Deferred));  // 64 entries per warp
+    if (ensure_constants() != cudaSuccess) return 1;
+    int nb = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, block, smem_for(shape));
+    return nb > 0 ? nb : 1;
 }
 
-cudaError_t launch_pass_screened(const PassArgs &a, int layout, int block, int grid, cudaStream_t s)
+}  // namespace
+
+cudaError_t launch_pass_screened(const PassArgs &a, int layout, int block, int grid, const WindowShape &shape,
+                                 cudaStream_t s)
 {
     cudaError_t e = ensure_constants();
     if (e != cudaSuccess) return e;
-    const size_t smem = screened_smem_bytes(block);
-    if (layout == 0) pass_screened_kernel<0><<<grid, block, smem, s>>>(a);
-    else pass_screened_kernel<1><<<grid, block, smem, s>>>(a);
-    return cudaGetLastError();
+    if (a.win_count < grid) grid = a.win_count > 0 ? (int)a.win_count : 1;
+    void *args[] = {const_cast<PassArgs *>(&a), const_cast<WindowShape *>(&shape)};
+    return cudaLaunchKernel(kernel_of(layout, shape.bits), dim3(grid), dim3(block), args, smem_for(shape), s);
 }
 
-cudaError_t launch_batch_pass(const JobDesc *jobs, const WarpTask *tasks, int64_t ntasks, int round,
-                              int layout, int block, int grid, cudaStream_t s, int64_t chunk,
+bool resident_fits(const PassArgs &a, int layout, int block, const WindowShape &shape)
+{
+    return a.win_count > 0 &&
+           a.win_count <= (int64_t)device_sm_count() * occupancy(resident_kernel_of(layout, shape.bits), block, shape);
+}
+
+cudaError_t launch_resident(const PassArgs &a, int layout, int block, const WindowShape &shape, int passes,
+                            unsigned *barrier, cudaStream_t s)
+{
+    static_assert(sizeof(GridBarrier) == kBarrierWords * sizeof(unsigned), "barrier words");
+    cudaError_t e = ensure_constants();
+    if (e != cudaSuccess) return e;
+    GridBarrier *b = reinterpret_cast<GridBarrier *>(barrier);
+    void *args[] = {const_cast<PassArgs *>(&a), const_cast<WindowShape *>(&shape), &passes, &b};
+    return cudaLaunchCooperativeKernel(resident_kernel_of(layout, shape.bits), dim3((unsigned)a.win_count), dim3(block),
+                                       args, smem_for(shape), s);
+}
+
+cudaError_t launch_batch_pass(const JobDesc *jobs, const WindowTask *tasks, int64_t ntasks, int round, int layout,
+                              int block, int grid, const WindowShape &shape, cudaStream_t s, int64_t chunk,
                               unsigned long long *claim)
 {
     cudaError_t e = ensure_constants();
     if (e != cudaSuccess) return e;
     if (ntasks <= 0) return cudaSuccess;
     if (chunk < 0 && !claim) return cudaErrorInvalidValue;
-    const size_t smem = screened_smem_bytes(block);
-    if (layout == 0) batch_pass_kernel<0><<<grid, block, smem, s>>>(jobs, tasks, ntasks, round, chunk, claim);
-    else batch_pass_kernel<1><<<grid, block, smem, s>>>(jobs, tasks, ntasks, round, chunk, claim);
-    return cudaGetLastError();
+    if (ntasks < grid) grid = (int)ntasks;
+    void *args[] = {&jobs, &tasks, &ntasks, &round, &chunk, &claim, const_cast<WindowShape *>(&shape)};
+    return cudaLaunchKernel(batch_kernel_of(layout, shape.bits), dim3(grid), dim3(block), args, smem_for(shape), s);
 }
 
 namespace {
@@ -582,20 +1231,19 @@ __global__ void gather_round_kernel(const JobDesc *__restrict__ jobs, int na, in
     out[j] = J.stats[q];
 }
 
-// The warp tasks of na jobs: job j's 32-node tasks at task_off[j] onwards.
+// The window tasks of na jobs: job j's at task_off[j] onwards.
 __global__ void expand_tasks_kernel(const JobDesc *__restrict__ jobs, const int64_t *__restrict__ task_off, int na,
-                                    WarpTask *__restrict__ tasks)
+                                    WindowTask *__restrict__ tasks)
 {
     for (int j = blockIdx.x; j < na; j += gridDim.x) {
-        const int64_t n = jobs[j].n, t0 = task_off[j];
-        for (int64_t f = (int64_t)threadIdx.x * 32; f < n; f += (int64_t)blockDim.x * 32)
-            tasks[t0 + f / 32] = WarpTask{j, (int32_t)f};
+        const int64_t t0 = task_off[j];
+        for (int k = threadIdx.x; k < jobs[j].windows; k += blockDim.x) tasks[t0 + k] = WindowTask{j, k};
     }
 }
 
 }  // namespace
 
-cudaError_t launch_expand_tasks(const JobDesc *jobs, const int64_t *task_off, int na, WarpTask *tasks,
+cudaError_t launch_expand_tasks(const JobDesc *jobs, const int64_t *task_off, int na, WindowTask *tasks,
                                 cudaStream_t s)
 {
     if (na <= 0) return cudaSuccess;
@@ -610,28 +1258,14 @@ cudaError_t launch_gather_round(const JobDesc *jobs, int na, int round, PassStat
     return cudaGetLastError();
 }
 
-int batch_pass_occupancy(int layout, int block)
+int batch_pass_occupancy(int layout, int block, const WindowShape &shape)
 {
-    if (ensure_constants() != cudaSuccess) return 1;
-    int nb = 0;
-    const size_t smem = screened_smem_bytes(block);
-    if (layout == 0)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_pass_kernel<0>, block, smem);
-    else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_pass_kernel<1>, block, smem);
-    return nb > 0 ? nb : 1;
+    return occupancy(batch_kernel_of(layout, shape.bits), block, shape);
 }
 
-int pass_screened_occupancy(int layout, int block)
+int pass_screened_occupancy(int layout, int block, const WindowShape &shape)
 {
-    if (ensure_constants() != cudaSuccess) return 1;
-    int nb = 0;
-    const size_t smem = screened_smem_bytes(block);
-    if (layout == 0)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, pass_screened_kernel<0>, block, smem);
-    else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, pass_screened_kernel<1>, block, smem);
-    return nb > 0 ? nb : 1;
+    return occupancy(kernel_of(layout, shape.bits), block, shape);
 }
 
 }  // namespace sls

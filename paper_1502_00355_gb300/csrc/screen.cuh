@@ -70,16 +70,17 @@ SLS_SC_HD float rcp_approx(float s)
 SLS_SC_HD bool head_tail(unsigned long long b, float &hd, float &tl)
 {
     const unsigned hw = (unsigned)(b >> 32), lw = (unsigned)b;
-    const unsigned e = (hw >> 20) & 0x7ffu;
-    const bool zero = (hw & 0x7fffffffu) == 0u && lw == 0u;
-    const unsigned sign = hw & 0x80000000u;
-    const float h = u2f(sign | ((e - 896u) << 23) | ((hw & 0xfffffu) << 3) | (lw >> 29));
-    // tail bits 28..6 of the low word, value t * 2^(E - 46): exact in FP32
-    const float t = u2f(0x4b000000u | ((lw >> 6) & 0x7fffffu)) - 8388608.0f;
-    const float l = u2f(f2u(t * u2f((e - 942u) << 23)) | sign);
-    hd = zero ? 0.0f : h;
-    tl = zero ? 0.0f : l;
-    return zero || (e - 943u <= 206u);  // [2^-80, 2^127) in magnitude, normal
+    const unsigned mag = hw & 0x7fffffffu;
+    const bool in = mag - (943u << 20) < (207u << 20);  // [2^-80, 2^127) in magnitude
+    // head: the double's exponent field less 896 and its top 23 fraction bits
+    const unsigned h = (((hw << 3) | (lw >> 29)) + 0x40000000u) | (hw & 0x80000000u);
+    // tail: bits 28..6 of the low word as a fraction of the head's power of
+    // two, 2^-23 of it apart: exact in FP32
+    const float f = u2f(0x3f800000u | ((lw >> 6) & 0x7fffffu)) - 1.0f;
+    const float t = f * u2f((h & 0xff800000u) - (23u << 23));
+    hd = in ? u2f(h) : 0.0f;
+    tl = in ? t : 0.0f;
+    return in | ((mag | lw) == 0u);
 }
 
 // FP32 value of a double, truncated to 24 significant bits (relative error
@@ -216,6 +217,80 @@ SLS_SC_HD int diff_screen(float Ax, float Ay, float Bx, float By, float Cx, floa
     if (!(fabsf(N) - 2.0f * eN > need)) return 0;
     return ((N > 0.0f) == (sgn > 0.0f)) ? 1 : -1;
 }
+
+// ---- the ring form of the screen ------------------------------------------
+// A node's triangles walked around its ring (window.cuh): consecutive
+// triangles share a vertex, so every vertex's part of an alpha is computed
+// once.  For the triangle (X, P, Q) with X = 0 before the move and X = C
+// after it, P -> Q the stored orientation:
+//   cross = (P - X) x (Q - X),   s = (|P - X|^2 + |Q - X|^2) + |Q - P|^2
+// and the value kept is cross / s, alpha without its factor 2 sqrt(3), with
+// the step's number in the low four bits (so a minimum names its triangle).
+//
+// Error budget against screen_alpha's (above): the same coordinates and cross
+// products; s is a sum of three squared lengths (4 e s of rounding instead of
+// 6.1 e s); the same number of roundings after it (the constant is multiplied
+// in last).  The step's number changes a value by at most 15 units of 2^-23
+// of it, 30 e |alpha|.  Exact alpha is at most 1 in magnitude, and within the
+// bound's range (g <= kGMax) the computed one is within 0.03 of it, so 1.05
+// stands for the side's largest |alpha|; and one bound, from the larger
+// radius and the smallest edge sum of both sides, serves both.
+constexpr float kPackEps = 1.5f * 32.0f * kEps;
+
+// 1/s to within 2 ulp for normal s (rcp.approx.ftz is within 1); an s of zero
+// or below the normal range gives infinity, and the bound then does not hold.
+SLS_SC_HD float rcp_ring(float s)
+{
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(s));
+    return r;
+#else
+    return SLS_SCREEN_HOST_RCP(s);
+#endif
+}
+
+// A ring vertex: its local coordinates before (x, y) and after the move
+// (xc, yc), with their squared lengths.
+struct RingVertex {
+    float x, y, n, xc, yc, nc;
+};
+
+// From the vertex's head/tail splits (hx, lx, hy, ly), the node's
+// (phx, plx, phy, ply) and the centre's offset C.
+SLS_SC_HD RingVertex ring_vertex(float hx, float lx, float hy, float ly, float phx, float plx, float phy, float ply,
+                                 float Cx, float Cy)
+{
+    RingVertex v;
+    v.x = (hx - phx) + (lx - plx);
+    v.y = (hy - phy) + (ly - ply);
+    v.n = fmaf(v.x, v.x, v.y * v.y);
+    v.xc = v.x - Cx;
+    v.yc = v.y - Cy;
+    v.nc = fmaf(v.xc, v.xc, v.yc * v.yc);
+    return v;
+}
+
+// cross / s of the triangle (node, P, Q) before (vo) and after the move (vn),
+// and both edge sums.
+SLS_SC_HD void ring_values(const RingVertex &P, const RingVertex &Q, float &vo, float &vn, float &so, float &sn)
+{
+    const float bx = Q.x - P.x, by = Q.y - P.y;
+    const float b2 = fmaf(bx, bx, by * by);
+    so = (P.n + Q.n) + b2;
+    sn = (P.nc + Q.nc) + b2;
+    vo = fmaf(P.x, Q.y, -(P.y * Q.x)) * rcp_ring(so);
+    vn = fmaf(P.xc, Q.yc, -(P.yc * Q.xc)) * rcp_ring(sn);
+}
+
+SLS_SC_HD float with_step(float v, uint32_t step) { return u2f((f2u(v) & 0xfffffff0u) | step); }
+SLS_SC_HD uint32_t step_of(float v) { return f2u(v) & 15u; }
+
+// Whether the ring form's bound holds (smin the smallest edge sum of both
+// sides, g = R^2 / smin), and the bound: alpha (FP64) of every triangle lies
+// within it of 2 sqrt(3) times the packed value.
+SLS_SC_HD bool ring_ok(float smin, float g) { return (smin > 0.0f) & (g <= kGMax); }
+SLS_SC_HD float ring_bound(float g) { return side_bound(1.05f, g) + kPackEps; }
 
 }  // namespace scr
 }  // namespace sls

@@ -42,9 +42,9 @@ namespace {
 using Clock = std::chrono::steady_clock;
 
 constexpr int kBuilders = 4;  // builder threads (and streams) per server (12 measured no faster)
-// Warp tasks of a round: one contiguous share of the list per warp (short
-// chunks make warps change job often, and every change drains the warp's
-// deferred nodes at partial width; measured on the batched form).
+// Window tasks of a round: one contiguous share of the list per block (short
+// chunks make blocks change job often, and every change works off the block's
+// queue at partial width; measured on the batched form).
 constexpr int64_t kServerChunk = 0;
 
 enum JobState { kQueued, kBuilding, kActive, kRetiring, kDone, kFailed };
@@ -139,7 +139,8 @@ struct ServerJob {
     // device state (stream-ordered allocations)
     double *d_xy[2] = {nullptr, nullptr};
     uint32_t *d_off = nullptr, *d_adj = nullptr;
-    uint32_t *d_perm = nullptr;  // grouped numbering: internal id -> the caller's id (NULL: none)
+    WindowStream windows;
+    uint32_t *d_perm = nullptr;  // renumbered: internal id -> the caller's id (NULL: not)
     PassStats *d_stats = nullptr;
     cudaStream_t build_stream = nullptr;  // the builder stream the memory was allocated on
     cudaEvent_t uploaded = nullptr;
@@ -204,7 +205,7 @@ struct sls_server {
     // is launched before the records of round r are read
     JobDesc *d_jobs = nullptr, *h_jobs[2] = {nullptr, nullptr};
     int64_t *d_toff = nullptr, *h_toff[2] = {nullptr, nullptr};  // first task of each job
-    WarpTask *d_tasks = nullptr;
+    WindowTask *d_tasks = nullptr;
     size_t jobs_cap = 0, jobs_hcap[2] = {0, 0}, toff_cap = 0, toff_hcap[2] = {0, 0}, tasks_cap = 0;
     PassStats *h_round[2] = {nullptr, nullptr};  // pinned: a round's record of each job it ran over
     PassStats *d_round[2] = {nullptr, nullptr};  // the same records gathered on the device
@@ -212,6 +213,7 @@ struct sls_server {
     cudaEvent_t ev_start[2] = {nullptr, nullptr}, ev_done[2] = {nullptr, nullptr};
     int64_t ntasks = 0;
     int block = 256, grid = 0;
+    WindowShape shape;  // covers the windows of the active set
     int round = 0;
 
     // statistics
@@ -225,21 +227,24 @@ struct sls_server {
 namespace {
 
 // Device bytes a job holds once built: two coordinate arrays, node offsets,
-// adjacency words, the numbering map, one statistics record per pass.
-size_t built_footprint(int64_t n, uint64_t adj_words, int32_t max_iter)
+// adjacency words, the window stream, the numbering map, one statistics
+// record per pass.
+size_t built_footprint(int64_t n, uint64_t adj_words, size_t stream_bytes, int32_t max_iter)
 {
     return 2 * sizeof(double) * 2 * (size_t)n + sizeof(uint32_t) * (size_t)(n + 1) + sizeof(uint32_t) * adj_words +
-           sizeof(uint32_t) * (size_t)n + sizeof(PassStats) * (size_t)std::max(1, max_iter);
+           stream_bytes + sizeof(uint32_t) * (size_t)n + sizeof(PassStats) * (size_t)std::max(1, max_iter);
 }
 
 // A bound on what a job holds while it is built: the built footprint with
 // at most n + 9m adjacency words (a meta word per node; per corner of a
-// triangle at most two neighbours and one triangle code), plus the build's
-// scratch (triangles, incidences, neighbour candidates, counts and flags;
-// the numbering's inverse map and new offsets).
+// triangle at most two neighbours and one triangle code) and a window stream
+// whose every subtile has rings of the longest kind and whose every
+// neighbour is in a halo, plus the build's scratch (triangles, incidences,
+// neighbour candidates, counts and flags).
 size_t admission_bound(int64_t n, int64_t m, int32_t max_iter)
 {
-    return built_footprint(n, (uint64_t)(n + 9 * m), max_iter) + 26 * (size_t)n + 48 * (size_t)m + 65536;
+    return built_footprint(n, (uint64_t)(n + 9 * m), 76 * (size_t)n + 24 * (size_t)m, max_iter) + 74 * (size_t)n +
+           48 * (size_t)m + 65536;
 }
 
 void fail_job(sls_server *S, ServerJob &J, sls_status st, const std::string &msg)
@@ -256,6 +261,7 @@ void free_job_device(ServerJob &J, cudaStream_t s)
     for (void *p : {(void *)J.d_xy[0], (void *)J.d_xy[1], (void *)J.d_off, (void *)J.d_adj, (void *)J.d_perm,
                     (void *)J.d_stats})
         if (p) cudaFreeAsync(p, s);
+    J.windows.release(s);
     if (J.uploaded) cudaEventDestroy(J.uploaded);
     J.d_xy[0] = J.d_xy[1] = nullptr;
     J.d_off = J.d_adj = J.d_perm = nullptr;
@@ -266,7 +272,7 @@ void free_job_device(ServerJob &J, cudaStream_t s)
 // Uploads job J on stream s and builds its adjacency there.  On success the
 // job's device state is complete once J.uploaded has fired; *footprint is
 // what it holds.  On failure everything is freed behind the stream's work.
-sls_status build_job(ServerJob &J, bool group, cudaStream_t s, size_t *footprint)
+sls_status build_job(ServerJob &J, bool group, bool numbers, cudaStream_t s, size_t *footprint)
 {
     const int64_t n = J.n, m = J.m;
     const size_t cbytes = sizeof(double) * 2 * (size_t)n;
@@ -294,7 +300,7 @@ sls_status build_job(ServerJob &J, bool group, cudaStream_t s, size_t *footprint
     if (e == cudaSuccess) e = cudaEventRecord(J.in_done, s);
     if (e != cudaSuccess) return cuda_err(e, "upload");
     DeviceAdjacency da;
-    sls_status st = build_device_adjacency(n, m, J.d_xy[0], d_tri, J.boundary, true, s, da);
+    sls_status st = build_device_adjacency(n, m, J.d_xy[0], d_tri, J.boundary, numbers, s, da);
     if (st == SLS_ERR_NOT_FOUND) {
         // a node in more triangles than the device build handles: host build
         HostMesh hm;
@@ -307,6 +313,8 @@ sls_status build_job(ServerJob &J, bool group, cudaStream_t s, size_t *footprint
         if (e == cudaSuccess) e = pool_alloc((void **)&da.adj, sizeof(uint32_t) * std::max<uint64_t>(1, da.adj_words), s);
         J.d_off = da.node_off;  // freed with the job on any failure below
         J.d_adj = da.adj;
+        if (e == cudaSuccess)  // the device build may have renumbered what was uploaded
+            e = cudaMemcpyAsync(J.d_xy[0], J.xy, cbytes, cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(da.node_off, hm.node_off.data(), sizeof(uint32_t) * (size_t)(n + 1),
                                 cudaMemcpyHostToDevice, s);
@@ -319,25 +327,22 @@ sls_status build_job(ServerJob &J, bool group, cudaStream_t s, size_t *footprint
     }
     J.d_off = da.node_off;
     J.d_adj = da.adj;
+    J.d_perm = da.perm;
     J.diag = da.diag;
+    pool_free(da.inv, s);
     e = cudaFreeAsync(d_tri, s);
     d_tri = nullptr;
     if (e != cudaSuccess) return cuda_err(e, "build");
-    if (group) {
-        // Form A's grouped numbering (as for a single mesh): the coordinates
-        // move to the new ids; the result goes back at retirement
-        st = group_adjacency(n, &J.d_off, J.d_adj, true, s, &J.d_perm, nullptr);
-        if (st != SLS_OK) return cleanup(st);
-        e = launch_permute_coords(J.d_xy[0], J.d_xy[1], 0, false, n, J.d_perm, device_sm_count() * 4, s);
-        std::swap(J.d_xy[0], J.d_xy[1]);
-    }
+    st = build_windows(n, {}, J.d_off, J.d_adj, group, s, J.windows);
+    if (st != SLS_OK) return cleanup(st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(J.d_xy[1], J.d_xy[0], cbytes, cudaMemcpyDeviceToDevice, s);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(J.d_stats, 0, sizeof(PassStats) * (size_t)std::max(1, J.max_iter), s);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&J.uploaded, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventRecord(J.uploaded, s);
     if (e != cudaSuccess) return cuda_err(e, "build");
-    *footprint = built_footprint(n, da.adj_words, J.max_iter);
+    *footprint = built_footprint(n, da.adj_words,
+                                 J.windows.rows_bytes + 32 * (size_t)J.windows.count, J.max_iter);
     return SLS_OK;
 }
 
@@ -356,7 +361,7 @@ void builder_loop(sls_server *S, cudaStream_t s)
         }
         size_t fp = 0;
         J->build_stream = s;
-        const sls_status st = build_job(*J, groups_nodes(S->opt, J->n), s, &fp);
+        const sls_status st = build_job(*J, groups_lanes(S->opt), numbers_spatially(S->opt), s, &fp);
         const std::string err = st == SLS_OK ? std::string() : std::string(sls_last_error());
         if (st != SLS_OK) cudaStreamSynchronize(s);  // a failed build may leave an upload in flight
         J->release_inputs();  // once its uploads are done; outside the lock
@@ -426,6 +431,7 @@ bool rebuild_table(sls_server *S, int slot)
     JobDesc *hj = S->h_jobs[slot];
     int64_t *ht = S->h_toff[slot];
     int64_t t = 0;
+    S->shape = WindowShape{};
     for (size_t j = 0; j < na; ++j) {
         ServerJob &J = *S->active[j];
         JobDesc &D = hj[j];
@@ -442,14 +448,19 @@ bool rebuild_table(sls_server *S, int slot)
         D.max_iter = J.max_iter;
         D.base_round = J.base_round;
         D.cur0 = 0;
-        D.pad = 0;
+        D.windows = (int32_t)J.windows.count;
+        D.bits = J.windows.shape.bits;
+        D.win_hdr = J.windows.hdr;
+        D.win_rows = J.windows.rows;
         D.accept = nullptr;
+        S->shape.cover(J.windows.shape);
         ht[j] = t;
-        t += (J.n + 31) / 32;
+        t += J.windows.count;
     }
     ht[na] = t;
     if (!grow_dev(S->d_tasks, S->tasks_cap, (size_t)std::max<int64_t>(1, t))) return false;
     S->ntasks = t;
+    S->grid = device_sm_count() * batch_pass_occupancy(S->opt.layout, S->block, S->shape);
     return cudaMemcpyAsync(S->d_jobs, hj, sizeof(JobDesc) * na, cudaMemcpyHostToDevice, S->stream) == cudaSuccess &&
            cudaMemcpyAsync(S->d_toff, ht, sizeof(int64_t) * (na + 1), cudaMemcpyHostToDevice, S->stream) ==
                cudaSuccess &&
@@ -658,7 +669,7 @@ void scheduler_loop(sls_server *S)
             cudaError_t e = cudaEventRecord(S->ev_start[slot], S->stream);
             if (e == cudaSuccess)
                 e = launch_batch_pass(S->d_jobs, S->d_tasks, S->ntasks, S->round, S->opt.layout, S->block, S->grid,
-                                      S->stream, kServerChunk, nullptr);
+                                      S->shape, S->stream, kServerChunk, nullptr);
             // every job's record of this round, gathered by one kernel, read back by one copy
             if (e == cudaSuccess) e = launch_gather_round(S->d_jobs, (int)na, S->round, S->d_round[slot], S->stream);
             if (e == cudaSuccess)
@@ -790,7 +801,7 @@ sls_status sls_server_create(size_t hbm_budget, int32_t max_queue, const sls_opt
         return fail(SLS_ERR_CUDA, "stream or event creation failed");
     }
     S->block = (opt != nullptr && opt->block_size >= 32 && opt->block_size <= 128) ? opt->block_size : 128;
-    S->grid = device_sm_count() * batch_pass_occupancy(o.layout, S->block);
+    S->grid = device_sm_count() * batch_pass_occupancy(o.layout, S->block, WindowShape{});
     sls_server *raw = S.release();
     raw->builders_live = nb;
     for (int b = 0; b < nb; ++b) raw->builders.emplace_back(builder_loop, raw, raw->build_streams[b]);
