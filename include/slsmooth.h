@@ -230,7 +230,8 @@ sls_status sls_mesh_destroy(sls_mesh *mesh);
  * in the pool for later handles, so creating a mesh of a size seen before
  * maps no new memory.  sls_trim_memory waits for the current device and then
  * hands the pool's unused memory back to the driver, keeping at most
- * keep_bytes.  Not a counterpart of anything in the paper: a memory policy of
+ * keep_bytes.  (Destroyed handles' streams and page-locked records, at most 16
+ * of each, are kept for later handles too; it frees them as well.)  Not a counterpart of anything in the paper: a memory policy of
  * this library. */
 sls_status sls_trim_memory(size_t keep_bytes);
 

@@ -24,6 +24,16 @@ struct WindowStream {
     void release(cudaStream_t s);
 };
 
+// What a mesh handle needs besides device memory and is slow to make: a
+// non-blocking stream and kHostStats page-locked records (take_kit).
+constexpr int kHostStats = 512;
+struct HandleKit {
+    cudaStream_t stream = nullptr;
+    PassStats *host = nullptr;
+    int device = -1;
+    unsigned long long ctx = 0;
+};
+
 }  // namespace sls
 
 struct sls_mesh {
@@ -31,8 +41,8 @@ struct sls_mesh {
     int64_t n = 0, m = 0, n_free = 0;
     double diag = 0.0;            // bounding-box diagonal of the creation coordinates
     int device = 0;
-    cudaStream_t stream = nullptr;
-    bool own_stream = false;
+    cudaStream_t stream = nullptr;  // the caller's or the kit's
+    sls::HandleKit kit;
     double *xy[2] = {nullptr, nullptr};  // the two coordinate arrays (2n doubles each, 2n floats when f32)
     bool f32 = false;             // binary32 coordinates and arithmetic
     int cur = 0;                  // which of the two holds the current coordinates
@@ -49,7 +59,7 @@ struct sls_mesh {
     sls::PassStats *stats = nullptr;  // one record per pass of a call; the record before the first
                                       // holds the blocks' barrier of the resident form
     int stats_cap = 0;
-    sls::PassStats *h_stats = nullptr;  // pinned, one record
+    sls::PassStats *h_stats = nullptr;  // page-locked, kHostStats records
     uint8_t *accept = nullptr;    // n, when record_accept
     uint2 *halo = nullptr;        // skip_unchanged: kHaloEntries (tile, mask) pairs per 32-node tile
     uint32_t *chg[2] = {nullptr, nullptr};  // per tile: nodes changed by the last two passes
@@ -112,6 +122,11 @@ inline bool numbers_spatially(const sls_options &o)
 // later handles (sls_trim_memory returns it).  Allocate and free on the
 // stream that uses the buffer; pool_free ignores NULL.
 cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t s);
+// A handle's stream and page-locked records, from a small cache on the current
+// device (memory.cu); give back a kit whose stream is idle (keep = false: not
+// for reuse).  sls_trim_memory empties the current device's cache.
+cudaError_t take_kit(HandleKit *kit);
+void give_kit(const HandleKit &kit, bool keep);
 void pool_free(void *p, cudaStream_t s);
 // The window stream of a built adjacency (window_build.cu); segments: the id
 // ranges to cover one after another (Form B: the colour classes' bounds),

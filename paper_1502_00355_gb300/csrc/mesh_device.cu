@@ -57,15 +57,11 @@ static sls_status mesh_setup(sls_mesh *M, const sls_options &o)
 {
     M->opt = o;
     SLS_CUDA_TRY(cudaGetDevice(&M->device), "cudaGetDevice");
-    if (o.stream) {
-        M->stream = (cudaStream_t)o.stream;
-    } else {
-        SLS_CUDA_TRY(cudaStreamCreateWithFlags(&M->stream, cudaStreamNonBlocking), "cudaStreamCreate");
-        M->own_stream = true;
-    }
+    SLS_CUDA_TRY(take_kit(&M->kit), "stream");
+    M->stream = o.stream ? (cudaStream_t)o.stream : M->kit.stream;
+    M->h_stats = M->kit.host;
     sls_status st;
     if ((st = alloc_stats(M, 256)) != SLS_OK) return st;
-    SLS_CUDA_TRY(cudaMallocHost((void **)&M->h_stats, sizeof(PassStats)), "cudaMallocHost");
     if (o.record_accept) {
         if ((st = dev_alloc(M, (void **)&M->accept, (size_t)M->n, "accept mask")) != SLS_OK) return st;
         SLS_CUDA_TRY(cudaMemsetAsync(M->accept, 0, (size_t)M->n, M->stream), "cudaMemset");
@@ -252,8 +248,10 @@ void mesh_release(sls_mesh *M)
     pool_free(M->chg[1], M->stream);
     pool_free(M->accm, M->stream);
     pool_free(M->xfer_bad, M->stream);
-    if (M->h_stats) cudaFreeHost(M->h_stats);
-    if (M->own_stream && M->stream) cudaStreamDestroy(M->stream);
+    // (the frees above are queued on the stream; whoever takes it next queues
+    // after them)
+    give_kit(M->kit, !M->opt.l2_window);  // (a window may still be set on the stream)
+    M->kit = HandleKit{};
     M->stream = nullptr;
 }
 
@@ -390,12 +388,16 @@ sls_status mesh_run(sls_mesh *M, int32_t max_iter, double tol_rel, sls_info &inf
         SLS_CUDA_TRY(cudaStreamSynchronize(M->stream), "pass");
         if (cudaCtxResetPersistingL2Cache() != cudaSuccess) cudaGetLastError();
     }
-    std::vector<PassStats> all((size_t)launched + 1);
-    SLS_CUDA_TRY(cudaMemcpyAsync(all.data(), M->stats - 1, sizeof(PassStats) * all.size(),
-                                 cudaMemcpyDeviceToHost, M->stream), "read pass statistics");
+    // the records of the call, with the one in front of them: into page-locked
+    // memory where they fit
+    const size_t nrec = (size_t)launched + 1;
+    std::vector<PassStats> big(nrec > (size_t)kHostStats ? nrec : 0);
+    PassStats *all = big.empty() ? M->h_stats : big.data();
+    SLS_CUDA_TRY(cudaMemcpyAsync(all, M->stats - 1, sizeof(PassStats) * nrec, cudaMemcpyDeviceToHost, M->stream),
+                 "read pass statistics");
     SLS_CUDA_TRY(cudaStreamSynchronize(M->stream), "passes");
-    const PassStats *hs = all.data() + 1;
-    if (reinterpret_cast<const unsigned *>(all.data())[1])
+    const PassStats *hs = all + 1;
+    if (reinterpret_cast<const unsigned *>(all)[1])
         return fail(SLS_ERR_TIMEOUT, "a wait between the blocks of a launch ran out");
     int it = 0;
     long long fb = 0, sk = 0;
