@@ -42,7 +42,7 @@ CSRC = os.path.join(ROOT, "paper_1502_00355_gb300", "csrc")
 # figures no longer describe the kernel and the bench line reports null.
 PROFILE_FIGURES = {
     "pass_screened": {
-        "files": ["pass_screened.cu", "screen.cuh", "window.cuh", "window_build.cu", "node_exact.cuh",
+        "files": ["pass_screened.cu", "screen.cuh", "window.cuh", "window_pipe.cuh", "window_build.cu", "node_exact.cuh",
                   "div_small.cuh", "device.cuh"],
         "sha256": "db9df0c964a12160525e9538431b1f0be20dcc278b1dfac8ff092a618a9895ef",
         "dram_bytes_per_node": (309215744 + 54800128) / (2048 * 2048),
@@ -50,7 +50,7 @@ PROFILE_FIGURES = {
         "source": "profiles/pass_screened_grid2048.md (2048x2048 capture, per node)",
     },
     "batch_pass": {
-        "files": ["pass_screened.cu", "screen.cuh", "window.cuh", "window_build.cu", "node_exact.cuh",
+        "files": ["pass_screened.cu", "screen.cuh", "window.cuh", "window_pipe.cuh", "window_build.cu", "node_exact.cuh",
                   "div_small.cuh", "device.cuh", "batch.cu"],
         "sha256": "716f3492b8a2cc0ea034315c6b2a5adf884f3866f6fbc7a78722a5074c3f14d3",
         "dram_per_alg_byte": (1008215808 + 171628032) / 994046024,

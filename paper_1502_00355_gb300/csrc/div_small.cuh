@@ -68,13 +68,11 @@ SLS_DS_HD double div_rn(double a, double b)
 #endif
 }
 
-// RN(s / N) for an integer 2 <= N <= 16, given y = RN(1/N) and fN = N as a
-// double.  Returns the quotient's bit pattern.
-SLS_DS_HD uint64_t div_small_bits(uint64_t sb, uint32_t N, double y, double fN)
+// The bit pattern of RN(s / N) for an integer 2 <= N <= 16, given
+// y = RN(1/N), where ok; elsewhere the division has to be done.
+SLS_DS_HD uint64_t div_small_fast(uint64_t sb, uint32_t N, double y, bool &ok)
 {
     const uint32_t es = (uint32_t)(sb >> 52) & 0x7ffu;
-    // normal s well inside the range: q0 and the quotient are normal too
-    if (es - 63u > 1937u) return bits_of(div_rn(of_bits(sb), fN));
     const uint64_t qb = bits_of(mul_rn(of_bits(sb), y));
     const uint32_t eq = (uint32_t)(qb >> 52) & 0x7ffu;
     // s/N < s, so eq <= es; s/N >= s/16, so es - eq <= 5.  The remainder is
@@ -88,10 +86,18 @@ SLS_DS_HD uint64_t div_small_bits(uint64_t sb, uint32_t N, double y, double fN)
     const int32_t a2 = r < 0 ? -2 * r : 2 * r;
     const int32_t k = (a2 > n ? 1 : 0) + (a2 > 3 * n ? 1 : 0);
     const uint64_t qk = qb + (uint64_t)(int64_t)(r < 0 ? -k : k);
-    // a step out of the binade (also onto its top, which is rare) is left to
-    // the division
-    if (((uint32_t)((qk ^ qb) >> 32) & 0xfff00000u) != 0u || a2 > 5 * n) return bits_of(div_rn(of_bits(sb), fN));
+    // normal s well inside the range (q0 and the quotient are normal too), and
+    // no step out of the binade (also onto its top, which is rare)
+    ok = (es - 63u <= 1937u) & (((uint32_t)((qk ^ qb) >> 32) & 0xfff00000u) == 0u) & (a2 <= 5 * n);
     return qk;
+}
+
+// The same with the division done where it has to be; fN = N as a double.
+SLS_DS_HD uint64_t div_small_bits(uint64_t sb, uint32_t N, double y, double fN)
+{
+    bool ok;
+    const uint64_t q = div_small_fast(sb, N, y, ok);
+    return ok ? q : bits_of(div_rn(of_bits(sb), fN));
 }
 
 }  // namespace divs

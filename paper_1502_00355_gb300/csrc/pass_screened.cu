@@ -34,14 +34,14 @@
 // unless they take part in FP64 arithmetic: the compiler copies FP64
 // registers with FP64-pipe instructions.
 //
-// What bounds it: instruction issue (64% of slots), the FP64 pipe (54%) and
+// What bounds it: instruction issue (65% of slots), the FP64 pipe (58%) and
 // the latency of shared-memory loads together; HBM stands at about a sixth of
 // the measured copy rate.  Gathering and splitting a coordinate once per
 // window (1.4 times a node) instead of once per neighbour visit (6.5 times)
-// took 1,653 warp instructions per 32 nodes to 1,230 and 23.5 FP64
+// took 1,653 warp instructions per 32 nodes to 1,140 and 23.5 FP64
 // instructions to 13.7.  Measured, to the tolerance, against one thread per
-// node gathering for itself: 2048^2 jittered grid 293.7 -> 217 us a pass,
-// 1024^2 96.9 -> 64.5, 4096^2 942 -> 713.
+// node gathering for itself: 2048^2 jittered grid 293.7 -> 200.8 us a pass,
+// 1024^2 96.9 -> 59.2, 4096^2 942 -> 660.
 #include <atomic>
 #include <cfloat>
 #include <mutex>
@@ -51,7 +51,7 @@
 #include "kernels.h"
 #include "node_exact.cuh"
 #include "screen.cuh"
-#include "window.cuh"
+#include "window_pipe.cuh"
 
 namespace sls {
 
@@ -77,7 +77,7 @@ constexpr uint32_t kNoItem = 0xffffffffu;
 
 struct __align__(16) Queue {
     ulonglong2 p[kPending], c[kPending];                    // the node, its centre
-    double px[kItems], py[kItems], qx[kItems], qy[kItems];  // the step's two vertices, in ring order; then px: the quality
+    double px[kItems], py[kItems], qx[kItems], qy[kItems];  // the step's vertices in ring order; then px: quality
     uint32_t item[kItems];      // pending node | side << 8 (1: after the move) | step << 9
     int32_t node[kPending];     // -1: no entry
     uint32_t range[kPending];   // first item | items << 8 | lane << 16
@@ -86,14 +86,6 @@ struct __align__(16) Queue {
     unsigned int nacc, nexact;  // accepted and exactly decided nodes (flush)
     unsigned long long best;    // bits of the block's largest squared move
     float best_low;             // at most that (-1: none yet)
-};
-
-// A block keeps two windows in shared memory: the one it works on and the
-// next one, which is copied in meanwhile.  Headers are fetched three windows
-// ahead and halo ids two, because each names what the next copies.
-struct __align__(16) Ahead {
-    uint32_t hdr[4][win::kHeaderWords];  // window i's header in slot i & 3
-    uint8_t idle[4][4];                  // skip_unchanged: its subtiles that need no work
 };
 
 struct Block {
@@ -113,7 +105,6 @@ struct Block {
 // from the second.
 constexpr int kTwoBufferEntries = 320;
 __host__ __device__ inline int buffers_for(const WindowShape &s) { return s.entries <= kTwoBufferEntries ? 2 : 1; }
-__host__ __device__ inline uint32_t ids_words_of(const WindowShape &s) { return ((uint32_t)s.halo + 3u) & ~3u; }
 size_t smem_for(const WindowShape &s)
 {
     return sizeof(Queue) + sizeof(Ahead) + 2 * 4 * (size_t)ids_words_of(s) + 2 * 128 * (size_t)s.hot +
@@ -180,19 +171,6 @@ __device__ __forceinline__ Block block_memory(unsigned char *smem, const WindowS
     return b;
 }
 
-// Asynchronous copies global -> shared (no registers held while they fly).
-__device__ __forceinline__ void copy16(void *dst, const void *src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-__device__ __forceinline__ void copy8(void *dst, const void *src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
 // ---- the FP64 queue ---------------------------------------------------------
 
 // FP64 quality of step t (P -> Q) of a ring with the node at x.  The step runs
@@ -210,7 +188,7 @@ __device__ __forceinline__ double step_quality(ulonglong2 x, unsigned long long 
 
 // Evaluates every waiting item and finishes the nodes they belong to.  All
 // threads of the block call it, with no push in flight.
-template <int LAYOUT>
+template <int LAYOUT, bool HALO>
 __device__ __noinline__ Tally drain(const PassArgs &a, Queue *q, Tally tally)
 {
     const uint32_t ni = q->nitems < (uint32_t)kItems ? q->nitems : (uint32_t)kItems;
@@ -246,7 +224,7 @@ __device__ __noinline__ Tally drain(const PassArgs &a, Queue *q, Tally tally)
                              q_old, q_new, b2, acc, moved);
         note_move(q, b2);
         tally.nacc += acc ? 1u : 0u;
-        if (a.halo) {  // the node's bits in its tile's masks (written with the tile's other nodes)
+        if (HALO) {  // the node's bits in its tile's masks (written with the tile's other nodes)
             const uint32_t bit = 1u << (node & 31);
             if (moved) atomicOr(a.chg_cur + (node >> 5), bit);
             if (acc) atomicOr(a.accm + (node >> 5), bit);
@@ -260,53 +238,9 @@ __device__ __noinline__ Tally drain(const PassArgs &a, Queue *q, Tally tally)
 
 // ---- one subtile --------------------------------------------------------------
 
-// List entries of BITS bits in a lane's words (32 words apart), as byte
-// offsets of staged entries.
-template <int BITS>
-struct List {
-    static constexpr uint32_t kPer = 32 / BITS;
-    static __device__ __forceinline__ uint32_t in_word(uint32_t word, uint32_t j)
-    {
-        return ((word >> (BITS * j)) & ((1u << BITS) - 1u)) << 4;
-    }
-    static __device__ __forceinline__ uint32_t at(const uint32_t *list, uint32_t t)
-    {
-        return in_word(list[32u * (t / kPer)], t % kPer);
-    }
-};
-
 // ---- the ring walk: screen.cuh's ring form, both sides of the move in the
-// halves of packed FP32 pairs (one instruction for two operations, the same
-// roundings).
+// halves of packed FP32 pairs.
 
-__device__ __forceinline__ uint64_t pair(float lo, float hi)
-{
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void halves(uint64_t v, float &lo, float &hi)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
-{
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
-{
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
-{
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
 // The larger of two, NaN when either is.
 __device__ __forceinline__ float max_nan(float a, float b)
 {
@@ -356,37 +290,45 @@ struct Minima {
 };
 
 // ring_values of the step P -> Q (FROM_PLAIN: P is the plain one), packed with
-// its number, into the minima.  Padding steps are NaN and change nothing.
+// its number; NaN for a step that has no triangle.
 template <bool IRREGULAR, bool FROM_PLAIN>
 __device__ __forceinline__ void ring_step(const RingWalk &w, Minima &m, const PairVertex &P, const PairVertex &Q,
-                                          uint32_t t)
+                                          uint32_t t, float &vo, float &vn)
 {
     m.rn = fmaxf(m.rn, fmaxf(fabsf(Q.x), fabsf(Q.y)));
-    if (IRREGULAR && ((w.slots >> (2u * t)) & 3u) == 3u) return;
     const float bx = Q.x - P.x, by = Q.y + P.y;
     const float b2 = fmaf(bx, bx, by * by);
     float so, sn, co, cn;
     halves(add2(add2(P.nn, Q.nn), pair(b2, b2)), so, sn);
     halves(fma2(P.xx, Q.yy, mul2(P.yy, Q.xx)), co, cn);  // the cross product, negated from a plain vertex
-    float vo = (FROM_PLAIN ? -co : co) * rcp_ring(so), vn = (FROM_PLAIN ? -cn : cn) * rcp_ring(sn);
-    if (IRREGULAR && ((w.rev >> t) & 1u)) {
-        vo = -vo;
-        vn = -vn;
+    vo = (FROM_PLAIN ? -co : co) * rcp_ring(so);
+    vn = (FROM_PLAIN ? -cn : cn) * rcp_ring(sn);
+    if (IRREGULAR) {
+        if ((w.rev >> t) & 1u) {
+            vo = -vo;
+            vn = -vn;
+        }
+        if (((w.slots >> (2u * t)) & 3u) == 3u) vo = vn = so = sn = __int_as_float(0x7fffffff);
     }
     vo = with_step(vo, t);
     vn = with_step(vn, t);
-    m.m2o = fminf(m.m2o, max_nan(m.m1o, vo));
-    m.m1o = fminf(m.m1o, vo);
-    m.m2n = fminf(m.m2n, max_nan(m.m1n, vn));
-    m.m1n = fminf(m.m1n, vn);
     m.smin = fminf(m.smin, fminf(so, sn));
+}
+
+// Two values into the smallest two.  Values of padding steps are NaN and
+// change nothing.
+__device__ __forceinline__ void two_least(float &m1, float &m2, float v1, float v2)
+{
+    const float lo = fminf(v1, v2);
+    m2 = fminf(m2, fminf(max_nan(m1, lo), max_nan(v1, v2)));
+    m1 = fminf(m1, lo);
 }
 
 // Walks the rings of a warp's lanes to the subtile's largest step number l,
 // two steps between branches (so that the loads of one overlap the other's
 // arithmetic).
 template <bool IRREGULAR, int BITS>
-__device__ __forceinline__ Minima walk_ring(const RingWalk &w, uint32_t l, const uint32_t *list)
+__device__ __forceinline__ Minima walk_ring(RingWalk w, uint32_t l, const uint32_t *list)
 {
     using L = List<BITS>;
     Minima m;
@@ -405,12 +347,22 @@ __device__ __forceinline__ Minima walk_ring(const RingWalk &w, uint32_t l, const
             const uint32_t e2 = L::in_word(word, (j + 2) % L::kPer);
             const PairVertex B = pair_vertex<true>(w, e1);
             const PairVertex C = pair_vertex<false>(w, e2);
-            ring_step<IRREGULAR, true>(w, m, A, B, t + j);
-            ring_step<IRREGULAR, false>(w, m, B, C, t + j + 1u);
+            float vo1, vn1, vo2, vn2;
+            ring_step<IRREGULAR, true>(w, m, A, B, t + j, vo1, vn1);
+            ring_step<IRREGULAR, false>(w, m, B, C, t + j + 1u, vo2, vn2);
+            two_least(m.m1o, m.m2o, vo1, vo2);
+            two_least(m.m1n, m.m2n, vn1, vn2);
             A = C;
             if (t + j + 2u >= l) return m;
         }
     }
+}
+
+// (kept out of line: it would cost the regular walk registers)
+template <int BITS>
+__device__ __noinline__ Minima walk_irregular(RingWalk w, uint32_t l, const uint32_t *list)
+{
+    return walk_ring<true, BITS>(w, l, list);
 }
 
 // What a lane knows of a node that its screen left open.
@@ -595,9 +547,15 @@ __device__ __forceinline__ bool update_lane(const PassArgs &a, Queue *q, const c
     const ulonglong2 pb = *reinterpret_cast<const ulonglong2 *>(xy + own);
     ulonglong2 cb = pb;
     if (free) {
-        const double fd = c_degree[deg], y = c_recip[deg];
-        cb.x = divs::div_small_bits(dbits(sx), deg, y, fd);
-        cb.y = divs::div_small_bits(dbits(sy), deg, y, fd);
+        const double y = c_recip[deg];
+        bool okx, oky;
+        cb.x = divs::div_small_fast(dbits(sx), deg, y, okx);
+        cb.y = divs::div_small_fast(dbits(sy), deg, y, oky);
+        if (!(okx & oky)) {
+            const double fd = c_degree[deg];
+            cb.x = dbits(__ddiv_rn(sx, fd));
+            cb.y = dbits(__ddiv_rn(sy, fd));
+        }
     }
     bool act = cb.x != pb.x || cb.y != pb.y;
     if (free && !act) {
@@ -608,54 +566,53 @@ __device__ __forceinline__ bool update_lane(const PassArgs &a, Queue *q, const c
         tally.nacc += acc ? 1u : 0u;
         res = acc ? 1u : 0u;
     }
-    if (!__any_sync(0xffffffffu, act)) return false;
-    RingWalk w;
-    w.split = xy + half;
-    {
-        const float4 h = *reinterpret_cast<const float4 *>(xy + half + own);
-        w.phx = h.x;
-        w.plx = h.y;
-        w.phy = h.z;
-        w.ply = h.w;
-    }
-    w.Cx = w.Cy = 0.0f;
-    if (act) offset_of(cb, pb, w.Cx, w.Cy);
-    w.slots = w.rev = 0u;
-    Minima m;
-    if (r.irregular) {
-        const uint32_t *row = a.win_rows + (size_t)r.cold * 32u + (threadIdx.x & 31u);
-        w.slots = __ldg(row);
-        w.rev = __ldg(row + 32);
-        m = walk_ring<true, BITS>(w, r.l, list);
-    } else {
-        m = walk_ring<false, BITS>(w, r.l, list);
-    }
-    // a coordinate of the node or of a neighbour outside the splits' range
-    const bool record = act && !(fmaxf(m.rn, fmaxf(fabsf(w.phx), fabsf(w.phy))) < FLT_MAX);
-    act = act && !record;
-    const float rN = fmaxf(m.rn, fmaxf(fabsf(w.Cx), fabsf(w.Cy)));
-    const float M = fmaxf(fabsf(w.phx), fabsf(w.phy)) * 1.0001f + rN;
-    const float g = side_g(rN, m.smin);
-    const bool bok = frame_ok(m.rn, rN, M) & ring_ok(m.smin, g);
-    Open o;
-    o.b = ring_bound(g);
-    // per side: q (FP64) lies in [amin - b, amin + b]; the minimum is attained
-    // by one triangle alone when every other value lies above amin + b + b
-    const float amin_o = kTwoSqrt3f * m.m1o, amin_n = kTwoSqrt3f * m.m1n;
-    o.up_o = amin_o + o.b;
-    o.up_n = amin_n + o.b;
-    int verdict = 0;
-    if (bok) verdict = amin_n - o.b > o.up_o ? 1 : (o.up_n < amin_o - o.b ? -1 : 0);
-    const uint32_t to = step_of(m.m1o);
-    if (act && verdict == 0 && bok && to == step_of(m.m1n) && kTwoSqrt3f * m.m2o - o.b > o.up_o &&
-        kTwoSqrt3f * m.m2n - o.b > o.up_n) {
-        const RingVertex P = w.vertex(L::at(list, to)), Q = w.vertex(L::at(list, to + 1u));
-        verdict = diff_screen(P.x, P.y, Q.x, Q.y, w.Cx, w.Cy, ((w.rev >> to) & 1u) ? -1.0f : 1.0f, M * M);
-    }
-    const unsigned open = __ballot_sync(0xffffffffu, act && verdict == 0);
-    if (act && verdict != 0) {
-        const bool acc = verdict > 0;
-        if (acc) {
+    bool record = false;
+    if (__any_sync(0xffffffffu, act)) {
+        int verdict = 0;
+        RingWalk w;
+        w.split = xy + half;
+        {
+            const float4 h = *reinterpret_cast<const float4 *>(xy + half + own);
+            w.phx = h.x;
+            w.plx = h.y;
+            w.phy = h.z;
+            w.ply = h.w;
+        }
+        w.Cx = w.Cy = 0.0f;
+        if (act) offset_of(cb, pb, w.Cx, w.Cy);
+        w.slots = w.rev = 0u;
+        Minima m;
+        if (r.irregular) {
+            const uint32_t *row = a.win_rows + (size_t)r.cold * 32u + (threadIdx.x & 31u);
+            w.slots = __ldg(row);
+            w.rev = __ldg(row + 32);
+            m = walk_irregular<BITS>(w, r.l, list);
+        } else {
+            m = walk_ring<false, BITS>(w, r.l, list);
+        }
+        // a coordinate of the node or of a neighbour outside the splits' range
+        record = act && !(fmaxf(m.rn, fmaxf(fabsf(w.phx), fabsf(w.phy))) < FLT_MAX);
+        act = act && !record;
+        const float rN = fmaxf(m.rn, fmaxf(fabsf(w.Cx), fabsf(w.Cy)));
+        const float M = fmaxf(fabsf(w.phx), fabsf(w.phy)) * 1.0001f + rN;
+        const float g = side_g(rN, m.smin);
+        const bool bok = frame_ok(m.rn, rN, M) & ring_ok(m.smin, g);
+        Open o;
+        o.b = ring_bound(g);
+        // per side: q (FP64) lies in [amin - b, amin + b]; the minimum is attained
+        // by one triangle alone when every other value lies above amin + b + b
+        const float amin_o = kTwoSqrt3f * m.m1o, amin_n = kTwoSqrt3f * m.m1n;
+        o.up_o = amin_o + o.b;
+        o.up_n = amin_n + o.b;
+        if (act && bok) verdict = amin_n - o.b > o.up_o ? 1 : (o.up_n < amin_o - o.b ? -1 : 0);
+        const uint32_t to = step_of(m.m1o);
+        if (act && verdict == 0 && bok && to == step_of(m.m1n) && kTwoSqrt3f * m.m2o - o.b > o.up_o &&
+            kTwoSqrt3f * m.m2n - o.b > o.up_n) {
+            const RingVertex P = w.vertex(L::at(list, to)), Q = w.vertex(L::at(list, to + 1u));
+            verdict = diff_screen(P.x, P.y, Q.x, Q.y, w.Cx, w.Cy, ((w.rev >> to) & 1u) ? -1.0f : 1.0f, M * M);
+        }
+        const unsigned open = __ballot_sync(0xffffffffu, act && verdict == 0);
+        if (act && verdict > 0) {
             // the exact squared move is needed only where it can be the block's
             // largest: the screen's offset gives it to within a few units of 2^-24
             const float about = fmaf(w.Cx, w.Cx, w.Cy * w.Cy) * 1.000001f + 1e-37f;
@@ -666,26 +623,28 @@ __device__ __forceinline__ bool update_lane(const PassArgs &a, Queue *q, const c
             }
             tally.nacc += 1u;
             res = 3u;  // the centre differs from the node (equal centres are done above)
-        } else {
-            cb = *reinterpret_cast<const ulonglong2 *>(xy + own);
         }
-        CoordBits<LAYOUT>::put(a.out, a.n, node, cb);
-        if (a.accept) a.accept[node] = acc ? 1 : 0;
-    }
-    if (open) {
-        if (act && verdict == 0) tally.nexact += 1u;
-        if (!bok) {  // every step is a candidate
-            o.b = 0.0f;
-            o.up_o = o.up_n = __int_as_float(0x7f800000);
+        if (verdict != 0) {
+            if (verdict < 0) cb = *reinterpret_cast<const ulonglong2 *>(xy + own);
+            CoordBits<LAYOUT>::put(a.out, a.n, node, cb);
+            if (a.accept) a.accept[node] = verdict > 0 ? 1 : 0;
         }
-        o.Cx = w.Cx;
-        o.Cy = w.Cy;
-        o.own = own;
-        o.steps = steps;
-        const uint32_t done = settle_open<LAYOUT, BITS>(a, q, xy, half, list, r.cold, r.irregular, node, cb, o, open);
-        full = full || (done & 8u);
-        if (done & 3u) res = done & 3u;
-        tally.nacc += done & 1u;
+        if (open) {
+            if (act && verdict == 0) tally.nexact += 1u;
+            if (!bok) {  // every step is a candidate
+                o.b = 0.0f;
+                o.up_o = o.up_n = __int_as_float(0x7f800000);
+            }
+            o.Cx = w.Cx;
+            o.Cy = w.Cy;
+            o.own = own;
+            o.steps = steps;
+            const uint32_t done =
+                settle_open<LAYOUT, BITS>(a, q, xy, half, list, r.cold, r.irregular, node, cb, o, open);
+            full = full || (done & 8u);
+            if (done & 3u) res = done & 3u;
+            tally.nacc += done & 1u;
+        }
     }
     return record;
 }
@@ -693,7 +652,7 @@ __device__ __forceinline__ bool update_lane(const PassArgs &a, Queue *q, const c
 // ---- a block's windows ----------------------------------------------------------
 
 // Nodes of a subtile that their records decide, a warp each.
-template <int LAYOUT, bool COHERENT>
+template <int LAYOUT, bool COHERENT, bool HALO>
 __device__ __noinline__ Tally by_record(const PassArgs &a, Queue *q, int32_t node, unsigned left, Tally tally)
 {
     while (left) {
@@ -707,7 +666,7 @@ __device__ __noinline__ Tally by_record(const PassArgs &a, Queue *q, int32_t nod
             note_move(q, b2);
             tally.nacc += acc ? 1u : 0u;
             tally.nexact += 1u;
-            if (a.halo) {
+            if (HALO) {
                 const uint32_t bit = 1u << (nd & 31);
                 if (moved) atomicOr(a.chg_cur + (nd >> 5), bit);
                 if (acc) atomicOr(a.accm + (nd >> 5), bit);
@@ -732,7 +691,7 @@ __device__ __forceinline__ void split_staged(char *xy, uint32_t half, uint32_t s
 
 // Updates the nodes of subtile `sub` of a staged window (h: its header, rows:
 // its hot rows in shared memory).
-template <int LAYOUT, int BITS, bool COHERENT>
+template <int LAYOUT, int BITS, bool COHERENT, bool HALO>
 __device__ __forceinline__ void work_subtile(const PassArgs &a, Queue *q, const char *xy, uint32_t half,
                                              const uint32_t *h, const uint32_t *rows, int sub, Tally &tally,
                                              bool &full)
@@ -752,7 +711,7 @@ __device__ __forceinline__ void work_subtile(const PassArgs &a, Queue *q, const 
     bool record = have && (r.meta & win::kBig);
     if (r.d > 0u) record |= update_lane<LAYOUT, BITS>(a, q, xy, half, r, node, tally, res, full);
     __syncwarp();
-    if (a.halo) {  // before any other write to the tile's masks
+    if (HALO) {  // before any other write to the tile's masks
         const int64_t wt = (int64_t)(h[1] >> 5) + sub;
         const unsigned cb = __ballot_sync(0xffffffffu, (res & 2u) != 0u);
         const unsigned ab = __ballot_sync(0xffffffffu, (res & 1u) != 0u);
@@ -762,7 +721,7 @@ __device__ __forceinline__ void work_subtile(const PassArgs &a, Queue *q, const 
         }
     }
     const unsigned left = __ballot_sync(0xffffffffu, record);
-    if (left) tally = by_record<LAYOUT, COHERENT>(a, q, node, left, tally);
+    if (left) tally = by_record<LAYOUT, COHERENT, HALO>(a, q, node, left, tally);
 }
 
 // Works windows w0, w0 + stride, ... (n of them).  Every thread of the block
@@ -773,7 +732,7 @@ __device__ __forceinline__ void work_subtile(const PassArgs &a, Queue *q, const 
 // per window says that it is there and that window i - 1, whose buffer the
 // next copies overwrite, is finished.  (With one buffer of staged entries the
 // copies wait for that barrier, and a second one says that they are there.)
-template <int LAYOUT, int BITS>
+template <int LAYOUT, int BITS, bool HALO>
 __device__ __forceinline__ void run_windows(const PassArgs &a, const Block &blk, int64_t w0, int n, int64_t stride,
                                             Tally &tally, unsigned &nskip, bool &full)
 {
@@ -791,7 +750,9 @@ __device__ __forceinline__ void run_windows(const PassArgs &a, const Block &blk,
         uint32_t *dst = blk.ids + (i & 1) * blk.ids_words;
         for (uint32_t k = 4 * tid; k < win::hdr_halo(h[2]); k += 4 * nthr) copy16(dst + k, src + k);
     };
-    auto all_idle = [&](int i) { return a.skip && *reinterpret_cast<const uint32_t *>(ah->idle[i & 3]) == 0x01010101u; };
+    auto all_idle = [&](int i) {
+        return HALO && a.skip && *reinterpret_cast<const uint32_t *>(ah->idle[i & 3]) == 0x01010101u;
+    };
     auto fetch_data = [&](int i) {
         if (i >= n || all_idle(i)) return;
         const uint32_t *h = ah->hdr[i & 3];
@@ -815,7 +776,7 @@ __device__ __forceinline__ void run_windows(const PassArgs &a, const Block &blk,
     // inputs; such a tile's results are those of the previous pass, which
     // `out` and the masks already hold
     auto check_idle = [&](int i) {
-        if (!a.skip || i >= n) return;
+        if (!HALO || !a.skip || i >= n) return;
         const uint32_t *h = ah->hdr[i & 3];
         for (int sub = warp; sub < 4; sub += nwarps) {
             const int64_t wt = (int64_t)(h[1] >> 5) + sub;
@@ -863,7 +824,7 @@ __device__ __forceinline__ void run_windows(const PassArgs &a, const Block &blk,
             split_staged(xy, blk.half, win::hdr_count(h[2]) + win::hdr_halo(h[2]), tid, nthr);
         }
         if (__syncthreads_or(full)) {
-            tally = drain<LAYOUT>(a, blk.q, tally);
+            tally = drain<LAYOUT, HALO>(a, blk.q, tally);
             full = false;
         }
         if (blk.stage) fetch_data(i + 1);
@@ -872,19 +833,21 @@ __device__ __forceinline__ void run_windows(const PassArgs &a, const Block &blk,
         check_idle(i + 2);
         if (rest) continue;
         for (int sub = warp; sub < 4; sub += nwarps) {
-            if (a.skip && ah->idle[i & 3][sub]) continue;
-            work_subtile<LAYOUT, BITS, false>(a, blk.q, xy, blk.half, h, blk.rows + (i & 1) * blk.rows_words, sub, tally,
-                                              full);
+            if (HALO && a.skip && ah->idle[i & 3][sub]) continue;
+            work_subtile<LAYOUT, BITS, false, HALO>(a, blk.q, xy, blk.half, h, blk.rows + (i & 1) * blk.rows_words,
+                                                    sub, tally, full);
         }
     }
 }
 
 // The kernels are compiled for 7 blocks of 128 threads per SM (72 registers):
-// 2048^2 runs 228 us a pass with 7, 233 with 6 and 239 with 8, whose 64
+// 2048^2 runs 201 us a pass with 7, 207 with 6 and 218 with 8, whose 64
 // registers spill.
 constexpr int kBlocksPerSm = 7;
 
-template <int LAYOUT, int BITS>
+// HALO: the mesh keeps the masks of skip_unchanged (apart: their code costs
+// other meshes registers, 217 against 202 us a pass on 2048^2).
+template <int LAYOUT, int BITS, bool HALO>
 __global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
     pass_screened_kernel(const __grid_constant__ PassArgs a, const __grid_constant__ WindowShape shape)
 {
@@ -896,11 +859,11 @@ __global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
     unsigned nskip = 0u;  // node updates this warp left as they were (lane 0)
     bool full = false;
     if ((int64_t)blockIdx.x < a.win_count)
-        run_windows<LAYOUT, BITS>(a, blk, a.win_first + blockIdx.x,
+        run_windows<LAYOUT, BITS, HALO>(a, blk, a.win_first + blockIdx.x,
                                   (int)((a.win_count - blockIdx.x + gridDim.x - 1) / gridDim.x), gridDim.x, tally,
                                   nskip, full);
     __syncthreads();
-    if (blk.q->npending) tally = drain<LAYOUT>(a, blk.q, tally);
+    if (blk.q->npending) tally = drain<LAYOUT, HALO>(a, blk.q, tally);
     if (nskip) atomicAdd(&a.stats[a.q].nodes_skipped, nskip);
     flush(blk.q, a.stats + a.q, tally);
 }
@@ -996,9 +959,9 @@ __global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
         Tally tally{0u, 0u};
         bool full = false;  // (one window: the queue is worked off after it)
         for (int sub = warp; sub < 4; sub += nwarps)
-            work_subtile<LAYOUT, BITS, true>(a, blk.q, blk.xy, blk.half, h, blk.rows, sub, tally, full);
+            work_subtile<LAYOUT, BITS, true, false>(a, blk.q, blk.xy, blk.half, h, blk.rows, sub, tally, full);
         __syncthreads();
-        if (blk.q->npending) tally = drain<LAYOUT>(a, blk.q, tally);
+        if (blk.q->npending) tally = drain<LAYOUT, false>(a, blk.q, tally);
         flush(blk.q, a.stats + a.q, tally);
         if (done == passes) return;
         in = (done & 1) ? a0.out : a0.in;
@@ -1057,7 +1020,7 @@ __global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
         if (job != cur_job) {
             __syncthreads();
             if (cur_job >= 0 && active) {
-                if (blk.q->npending) tally = drain<LAYOUT>(s_args, blk.q, tally);
+                if (blk.q->npending) tally = drain<LAYOUT, false>(s_args, blk.q, tally);
                 flush(blk.q, s_args.stats + s_args.q, tally);
                 __syncthreads();
             }
@@ -1100,17 +1063,19 @@ __global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
         if (!active) continue;
         if (window == 0 && threadIdx.x == 0) s_args.stats[s_args.q].executed = 1u;
         if (WIDE && s_wide)
-            run_windows<LAYOUT, 16>(s_args, blk, window, (int)run, 1, tally, nskip, full);
+            run_windows<LAYOUT, 16, false>(s_args, blk, window, (int)run, 1, tally, nskip, full);
         else
-            run_windows<LAYOUT, 8>(s_args, blk, window, (int)run, 1, tally, nskip, full);
+            run_windows<LAYOUT, 8, false>(s_args, blk, window, (int)run, 1, tally, nskip, full);
     }
 }
 
+template <bool HALO>
 const void *kernel_of(int layout, int bits)
 {
     if (layout == 0)
-        return bits == 8 ? (const void *)pass_screened_kernel<0, 8> : (const void *)pass_screened_kernel<0, 16>;
-    return bits == 8 ? (const void *)pass_screened_kernel<1, 8> : (const void *)pass_screened_kernel<1, 16>;
+        return bits == 8 ? (const void *)pass_screened_kernel<0, 8, HALO>
+                         : (const void *)pass_screened_kernel<0, 16, HALO>;
+    return bits == 8 ? (const void *)pass_screened_kernel<1, 8, HALO> : (const void *)pass_screened_kernel<1, 16, HALO>;
 }
 
 const void *resident_kernel_of(int layout, int bits)
@@ -1155,14 +1120,13 @@ cudaError_t ensure_constants()
     e = cudaMemcpyToSymbol(c_recip, r, sizeof r);
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_degree, dg, sizeof dg);
     if (e != cudaSuccess) return e;
-    const void *fns[12] = {kernel_of(0, 8),       kernel_of(0, 16),      kernel_of(1, 8),
-                          kernel_of(1, 16),      batch_kernel_of(0, 8), batch_kernel_of(0, 16),
-                          batch_kernel_of(1, 8), batch_kernel_of(1, 16), resident_kernel_of(0, 8),
-                          resident_kernel_of(0, 16), resident_kernel_of(1, 8), resident_kernel_of(1, 16)};
-    for (const void *f : fns) {
-        e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        if (e != cudaSuccess) return e;
-    }
+    const int forms[4][2] = {{0, 8}, {0, 16}, {1, 8}, {1, 16}};
+    for (const auto &f : forms)
+        for (const void *k : {kernel_of<false>(f[0], f[1]), kernel_of<true>(f[0], f[1]), batch_kernel_of(f[0], f[1]),
+                              resident_kernel_of(f[0], f[1])}) {
+            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+            if (e != cudaSuccess) return e;
+        }
     g_consts_ctx[dev].store(key, std::memory_order_release);
     return cudaSuccess;
 }
@@ -1184,7 +1148,8 @@ cudaError_t launch_pass_screened(const PassArgs &a, int layout, int block, int g
     if (e != cudaSuccess) return e;
     if (a.win_count < grid) grid = a.win_count > 0 ? (int)a.win_count : 1;
     void *args[] = {const_cast<PassArgs *>(&a), const_cast<WindowShape *>(&shape)};
-    return cudaLaunchKernel(kernel_of(layout, shape.bits), dim3(grid), dim3(block), args, smem_for(shape), s);
+    return cudaLaunchKernel(a.halo ? kernel_of<true>(layout, shape.bits) : kernel_of<false>(layout, shape.bits),
+                            dim3(grid), dim3(block), args, smem_for(shape), s);
 }
 
 bool resident_fits(const PassArgs &a, int layout, int block, const WindowShape &shape)
@@ -1265,7 +1230,7 @@ int batch_pass_occupancy(int layout, int block, const WindowShape &shape)
 
 int pass_screened_occupancy(int layout, int block, const WindowShape &shape)
 {
-    return occupancy(kernel_of(layout, shape.bits), block, shape);
+    return occupancy(kernel_of<false>(layout, shape.bits), block, shape);
 }
 
 }  // namespace sls

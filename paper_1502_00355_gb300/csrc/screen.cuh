@@ -179,8 +179,8 @@ SLS_SC_HD float side_bound(float amax, float g) { return fmaf(kC1, amax, fmaf(kC
 // the move (no cancellation between two nearly equal qualities).  Error
 // budget (e = 2^-24; A, B within 3 e R, C within 2 e |C|; R >= every local
 // coordinate of the triangle and the centre, r >= |C| components): dcr
-// 32 e r R, ds 100 e r R, cr_old 16 e R^2, s_old 170 e R^2, s_new 280 e R^2,
-// and the roundings of N.  kE64 bounds |FP64 alpha - exact alpha| (about 14.2
+// 32 e r R, ds 100 e r R, cr_old 16 e R^2, s_old 170 e R^2, s_new = s_old + ds
+// 300 e R^2 (r <= R), and the roundings of N.  kE64 bounds |FP64 alpha - exact alpha| (about 14.2
 // units of 2^-53 for |alpha| <= 1, second-order terms included with margin).
 // Returns +1 when q_new > q_old certainly, -1 when q_new < q_old certainly,
 // 0 otherwise.
@@ -197,22 +197,21 @@ SLS_SC_HD int diff_screen(float Ax, float Ay, float Bx, float By, float Cx, floa
     const float ba2 = fmaf(bax, bax, bay * bay);
     const float cro = fmaf(Ax, By, -(Ay * Bx));
     const float so = fmaf(Ax, Ax, fmaf(Ay, Ay, fmaf(Bx, Bx, fmaf(By, By, ba2))));
-    const float ax = Ax - Cx, ay = Ay - Cy, bx = Bx - Cx, by = By - Cy;
-    const float sn = fmaf(ax, ax, fmaf(ay, ay, fmaf(bx, bx, fmaf(by, by, ba2))));
-    const float dabx = Ax - Bx, daby = Ay - By;
-    const float dcr = fmaf(Cx, daby, -(Cy * dabx));
-    const float sabx = Ax + Bx, saby = Ay + By;
-    const float t = fmaf(Cx, sabx, Cy * saby);
-    const float c2 = fmaf(Cx, Cx, Cy * Cy);
-    const float ds = 2.0f * (c2 - t);
+    const float dcr = fmaf(Cy, bax, -(Cx * bay));
+    const float t = fmaf(Cx, Ax + Bx, Cy * (Ay + By));
+    const float ds = 2.0f * (fmaf(Cx, Cx, Cy * Cy) - t);
+    const float sn = so + ds;
     const float N = fmaf(dcr, so, -(cro * ds));
     const float rR = r * R, R2 = R * R;
-    const float e_dcr = 32.0f * kEps * rR, e_ds = 100.0f * kEps * rR;
-    const float e_cro = 16.0f * kEps * R2, e_so = 170.0f * kEps * R2, e_sn = 280.0f * kEps * R2;
+    const float e_so = 170.0f * kEps * R2, e_sn = 300.0f * kEps * R2;
     if (!(so > e_so && sn > e_sn)) return 0;  // degenerate: no information
+    // e_dcr so + (|dcr| + e_dcr) e_so + e_cro |ds| + (|cro| + e_cro) e_ds
+    // + e (|dcr| so + 2 |cro| |ds|), with e_dcr = 32 e r R, e_ds = 100 e r R,
+    // e_cro = 16 e R^2 (products of two of them: 7040 e^2 r R^3)
     const float adcr = fabsf(dcr), ads = fabsf(ds), acro = fabsf(cro);
-    const float eN = e_dcr * so + (adcr + e_dcr) * e_so + e_cro * ads + (acro + e_cro) * e_ds +
-                     kEps * (adcr * so + 2.0f * acro * ads);
+    const float e1 = fmaf(32.0f, so, fmaf(100.0f, acro, 7040.0f * kEps * R2));
+    const float e2 = fmaf(170.0f, adcr, 16.0f * ads);
+    const float eN = kEps * fmaf(rR, e1, fmaf(R2, e2, fmaf(adcr, so, 2.0f * (acro * ads))));
     const float need = (2.02f * kE64 / kTwoSqrt3f) * (sn + e_sn) * (so + e_so);
     if (!(fabsf(N) - 2.0f * eN > need)) return 0;
     return ((N > 0.0f) == (sgn > 0.0f)) ? 1 : -1;

@@ -1,0 +1,85 @@
+// window_pipe.cuh -- what the pass kernels share in working through a window
+// stream (window.cuh): list entries, asynchronous copies, the slots in which
+// headers and idle marks are held ahead of their use.
+#pragma once
+
+#include "device.cuh"
+#include "window.cuh"
+
+namespace sls {
+
+// A block keeps two windows in shared memory: the one it works on and the
+// next one, which is copied in meanwhile.  Headers are fetched three windows
+// ahead and halo ids two, because each names what the next copies.
+struct __align__(16) Ahead {
+    uint32_t hdr[4][win::kHeaderWords];  // window i's header in slot i & 3
+    uint8_t idle[4][4];                  // skip_unchanged: its subtiles that need no work
+};
+
+// Asynchronous copies global -> shared (no registers held while they fly).
+__device__ __forceinline__ void copy16(void *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void copy8(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void copy4(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// List entries of BITS bits in a lane's words (32 words apart), as byte
+// offsets of staged entries of 2^SHIFT bytes.
+template <int BITS, int SHIFT = 4>
+struct List {
+    static constexpr uint32_t kPer = 32 / BITS;
+    static __device__ __forceinline__ uint32_t in_word(uint32_t word, uint32_t j)
+    {
+        return ((word >> (BITS * j)) & ((1u << BITS) - 1u)) << SHIFT;
+    }
+    static __device__ __forceinline__ uint32_t at(const uint32_t *list, uint32_t t)
+    {
+        return in_word(list[32u * (t / kPer)], t % kPer);
+    }
+};
+
+// Packed FP32 pairs: one instruction for two operations, the same roundings.
+__device__ __forceinline__ uint64_t pair(float lo, float hi)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void halves(uint64_t v, float &lo, float &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// Words of the halo ids of a window, whole 16-byte copies.
+__host__ __device__ inline uint32_t ids_words_of(const WindowShape &s) { return ((uint32_t)s.halo + 3u) & ~3u; }
+
+}  // namespace sls
