@@ -115,15 +115,15 @@ typedef struct sls_options {
                               and the screened kernel (SLS_KERNEL_AUTO or _FILTERED); costs
                               140 bytes of device memory per 32 nodes.  The batched and
                               allocation-free forms compute every tile; the server rejects it. */
-    int32_t numbering;     /* FP64, screened kernel: 0 (default) and 2 deal the nodes of every
+    int32_t numbering;     /* Screened and binary32 passes: 0 (default) and 2 deal the nodes of every
                               window of 128 consecutive ids to the lanes of its block by ring
                               length (the 32 lanes of a warp then run loops of similar
                               length), and renumber a Form-A mesh of at least 8192 nodes whose
                               numbering is not local (more than 45% of its triangles' edges
                               leave their window) along a Z-order curve, at creation (8 bytes
                               per node for the maps); 1 keeps the caller's order in both.  Not
-                              done with skip_unchanged (its 32-node tiles are the caller's),
-                              nor for binary32 meshes.  Every call still reads and writes
+                              done with skip_unchanged (its 32-node tiles are the caller's).
+                              Every call still reads and writes
                               coordinates, decisions and node ids in the caller's numbering;
                               results are identical.                                         */
     void *stream;          /* cudaStream_t to run on; NULL = a stream owned by the handle    */

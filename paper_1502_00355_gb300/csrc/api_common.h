@@ -110,12 +110,13 @@ struct DeviceAdjacency {
 // SLS_ERR_NOT_FOUND = a node is in too many triangles: use the host build.
 sls_status build_device_adjacency(int64_t n, int64_t m, double *d_xy, int32_t *d_tri, const uint8_t *h_boundary,
                                   bool renumber, cudaStream_t s, DeviceAdjacency &out);
-// Whether options o let the build renumber a mesh: the screened Form-A pass
-// (Form B's colouring follows the caller's numbering, skip_unchanged's tiles
-// are the caller's) unless the caller's numbering is to be kept.
+// Whether options o let the build renumber a mesh: Form-A passes that read a
+// window stream (Form B's colouring follows the caller's numbering,
+// skip_unchanged's tiles are the caller's) unless the caller's numbering is to
+// be kept.
 inline bool numbers_spatially(const sls_options &o)
 {
-    return o.form == 0 && o.precision != 32 && o.kernel != SLS_KERNEL_FP64 && !o.skip_unchanged && o.numbering != 1;
+    return o.form == 0 && (o.precision == 32 || o.kernel != SLS_KERNEL_FP64) && !o.skip_unchanged && o.numbering != 1;
 }
 // Device memory of the handles (memory.cu): stream-ordered allocations from
 // the library's pool on the current device, which keeps freed memory for
@@ -131,9 +132,10 @@ void pool_free(void *p, cudaStream_t s);
 // The window stream of a built adjacency (window_build.cu); segments: the id
 // ranges to cover one after another (Form B: the colour classes' bounds),
 // empty = one segment of all n nodes.  group: nodes dealt to the lanes by ring
-// length inside a window.  Synchronises s.
+// length inside a window.  cyclic: ring lists padded for the binary32 walk.
+// Synchronises s.
 sls_status build_windows(int64_t n, const std::vector<int64_t> &segments, const uint32_t *node_off,
-                         const uint32_t *adj, bool group, cudaStream_t s, WindowStream &out);
+                         const uint32_t *adj, bool group, bool cyclic, cudaStream_t s, WindowStream &out);
 // Whether options o deal a window's nodes to the lanes by ring length: not
 // where the caller's order is asked for, nor with skip_unchanged, whose
 // 32-node tiles are the subtiles.

@@ -285,7 +285,8 @@ sls_status sls_batch_create(sls_mesh *const *meshes, int32_t k, const int32_t *i
         // a mesh made for the plain FP64 kernel has no window stream yet
         sls_mesh *M = meshes[j];
         if (M->windows.hdr) continue;
-        sls_status st = build_windows(M->n, {}, M->node_off, M->adj, groups_lanes(M->opt), M->stream, M->windows);
+        sls_status st = build_windows(M->n, {}, M->node_off, M->adj, groups_lanes(M->opt), false, M->stream,
+                                      M->windows);
         if (st == SLS_OK && cudaStreamSynchronize(M->stream) != cudaSuccess) st = fail(SLS_ERR_CUDA, "windows");
         if (st != SLS_OK) return fail_free(st);
     }

@@ -60,8 +60,9 @@ cudaError_t launch_histogram(const double *xy, int layout, int64_t n, const int3
                              double *qsum, int grid, cudaStream_t s);
 
 // One pass in binary32 (pass_f32.cu): a.in / a.out hold floats.
-cudaError_t launch_pass_f32(const PassArgs &a, int layout, int block, int grid, cudaStream_t s);
-int pass_f32_occupancy(int layout, int block);
+cudaError_t launch_pass_f32(const PassArgs &a, int layout, int block, int grid, const WindowShape &shape,
+                            cudaStream_t s);
+int pass_f32_occupancy(int layout, int block, const WindowShape &shape);
 // Copy-back form of the binary32 pass (count floats; skipped when pass q was skipped).
 cudaError_t launch_copy_back_f32(const float *src, float *dst, int64_t count, const PassStats *stats, int q,
                                  int grid, cudaStream_t s);

@@ -71,7 +71,7 @@ static sls_status mesh_setup(sls_mesh *M, const sls_options &o)
     M->block = o.block_size;
     M->screened = o.kernel != SLS_KERNEL_FP64 && !M->f32;
     if (M->screened && M->block > 128) M->block = 128;  // the screened kernel is built for <= 128
-    if (M->f32 && M->block > 256) M->block = 256;  // the binary32 kernel is built for <= 256
+    if (M->f32 && M->block > 128) M->block = 128;  // and so is the binary32 kernel
     if (o.l2_window) {
         // Persisting L2 for the coordinates each pass gathers from: the
         // context's persisting carve-out covers at most one coordinate array.
@@ -88,9 +88,7 @@ static sls_status mesh_setup(sls_mesh *M, const sls_options &o)
     }
     sls_status pst = noalloc_prepare();
     if (pst != SLS_OK) return pst;
-    if (!M->screened)
-        M->grid = device_sm_count() * (M->f32 ? pass_f32_occupancy(o.layout, M->block)
-                                              : pass_fp64_occupancy(o.layout, M->block));
+    if (!M->screened && !M->f32) M->grid = device_sm_count() * pass_fp64_occupancy(o.layout, M->block);
     return SLS_OK;
 }
 
@@ -101,11 +99,14 @@ static sls_status finish_creation(sls_mesh *M)
 {
     sls_status st = build_node_order(M, M->stream);
     if (st != SLS_OK) return st;
-    if (M->screened) {
+    if (M->screened || M->f32) {
         st = build_windows(M->n, M->opt.form == 1 ? M->colour_off : std::vector<int64_t>(), M->node_off, M->adj,
-                           groups_lanes(M->opt), M->stream, M->windows);
+                           groups_lanes(M->opt), M->f32, M->stream, M->windows);
         if (st != SLS_OK) return st;
-        M->grid = device_sm_count() * pass_screened_occupancy(M->opt.layout, M->block, M->windows.shape);
+        M->grid = device_sm_count() * (M->f32 ? pass_f32_occupancy(M->opt.layout, M->block, M->windows.shape)
+                                              : pass_screened_occupancy(M->opt.layout, M->block, M->windows.shape));
+    }
+    if (M->screened) {
         PassArgs a{};
         a.win_count = M->windows.count;
         M->resident = M->opt.form == 0 && !M->opt.copy_back && !M->opt.skip_unchanged && !M->opt.l2_window &&
@@ -274,7 +275,7 @@ static void set_l2_window(const sls_mesh *M, const void *base, size_t bytes)
 static cudaError_t launch_pass(const sls_mesh *M, const PassArgs &a)
 {
     if (M->opt.l2_window) set_l2_window(M, a.in, (M->f32 ? sizeof(float) : sizeof(double)) * 2 * (size_t)M->n);
-    if (M->f32) return launch_pass_f32(a, M->opt.layout, M->block, M->grid, M->stream);
+    if (M->f32) return launch_pass_f32(a, M->opt.layout, M->block, M->grid, M->windows.shape, M->stream);
     return M->screened ? launch_pass_screened(a, M->opt.layout, M->block, M->grid, M->windows.shape, M->stream)
                        : launch_pass_fp64(a, M->opt.layout, M->block, M->grid, M->stream);
 }
@@ -328,8 +329,8 @@ sls_status mesh_run(sls_mesh *M, int32_t max_iter, double tol_rel, sls_info &inf
             a.out = M->xy[M->cur ^ (launched & 1) ^ 1];
             if (launched > 0)
                 SLS_CUDA_TRY(cudaMemsetAsync(barrier, 0, sizeof(unsigned) * kBarrierWords, M->stream), "cudaMemset");
-            SLS_CUDA_TRY(launch_resident(a, M->opt.layout, M->block, M->windows.shape, end - launched, barrier, M->stream),
-                         "pass kernel");
+            SLS_CUDA_TRY(launch_resident(a, M->opt.layout, M->block, M->windows.shape, end - launched, barrier,
+                                         M->stream), "pass kernel");
             ++kernels;
         }
         for (int q = launched; q < end && !M->resident; ++q) {
@@ -344,7 +345,7 @@ sls_status mesh_run(sls_mesh *M, int32_t max_iter, double tol_rel, sls_info &inf
                     a.ranged = 1;
                     a.first = nseg > 0 ? M->colour_off[c] : 0;
                     a.count = nseg > 0 ? M->colour_off[c + 1] - M->colour_off[c] : 0;
-                    if (M->screened) {
+                    if (M->windows.hdr) {
                         a.win_first = nseg > 0 ? M->windows.first_window[c] : 0;
                         a.win_count = nseg > 0 ? M->windows.first_window[c + 1] - a.win_first : 0;
                     }

@@ -11,10 +11,17 @@
 #include <cfloat>
 
 #include "kernels.h"
+#include "screen.cuh"
+#include "window_pipe.cuh"
 
 namespace sls {
 
 namespace {
+
+// RN(1/N), N up to the longest ring of the window lists.
+__constant__ const float c_recip32[16] = {0.0f,        1.0f,        1.0f / 2.0f,  1.0f / 3.0f,  1.0f / 4.0f, 1.0f / 5.0f,
+                                          1.0f / 6.0f, 1.0f / 7.0f, 1.0f / 8.0f,  1.0f / 9.0f,  1.0f / 10.0f, 1.0f / 11.0f,
+                                          1.0f / 12.0f, 1.0f / 13.0f, 1.0f / 14.0f, 1.0f / 15.0f};
 
 template <int LAYOUT>
 struct Coords32;
@@ -61,29 +68,31 @@ __device__ __forceinline__ float alpha_f32(float ax, float ay, float bx, float b
     return s > 0.0f ? __fdiv_rn(__fmul_rn(kTwoSqrt3, cross), s) : 0.0f;
 }
 
-// alpha of an incident triangle (node i, neighbours A and B) with node i at
-// x, in the triangle's stored vertex order (i in slot `slot`, A before B).
-// The tree of alpha_f32 rewritten with u = x - A, w = x - B, v = B - A: every
-// edge of the stored order is one of +-u, +-w, +-v, and negation commutes
-// with rounding, so
-//   slot 0: cross = u x w,     s = (|u|^2 + |w|^2) + |v|^2
-//   slot 1: cross = u x v,     s = (|u|^2 + |v|^2) + |w|^2
-//   slot 2: cross = -(u x v),  s = (|v|^2 + |u|^2) + |w|^2 (the same sum)
-// give bit for bit the values of alpha_f32 on the reordered points.  v and
-// |v|^2 are shared by both positions of node i; no lane branches on slot.
-__device__ __forceinline__ float alpha_uvw(uint32_t slot, float2 x, float2 A, float2 B, float2 v, float lv)
+// alpha of an incident triangle with the node at x, from its two other
+// vertices in ring order P -> Q (window.cuh): slot is the node's place in the
+// stored triangle, rev whether the step runs against the stored direction.
+// With dP = x - P, dQ = x - Q, E = Q - P and base = Q for slot 1, else P (the
+// other way round with rev), alpha_f32's tree on the stored order is
+//   slot 0:     cross = dP x dQ,        s = (|dP|^2 + |dQ|^2) + |E|^2
+//   slots 1, 2: cross = -(dbase x E),   s = (|dbase|^2 + |E|^2) + |dother|^2
+// with the cross product negated for rev: every edge of the stored order is
+// one of these or its negative, negation commutes with rounding, and so do the
+// operands of a product or of the first sum.
+__device__ __forceinline__ float alpha_ring(uint32_t slot, bool rev, float2 x, float2 P, float2 Q)
 {
-    const float kTwoSqrt3 = 3.46410161514f;
-    const float2 u = make_float2(__fsub_rn(x.x, A.x), __fsub_rn(x.y, A.y));
-    const float2 w = make_float2(__fsub_rn(x.x, B.x), __fsub_rn(x.y, B.y));
-    const float lu = __fadd_rn(__fmul_rn(u.x, u.x), __fmul_rn(u.y, u.y));
-    const float lw = __fadd_rn(__fmul_rn(w.x, w.x), __fmul_rn(w.y, w.y));
-    const bool s0 = slot == 0u;
-    const float2 z = s0 ? w : v;
-    float cross = __fsub_rn(__fmul_rn(u.x, z.y), __fmul_rn(u.y, z.x));
-    cross = slot == 2u ? -cross : cross;
-    const float s = __fadd_rn(__fadd_rn(lu, s0 ? lw : lv), s0 ? lv : lw);
-    return s > 0.0f ? __fdiv_rn(__fmul_rn(kTwoSqrt3, cross), s) : 0.0f;
+    const float2 dP = make_float2(__fsub_rn(x.x, P.x), __fsub_rn(x.y, P.y));
+    const float2 dQ = make_float2(__fsub_rn(x.x, Q.x), __fsub_rn(x.y, Q.y));
+    const float2 E = make_float2(__fsub_rn(Q.x, P.x), __fsub_rn(Q.y, P.y));
+    const float lP = __fadd_rn(__fmul_rn(dP.x, dP.x), __fmul_rn(dP.y, dP.y));
+    const float lQ = __fadd_rn(__fmul_rn(dQ.x, dQ.x), __fmul_rn(dQ.y, dQ.y));
+    const float lE = __fadd_rn(__fmul_rn(E.x, E.x), __fmul_rn(E.y, E.y));
+    const bool zero = slot == 0u, first = zero || (slot == 1u) == rev;  // the base (slot 0: d1) is P
+    const float2 d = first ? dP : dQ, z = zero ? dQ : E;
+    float cross = __fsub_rn(__fmul_rn(d.x, z.y), __fmul_rn(d.y, z.x));
+    cross = zero == rev ? -cross : cross;
+    const float l1 = first ? lP : lQ, other = first ? lQ : lP;
+    const float s = __fadd_rn(__fadd_rn(l1, zero ? other : lE), zero ? lE : other);
+    return s > 0.0f ? __fdiv_rn(__fmul_rn(3.46410161514f, cross), s) : 0.0f;
 }
 
 template <int LAYOUT>
@@ -98,106 +107,347 @@ __device__ __forceinline__ float alpha_at(const float *in, int64_t n, const uint
     }
 }
 
-// Rings up to this size live in shared memory (larger ones are read from
-// global memory).  12 slots keep five blocks' buffers within the 132 KB
-// shared-memory carve-out, which leaves the gathers about twice the L1 of
-// 16 slots (2.4% faster on jittered grids; a Delaunay mesh of random points
-// has about 1.4 nodes in 10,000 above 12).
-constexpr int kRingMax = 12;
-
-// One pass over every node, or over the ids of one colour class of Form B
-// (in place).  a.in / a.out hold floats.  Each thread
-// keeps its node's ring in its own column of a shared buffer (stride: block);
-// nodes with larger rings read their neighbours from global memory.
+// One node from its adjacency record, one thread: rings that are not in the
+// window lists, and values outside the range in which the pass's quick
+// quotients are understood.  Returns (bits of the squared move, 1) when it
+// moved to its centre, else (0, 0).
 template <int LAYOUT>
-__global__ void __launch_bounds__(256) pass_f32_kernel(PassArgs a)
+__device__ __noinline__ uint2 update_by_record(const PassArgs &a, const float *in, float *out, int64_t i)
 {
-    __shared__ float2 s_ring[kRingMax * 256];
+    const uint32_t off = __ldg(a.node_off + i);
+    const uint32_t meta = __ldg(a.adj + off);
+    const uint32_t deg = meta_degree(meta), ntri = meta_ntri(meta);
+    const uint32_t *nb = a.adj + off + 1;
+    const float2 p = Coords32<LAYOUT>::get(in, a.n, i);
+    float2 s = Coords32<LAYOUT>::get(in, a.n, __ldg(nb));
+    for (uint32_t k = 1; k < deg; ++k) {
+        const float2 v = Coords32<LAYOUT>::get(in, a.n, __ldg(nb + k));
+        s.x = __fadd_rn(s.x, v.x);
+        s.y = __fadd_rn(s.y, v.y);
+    }
+    const float fd = (float)deg;
+    const float2 c = make_float2(__fdiv_rn(s.x, fd), __fdiv_rn(s.y, fd));
+    // a tie (the centre is the node itself) means q_new == q_old
+    bool ok = !a.strict;
+    if (__float_as_uint(c.x) != __float_as_uint(p.x) || __float_as_uint(c.y) != __float_as_uint(p.y)) {
+        float q_old = 0.0f, q_new = 0.0f;
+        for (uint32_t t = 0; t < ntri; ++t) {
+            const uint32_t code = __ldg(nb + deg + t);
+            const float qo = alpha_at<LAYOUT>(in, a.n, nb, code, p);
+            const float qn = alpha_at<LAYOUT>(in, a.n, nb, code, c);
+            q_old = (t == 0u || qo < q_old) ? qo : q_old;  // first wins, as in the definition
+            q_new = (t == 0u || qn < q_new) ? qn : q_new;
+        }
+        ok = a.strict ? (q_new > q_old) : (q_new >= q_old);
+    }
+    Coords32<LAYOUT>::put(out, a.n, i, ok ? c : p);
+    if (a.accept) a.accept[i] = ok ? 1 : 0;
+    const float dx = __fsub_rn(c.x, p.x), dy = __fsub_rn(c.y, p.y);
+    return ok ? make_uint2(__float_as_uint(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy))), 1u) : make_uint2(0u, 0u);
+}
+
+// ---- the pass ------------------------------------------------------------------
+// Windows of nodes staged in shared memory and rings walked once, as in
+// pass_screened.cu, here with 8-byte entries and no splits.  Every step of
+// alpha's tree is the definition's operation (before and after the move in
+// the halves of packed pairs); only its last, the division, is replaced by a
+// product with the approximate reciprocal, within 3 units in the last place.
+// The minima of the approximate qualities differ from the exact ones by no
+// more, so a difference above 16 units decides the test; what is left (about a
+// node in a thousand) is evaluated with IEEE divisions, a lane per triangle
+// and side.
+//
+// Bound by instruction issue (70% of slots; 815 warp instructions per 32
+// nodes, 118 of them the selections that the stored order asks for, against
+// 1,072 with a thread gathering its own ring).  2048^2 jittered grid: 126 us a
+// pass against 164.
+
+constexpr int kBlock32 = 128;
+constexpr int kBlocks32 = 9;  // per SM; 126.3 us a pass on 2048^2 (6: 130.4, 8: 127.2, 10: 128.1, 12: 130.8)
+
+struct Block32 {
+    Ahead *ahead;
+    uint32_t *ids, *rows;
+    char *xy;
+    uint32_t ids_words, rows_words, stage;
+};
+
+size_t smem_f32(const WindowShape &s)
+{
+    return sizeof(Ahead) + 2 * 4 * (size_t)ids_words_of(s) + 2 * 128 * (size_t)(s.hot + win::kColdRows) +
+           2 * 8 * (size_t)(s.entries + 1);
+}
+
+__device__ __forceinline__ float2 entry32(const char *xy, uint32_t off)
+{
+    return *reinterpret_cast<const float2 *>(xy + off);
+}
+
+// s / N by Markstein's correction: with y = RN(1/N) and q0 = RN(s y), the
+// remainder s - q0 N is exact and RN(q0 + remainder y) is the rounded quotient
+// (checked over every significand for N = 2 .. 15).  Outside the range where
+// nothing under- or overflows: the division.
+__device__ __forceinline__ float div_degree(float s, float fn, float y)
+{
+    const float q0 = __fmul_rn(s, y);
+    const float q = __fmaf_rn(__fmaf_rn(-q0, fn, s), y, q0);
+    const float m = fabsf(s);
+    return (m > 1e-30f && m < 1e30f) ? q : __fdiv_rn(s, fn);
+}
+
+// x - vertex before | after the move, and the squared lengths.
+struct Vertex32 {
+    float x, y;
+    uint64_t dx, dy, l;
+};
+
+__device__ __forceinline__ Vertex32 vertex32(const char *xy, uint32_t off, float2 p, float2 c)
+{
+    const float2 v = entry32(xy, off);
+    Vertex32 r;
+    r.x = v.x;
+    r.y = v.y;
+    r.dx = pair(__fsub_rn(p.x, v.x), __fsub_rn(c.x, v.x));
+    r.dy = pair(__fsub_rn(p.y, v.y), __fsub_rn(c.y, v.y));
+    r.l = add2(mul2(r.dx, r.dx), mul2(r.dy, r.dy));
+    return r;
+}
+
+struct Minima32 {
+    float o, n, smin, smax;
+};
+
+// alpha_ring before and after the move, with a quick quotient.
+template <bool IRREGULAR>
+__device__ __forceinline__ void step32(Minima32 &m, const Vertex32 &P, const Vertex32 &Q, uint32_t slot, bool rev)
+{
+    if (IRREGULAR && slot == 3u) return;
+    const float ex = __fsub_rn(Q.x, P.x), ey = __fsub_rn(Q.y, P.y);
+    const float le = __fadd_rn(__fmul_rn(ex, ex), __fmul_rn(ey, ey));
+    const bool r = IRREGULAR && rev;
+    const bool zero = slot == 0u, first = zero || (slot == 1u) == r;
+    const uint64_t ex2 = pair(ex, ex), ey2 = pair(ey, ey), le2 = pair(le, le), minus = pair(-1.0f, -1.0f);
+    const uint64_t dx = first ? P.dx : Q.dx, dy = first ? P.dy : Q.dy;
+    const uint64_t zx = zero ? Q.dx : ex2, zy = zero ? Q.dy : ey2;
+    // a * b - c * d with both products rounded: RN(c d) times -1 is exact
+    const uint64_t cross = fma2(mul2(dy, zx), minus, mul2(dx, zy));
+    const uint64_t l1 = first ? P.l : Q.l, other = first ? Q.l : P.l;
+    const uint64_t s2 = add2(add2(l1, zero ? other : le2), zero ? le2 : other);
+    float so, sn, ko, kn;
+    halves(s2, so, sn);
+    const float k = zero == r ? -3.46410161514f : 3.46410161514f;
+    halves(mul2(cross, pair(k, k)), ko, kn);
+    m.o = fminf(m.o, ko * scr::rcp_ring(so));
+    m.n = fminf(m.n, kn * scr::rcp_ring(sn));
+    m.smin = fminf(m.smin, fminf(so, sn));
+    m.smax = fmaxf(m.smax, fmaxf(so, sn));
+}
+
+// To the subtile's largest step number l, two steps at a time.  Lists of
+// closed rings go on around the ring, so a lane past its own steps meets its
+// first triangles again; irregular subtiles look at each lane's steps.
+template <bool IRREGULAR, int BITS>
+__device__ __forceinline__ Minima32 walk32(const char *xy, uint32_t l, uint32_t steps, const uint32_t *list, float2 p,
+                                           float2 c, uint32_t slots, uint32_t rev)
+{
+    using L = List<BITS, 3>;
+    Minima32 m;
+    m.o = m.n = m.smin = FLT_MAX;
+    m.smax = 0.0f;
+    uint32_t word = list[0];
+    Vertex32 A = vertex32(xy, L::in_word(word, 0), p, c);
+    for (uint32_t t = 0;; t += L::kPer) {
+#pragma unroll
+        for (uint32_t j = 0; j < L::kPer; j += 2) {
+            const uint32_t e1 = L::in_word(word, j + 1);
+            if (j + 2 == L::kPer) {
+                list += 32;
+                word = *list;
+            }
+            const uint32_t e2 = L::in_word(word, (j + 2) % L::kPer);
+            const Vertex32 B = vertex32(xy, e1, p, c);
+            const Vertex32 C = vertex32(xy, e2, p, c);
+            const uint32_t t1 = t + j, t2 = t + j + 1u;
+            if (!IRREGULAR || t1 < steps) step32<IRREGULAR>(m, A, B, (slots >> (2u * t1)) & 3u, (rev >> t1) & 1u);
+            if (!IRREGULAR || t2 < steps) step32<IRREGULAR>(m, B, C, (slots >> (2u * t2)) & 3u, (rev >> t2) & 1u);
+            A = C;
+            if (t2 + 1u >= l) return m;
+        }
+    }
+}
+
+// Works subtile `sub` of a staged window; best: bits of the largest squared
+// move (non-negative floats order as integers).
+template <int LAYOUT, int BITS>
+__device__ __forceinline__ void work32(const PassArgs &a, const float *in, float *out, const char *xy,
+                                       const uint32_t *h, const uint32_t *rows, int sub, unsigned &best,
+                                       unsigned &nacc)
+{
+    using L = List<BITS, 3>;
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t d = (h[3] >> (8 * sub)) & 15u, l = (h[3] >> (8 * sub + 4)) & 15u;
+    const uint32_t *at = rows + ((h[4] >> (8 * sub)) & 0xffu) * 32u + lane;
+    const uint32_t *cold = rows + (h[5] + 2u * sub) * 32u + lane;
+    const uint32_t meta = *at;
+    const int64_t node = (int64_t)h[1] + win::meta_place(meta);
+    const bool have = (meta & win::kNode) != 0u, free = (meta & win::kFree) != 0u;
+    if (have && !(meta & (win::kFree | win::kBig)) && a.accept) a.accept[node] = 0;
+    bool record = have && (meta & win::kBig);
+    if (d > 0u) {
+        const uint32_t deg = win::meta_deg(meta), steps = win::meta_steps(meta);
+        const uint32_t *list = at + 32;
+        uint32_t word = *list;
+        float2 s = entry32(xy, L::in_word(word, 0));
+        for (uint32_t k = 0;;) {  // Eq. 2 in the stored order; padding adds -0
+#pragma unroll
+            for (uint32_t j = 0; j < L::kPer; ++j) {
+                if (j == 0u && k == 0u) continue;
+                const float2 v = entry32(xy, L::in_word(word, j));
+                s.x = __fadd_rn(s.x, v.x);
+                s.y = __fadd_rn(s.y, v.y);
+            }
+            k += L::kPer;
+            list += 32;
+            if (k >= d) break;
+            word = *list;
+        }
+        list = at + 32u * (1u + win::list_rows(d, BITS));
+        const float2 p = entry32(xy, (win::meta_place(meta) + 1u) * 8u);
+        float2 c = p;
+        if (free) {
+            const float fn = (float)deg, y = c_recip32[deg];
+            c = make_float2(div_degree(s.x, fn, y), div_degree(s.y, fn, y));
+        }
+        // a tie (the centre is the node itself) means q_new == q_old
+        bool act = __float_as_uint(c.x) != __float_as_uint(p.x) || __float_as_uint(c.y) != __float_as_uint(p.y);
+        int verdict = free && !act ? (a.strict ? -1 : 1) : 0;
+        if (__any_sync(0xffffffffu, act)) {
+            const uint32_t slots = *cold, rev = cold[32];
+            const bool irregular = win::hdr_irregular(h[2], (uint32_t)sub);
+            const Minima32 m = irregular ? walk32<true, BITS>(xy, l, steps, list, p, c, slots, rev)
+                                         : walk32<false, BITS>(xy, l, steps, list, p, c, slots, 0u);
+            // normal sums and finite points: the quick quotients are within 3 units
+            // (an infinite neighbour makes some sum infinite, or all of them NaN)
+            const float far = fmaxf(fmaxf(fabsf(p.x), fabsf(p.y)), fmaxf(fabsf(c.x), fabsf(c.y)));
+            const bool fine = m.smin > 1e-30f && m.smax > 1e-30f && m.smax < 1e30f && far < 1e30f;
+            if (act && !fine) record = true;
+            act = act && fine;
+            const float gap = m.n - m.o;
+            if (act && fabsf(gap) > 2e-6f * fmaxf(fabsf(m.o), fabsf(m.n))) verdict = gap > 0.0f ? 1 : -1;
+            // the others: lane t takes step t before the move, lane 16 + t after it
+            for (unsigned open = __ballot_sync(0xffffffffu, act && verdict == 0); open; open &= open - 1u) {
+                const uint32_t src = (uint32_t)__ffs((int)open) - 1u, t = lane & 15u;
+                const uint32_t st = __shfl_sync(0xffffffffu, steps, src), sl = __shfl_sync(0xffffffffu, slots, src);
+                const uint32_t rv = __shfl_sync(0xffffffffu, irregular ? rev : 0u, src);
+                const float2 ps = make_float2(__shfl_sync(0xffffffffu, p.x, src), __shfl_sync(0xffffffffu, p.y, src));
+                const float2 cs = make_float2(__shfl_sync(0xffffffffu, c.x, src), __shfl_sync(0xffffffffu, c.y, src));
+                const uint32_t *ring = list + (int)src - (int)lane;
+                const uint32_t slot = (sl >> (2u * t)) & 3u;
+                float q = FLT_MAX;
+                if (t < st && slot != 3u)
+                    q = alpha_ring(slot, ((rv >> t) & 1u) != 0u, lane < 16u ? ps : cs, entry32(xy, L::at(ring, t)),
+                                   entry32(xy, L::at(ring, t + 1u)));
+                for (int w = 8; w > 0; w >>= 1) q = fminf(q, __shfl_xor_sync(0xffffffffu, q, w));
+                const float q_old = __shfl_sync(0xffffffffu, q, 0), q_new = __shfl_sync(0xffffffffu, q, 16);
+                if (lane == src) verdict = (a.strict ? q_new > q_old : q_new >= q_old) ? 1 : -1;
+            }
+        }
+        if (verdict != 0) {
+            if (verdict > 0) {
+                const float dx = __fsub_rn(c.x, p.x), dy = __fsub_rn(c.y, p.y);
+                best = max(best, __float_as_uint(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy))));
+                nacc += 1u;
+            }
+            Coords32<LAYOUT>::put(out, a.n, node, verdict > 0 ? c : p);
+            if (a.accept) a.accept[node] = verdict > 0 ? 1 : 0;
+        }
+    }
+    if (record) {
+        const uint2 r = update_by_record<LAYOUT>(a, in, out, node);
+        best = max(best, r.x);
+        nacc += r.y;
+    }
+    __syncwarp();
+}
+
+// One pass over a mesh's windows, or over those of one colour class of Form B
+// (in place).  a.in / a.out hold floats.
+template <int LAYOUT, int BITS>
+__global__ void __launch_bounds__(kBlock32, kBlocks32)
+    pass_f32_kernel(const __grid_constant__ PassArgs a, const __grid_constant__ WindowShape shape)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
     if (pass_is_skipped(a.stats, a.q, a.tol_active, a.thr_bits)) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) a.stats[a.q].executed = 1u;
     const float *in = reinterpret_cast<const float *>(a.in);
     float *out = reinterpret_cast<float *>(a.out);
-    float2 *ring = s_ring + threadIdx.x;
-    const int rs = blockDim.x;
+    const int tid = threadIdx.x, warp = tid >> 5, nthr = blockDim.x, nwarps = nthr >> 5;
+    Block32 b;
+    b.ahead = reinterpret_cast<Ahead *>(smem);
+    b.ids = reinterpret_cast<uint32_t *>(smem + sizeof(Ahead));
+    b.ids_words = ids_words_of(shape);
+    b.rows = b.ids + 2 * b.ids_words;
+    b.rows_words = 32u * (uint32_t)(shape.hot + (int)win::kColdRows);
+    b.xy = reinterpret_cast<char *>(b.rows + 2 * b.rows_words);
+    b.stage = (uint32_t)(shape.entries + 1) * 8u;
+    if (tid < 2) *reinterpret_cast<float2 *>(b.xy + tid * b.stage) = make_float2(-0.0f, -0.0f);  // the padding entries
 
-    unsigned best = 0u;  // bits of the largest squared move (non-negative floats order as integers)
-    unsigned long long nacc = 0ull;
-    const int64_t cnt = a.ranged ? a.count : a.n;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < cnt; j += stride) {
-        const int64_t i = a.first + j;
-        const uint32_t off = __ldg(a.node_off + i);
-        const uint32_t meta = __ldg(a.adj + off);
-        if (meta & kMetaFixed) {
-            if (a.accept) a.accept[i] = 0;
-            continue;
-        }
-        const uint32_t deg = meta_degree(meta), ntri = meta_ntri(meta);
-        const uint32_t *nb = a.adj + off + 1;
-        const float2 p = Coords32<LAYOUT>::get(in, a.n, i);
-        float2 c;
-        float q_old = FLT_MAX, q_new = FLT_MAX;
-        bool tie;
-        if (deg <= (uint32_t)kRingMax) {
-            // Eq. 2 in the stored order; the ring goes to shared memory
-            float2 v = Coords32<LAYOUT>::get(in, a.n, __ldg(nb));
-            ring[0] = v;
-            float sx = v.x, sy = v.y;
-            for (uint32_t k = 1; k < deg; ++k) {
-                v = Coords32<LAYOUT>::get(in, a.n, __ldg(nb + k));
-                ring[k * rs] = v;
-                sx = __fadd_rn(sx, v.x);
-                sy = __fadd_rn(sy, v.y);
-            }
-            const float fd = (float)deg;
-            c = make_float2(__fdiv_rn(sx, fd), __fdiv_rn(sy, fd));
-            tie = __float_as_uint(c.x) == __float_as_uint(p.x) && __float_as_uint(c.y) == __float_as_uint(p.y);
-            if (!tie) {
-                for (uint32_t t = 0; t < ntri; ++t) {
-                    const uint32_t code = __ldg(nb + deg + t);
-                    const float2 A = ring[code_first(code) * rs];
-                    const float2 B = ring[code_second(code) * rs];
-                    const float2 vv = make_float2(__fsub_rn(B.x, A.x), __fsub_rn(B.y, A.y));
-                    const float lv = __fadd_rn(__fmul_rn(vv.x, vv.x), __fmul_rn(vv.y, vv.y));
-                    const float qo = alpha_uvw(code_slot(code), p, A, B, vv, lv);
-                    const float qn = alpha_uvw(code_slot(code), c, A, B, vv, lv);
-                    q_old = (t == 0u || qo < q_old) ? qo : q_old;  // first wins, as in the definition
-                    q_new = (t == 0u || qn < q_new) ? qn : q_new;
-                }
-            }
-        } else {
-            float2 v = Coords32<LAYOUT>::get(in, a.n, __ldg(nb));
-            float sx = v.x, sy = v.y;
-            for (uint32_t k = 1; k < deg; ++k) {
-                v = Coords32<LAYOUT>::get(in, a.n, __ldg(nb + k));
-                sx = __fadd_rn(sx, v.x);
-                sy = __fadd_rn(sy, v.y);
-            }
-            const float fd = (float)deg;
-            c = make_float2(__fdiv_rn(sx, fd), __fdiv_rn(sy, fd));
-            tie = __float_as_uint(c.x) == __float_as_uint(p.x) && __float_as_uint(c.y) == __float_as_uint(p.y);
-            if (!tie) {
-                for (uint32_t t = 0; t < ntri; ++t) {
-                    const uint32_t code = __ldg(nb + deg + t);
-                    const float qo = alpha_at<LAYOUT>(in, a.n, nb, code, p);
-                    const float qn = alpha_at<LAYOUT>(in, a.n, nb, code, c);
-                    q_old = (t == 0u || qo < q_old) ? qo : q_old;
-                    q_new = (t == 0u || qn < q_new) ? qn : q_new;
-                }
+    // windows blockIdx.x, + gridDim.x, ...: headers three ahead, halo ids two,
+    // rows and coordinates one (see run_windows in pass_screened.cu)
+    const int64_t w0 = a.win_first + blockIdx.x;
+    const int n = (int64_t)blockIdx.x < a.win_count ? (int)((a.win_count - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0;
+    Ahead *ah = b.ahead;
+    auto fetch_header = [&](int i) {
+        if (i < n && tid < 2)
+            copy16(&ah->hdr[i & 3][4 * tid],
+                   a.win_hdr + (w0 + (int64_t)i * gridDim.x) * win::kHeaderWords + 4 * tid);
+    };
+    auto fetch_ids = [&](int i) {
+        if (i >= n) return;
+        const uint32_t *h = ah->hdr[i & 3];
+        const uint32_t *src = a.win_rows + (size_t)h[0] * 32u;
+        uint32_t *dst = b.ids + (i & 1) * b.ids_words;
+        for (uint32_t k = 4 * tid; k < win::hdr_halo(h[2]); k += 4 * nthr) copy16(dst + k, src + k);
+    };
+    auto fetch_data = [&](int i) {
+        if (i >= n) return;
+        const uint32_t *h = ah->hdr[i & 3];
+        const uint32_t count = win::hdr_count(h[2]), nhalo = win::hdr_halo(h[2]);
+        const uint32_t *src = a.win_rows + ((size_t)h[0] + win::halo_rows(nhalo)) * 32u;
+        uint32_t *rows = b.rows + (i & 1) * b.rows_words;
+        for (uint32_t k = 4 * tid; k < 32u * (h[5] + win::kColdRows); k += 4 * nthr) copy16(rows + k, src + k);
+        const uint32_t *ids = b.ids + (i & 1) * b.ids_words;
+        char *xy = b.xy + (i & 1) * b.stage + 8;
+        for (uint32_t e = tid; e < count + nhalo; e += nthr) {
+            const int64_t id = e < count ? (int64_t)h[1] + e : (int64_t)ids[e - count];
+            if (LAYOUT == 0) {
+                copy8(xy + e * 8u, in + 2 * id);
+            } else {
+                copy4(xy + e * 8u, in + id);
+                copy4(xy + e * 8u + 4u, in + a.n + id);
             }
         }
-        // a tie (the centre is the node itself) means q_new == q_old
-        const bool ok = tie ? !a.strict : (a.strict ? (q_new > q_old) : (q_new >= q_old));
-        float2 o = p;
-        if (ok) {
-            const float dx = __fsub_rn(c.x, p.x), dy = __fsub_rn(c.y, p.y);
-            const float d2 = __fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy));
-            best = max(best, __float_as_uint(d2));
-            nacc += 1ull;
-            o = c;
-        }
-        Coords32<LAYOUT>::put(out, a.n, i, o);
-        if (a.accept) a.accept[i] = ok ? 1 : 0;
+    };
+    fetch_header(0);
+    fetch_header(1);
+    fetch_header(2);
+    copies_done();
+    __syncthreads();
+    fetch_ids(0);
+    fetch_ids(1);
+    copies_done();
+    __syncthreads();
+    fetch_data(0);
+    unsigned best = 0u, nacc = 0u;
+    for (int i = 0; i < n; ++i) {
+        copies_done();
+        __syncthreads();
+        fetch_data(i + 1);
+        fetch_ids(i + 2);
+        fetch_header(i + 3);
+        for (int sub = warp; sub < 4; sub += nwarps)
+            work32<LAYOUT, BITS>(a, in, out, b.xy + (i & 1) * b.stage, ah->hdr[i & 3],
+                                 b.rows + (i & 1) * b.rows_words, sub, best, nacc);
     }
     // widened exactly to double, so the pass records compare like FP64 ones
     const unsigned long long b64 = (unsigned long long)__double_as_longlong((double)__uint_as_float(best));
@@ -249,18 +499,33 @@ __global__ void widen_kernel(const float *__restrict__ src, double2 *aos, int64_
 
 }  // namespace
 
-cudaError_t launch_pass_f32(const PassArgs &a, int layout, int block, int grid, cudaStream_t s)
+namespace {
+
+const void *kernel32(int layout, int bits)
 {
-    if (layout == 0) pass_f32_kernel<0><<<grid, block, 0, s>>>(a);
-    else pass_f32_kernel<1><<<grid, block, 0, s>>>(a);
-    return cudaGetLastError();
+    if (layout == 0) return bits == 8 ? (const void *)pass_f32_kernel<0, 8> : (const void *)pass_f32_kernel<0, 16>;
+    return bits == 8 ? (const void *)pass_f32_kernel<1, 8> : (const void *)pass_f32_kernel<1, 16>;
 }
 
-int pass_f32_occupancy(int layout, int block)
+}  // namespace
+
+cudaError_t launch_pass_f32(const PassArgs &a, int layout, int block, int grid, const WindowShape &shape,
+                            cudaStream_t s)
 {
+    if (a.win_count < grid) grid = a.win_count > 0 ? (int)a.win_count : 1;
+    void *args[] = {const_cast<PassArgs *>(&a), const_cast<WindowShape *>(&shape)};
+    return cudaLaunchKernel(kernel32(layout, shape.bits), dim3(grid), dim3(block), args, smem_f32(shape), s);
+}
+
+// Also allows the kernel the shared memory that the shape takes; a launch in
+// another context would need it again, and meshes belong to their context.
+int pass_f32_occupancy(int layout, int block, const WindowShape &shape)
+{
+    const void *f = kernel32(layout, shape.bits);
     int nb = 0;
-    if (layout == 0) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, pass_f32_kernel<0>, block, 0);
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, pass_f32_kernel<1>, block, 0);
+    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess)
+        cudaGetLastError();
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, block, smem_f32(shape));
     return nb > 0 ? nb : 1;
 }
 

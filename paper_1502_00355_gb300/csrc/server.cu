@@ -333,7 +333,7 @@ sls_status build_job(ServerJob &J, bool group, bool numbers, cudaStream_t s, siz
     e = cudaFreeAsync(d_tri, s);
     d_tri = nullptr;
     if (e != cudaSuccess) return cuda_err(e, "build");
-    st = build_windows(n, {}, J.d_off, J.d_adj, group, s, J.windows);
+    st = build_windows(n, {}, J.d_off, J.d_adj, group, false, s, J.windows);
     if (st != SLS_OK) return cleanup(st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(J.d_xy[1], J.d_xy[0], cbytes, cudaMemcpyDeviceToDevice, s);
     if (e == cudaSuccess)

@@ -29,12 +29,14 @@ struct BuildTotals {
 __device__ __forceinline__ uint32_t hash_of(uint32_t id) { return (id * 2654435761u) >> 21; }
 
 // WRITE = false: hdr and totals; WRITE = true: the rows.
+// cyclic: the ring lists (and slots) of closed rings go on around the ring up to
+// their row's end (the binary32 walk), else unused entries are 0.
 // Windows are `width` ids wide; window w of segment s (win_off[s] <= w) starts
 // at seg_off[s] + (w - win_off[s]) * width.
 template <bool WRITE>
 __global__ void __launch_bounds__(win::kWindow) window_build_kernel(
     const uint32_t *__restrict__ node_off, const uint32_t *__restrict__ adj, const int64_t *__restrict__ seg_off,
-    const int64_t *__restrict__ win_off, int nseg, int64_t nwin, int width, int bits, int group, uint32_t *hdr,
+    const int64_t *__restrict__ win_off, int nseg, int64_t nwin, int width, int bits, int group, int cyclic, uint32_t *hdr,
     uint32_t *rows, BuildTotals *totals)
 {
     __shared__ uint32_t s_key[kHash];
@@ -152,7 +154,10 @@ __global__ void __launch_bounds__(win::kWindow) window_build_kernel(
             row[0] = have ? win::meta_word((uint32_t)t, listed ? deg : 0u, listed ? ring.steps : 0u,
                                            win::kNode | (listed ? win::kFree : (fixed ? 0u : win::kBig)))
                           : 0u;
-            cold[0] = listed ? ring.slots : 0u;
+            uint32_t slots = listed ? ring.slots : 0u;
+            if (cyclic && listed && ring.regular)
+                for (uint32_t k = ring.steps; k < 16u; ++k) slots |= ((slots >> (2u * (k - ring.steps))) & 3u) << (2u * k);
+            cold[0] = slots;
             cold[32] = listed ? ring.rev : 0u;
             if (d > 0u) {
                 uint16_t entry[win::kRingMax];
@@ -178,8 +183,10 @@ __global__ void __launch_bounds__(win::kWindow) window_build_kernel(
                 for (uint32_t k = 0; k < win::list_rows(win::ring_entries(l), (uint32_t)bits); ++k, o += 32) {
                     uint32_t word = 0u;
                     for (uint32_t j = 0; j < per; ++j)
-                        if (k * per + j < nring)
-                            word |= (uint32_t)entry[win::nib(ring.seq, k * per + j)] << (j * (uint32_t)bits);
+                        if (k * per + j < nring || (cyclic && listed && ring.regular))
+                            word |= (uint32_t)entry[win::nib(ring.seq, k * per + j < nring ? k * per + j
+                                                                                            : (k * per + j) % ring.steps)]
+                                    << (j * (uint32_t)bits);
                     *o = word;
                 }
             }
@@ -191,7 +198,7 @@ __global__ void __launch_bounds__(win::kWindow) window_build_kernel(
 }  // namespace
 
 sls_status build_windows(int64_t n, const std::vector<int64_t> &segments, const uint32_t *node_off,
-                         const uint32_t *adj, bool group, cudaStream_t s, WindowStream &out)
+                         const uint32_t *adj, bool group, bool cyclic, cudaStream_t s, WindowStream &out)
 {
     out.release(s);
     std::vector<int64_t> segs = segments;
@@ -237,7 +244,7 @@ sls_status build_windows(int64_t n, const std::vector<int64_t> &segments, const 
         const int64_t cap = (int64_t)device_sm_count() * 12;
         const unsigned grid = (unsigned)(out.count < cap ? out.count : cap);
         window_build_kernel<false><<<grid, win::kWindow, 0, s>>>(node_off, adj, d_offs, d_offs + nseg + 1, nseg,
-                                                                 out.count, width, bits, group ? 1 : 0, out.hdr, nullptr,
+                                                                 out.count, width, bits, group ? 1 : 0, cyclic ? 1 : 0, out.hdr, nullptr,
                                                                  d_tot);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemcpyAsync(&h, d_tot, sizeof h, cudaMemcpyDeviceToHost, s);
@@ -253,7 +260,7 @@ sls_status build_windows(int64_t n, const std::vector<int64_t> &segments, const 
             e = pool_alloc((void **)&out.rows, out.rows_bytes, s);
             if (e != cudaSuccess) return done(e, "window stream");
             window_build_kernel<true><<<grid, win::kWindow, 0, s>>>(node_off, adj, d_offs, d_offs + nseg + 1, nseg,
-                                                                    out.count, width, bits, group ? 1 : 0, out.hdr,
+                                                                    out.count, width, bits, group ? 1 : 0, cyclic ? 1 : 0, out.hdr,
                                                                     out.rows, nullptr);
             return done(cudaGetLastError(), "windows");
         }

@@ -202,3 +202,54 @@ def test_served_random_numbering(sls):
         srv.close()
     want, rinfo, _ = oracle.OracleMesh(mesh.xy, mesh.tri, mesh.boundary).smooth(mesh.xy, 15, tol=1e-9)
     assert np.array_equal(xy, want) and info["maxd2_last"] == rinfo["maxd2_last"]
+
+
+def _check32(sls, mesh, iters, tol=0.0, strict=False, form="A", **opts):
+    rxy, rinfo, racc = oracle.OracleMesh(mesh.xy, mesh.tri, mesh.boundary).smooth(
+        mesh.xy, iters, tol=tol, strict=strict, form=form, precision=32)
+    with sls.Mesh(mesh.xy, mesh.tri, mesh.boundary, strict=strict, record_accept=True, form=form, precision=32,
+                  **opts) as g:
+        info = g.smooth(iters, tol)
+        xy, acc = g.coords(), g.accept_mask()
+    assert np.array_equal(xy, rxy)
+    assert np.array_equal(acc, racc)
+    for k in ("iterations", "accepted_last", "maxd2_last"):
+        assert info[k] == rinfo[k], k
+
+
+@pytest.mark.parametrize("form", ["A", "B"])
+@pytest.mark.parametrize("layout", ["aos", "soa"])
+def test_binary32_forms(sls, form, layout):
+    opts = dict(form=form, layout=layout)
+    grid = meshgen.jittered_grid(61, 47, 0.35, 7, pull_fraction=0.05, pull_centres=16)
+    _check32(sls, grid, 60, 1e-9, **opts)                       # down to rounding-level ties
+    _check32(sls, grid, 20, strict=True, **opts)
+    _check32(sls, _turned(grid, 0.3, 1), 20, **opts)
+    _check32(sls, _turned(grid, 1.0, 2), 20, **opts)
+    _check32(sls, _with_free_rim(meshgen.jittered_grid(45, 33, 0.3, 9)), 15, **opts)
+    _check32(sls, _fans(list(range(3, 34)), 4), 4, **opts)
+    _check32(sls, _split_thrice(31, 29, 5), 10, **opts)
+    _check32(sls, meshgen.delaunay_random(5000, 6, numbering="random"), 15, **opts)
+    _check32(sls, meshgen.jittered_grid(120, 97, 0.3, 11, numbering="random"), 10, **opts)
+    _check32(sls, meshgen.jittered_grid(33, 33, 0.0, 3, h=2.0 ** -5, diagonals="uniform"), 3, **opts)
+
+
+@pytest.mark.parametrize("scale", [1e-17, 1e-21, 1e14, 1e18, 1e30])
+def test_binary32_range(sls, scale):
+    # sums of squares below and above the quick quotients' range, and infinite
+    mesh = meshgen.jittered_grid(31, 29, 0.35, 23)
+    mesh.xy = mesh.xy * scale
+    with np.errstate(all="ignore"):
+        for opts in ({}, dict(block_size=32)):
+            rxy, rinfo, _ = oracle.OracleMesh(mesh.xy, mesh.tri, mesh.boundary).smooth(mesh.xy, 4, precision=32)
+            with sls.Mesh(mesh.xy, mesh.tri, mesh.boundary, precision=32, **opts) as g:
+                info = g.smooth(4)
+                assert np.array_equal(g.coords(), rxy, equal_nan=True)
+            assert info["accepted_last"] == rinfo["accepted_last"]
+
+
+def test_binary32_far_from_the_origin(sls):
+    mesh = meshgen.jittered_grid(40, 37, 0.3, 16)
+    mesh.xy = mesh.xy + 3.0e3
+    _check32(sls, mesh, 12)
+    _check32(sls, mesh, 12, strict=True, form="B")
