@@ -253,3 +253,44 @@ def test_binary32_far_from_the_origin(sls):
     mesh.xy = mesh.xy + 3.0e3
     _check32(sls, mesh, 12)
     _check32(sls, mesh, 12, strict=True, form="B")
+
+
+def _pinched(fans, seed):
+    """A free node where `fans` separate groups of three triangles meet."""
+    rng = np.random.default_rng(seed)
+    xy, tri = [np.array([0.03, -0.02])], []
+    for f in range(fans):
+        ang = 2 * np.pi * (f + np.array([0.1, 0.3, 0.5, 0.8]) + 0.05 * rng.random(4)) / fans
+        at = len(xy)
+        xy += list(np.c_[np.cos(ang), np.sin(ang)])
+        tri += [(0, at + k, at + k + 1) for k in range(3)]
+    bnd = np.ones(len(xy), np.uint8)
+    bnd[0] = 0
+    return meshgen.Mesh(xy=np.array(xy), tri=np.array(tri, np.int32), boundary=bnd)
+
+
+@pytest.mark.parametrize("share", [0.0, 0.5, 1.0])
+@pytest.mark.parametrize("rounded", [False, True])
+def test_records_built_on_the_device(sls, share, rounded):
+    # rings up to and beyond what the build keeps in registers (at most 32, so
+    # the host build does not take over), all orientations, coordinates that tie
+    fans = _fans(list(range(3, 33)), 16)
+    grid = meshgen.jittered_grid(23, 19, 0.3, 17)
+    for mesh in (fans, _with_free_rim(grid)):
+        m = _turned(mesh, share, 18)
+        if rounded:
+            m = meshgen.Mesh(xy=np.round(m.xy * 8) / 8, tri=m.tri, boundary=m.boundary)  # also -0.0
+        _check(sls, m, 3)
+        _check(sls, m, 3, numbering="given")
+
+
+@pytest.mark.parametrize("fans", [1, 2, 3, 5, 10])
+def test_records_longer_than_their_place(sls, fans):
+    # separate fans at a free node have more neighbours than its triangles
+    # leave room for: the whole mesh is built with exact lengths
+    mesh = _turned(_pinched(fans, 19), 0.5, 20)
+    rest = meshgen.jittered_grid(31, 17, 0.3, 21)
+    _check(sls, mesh, 3)
+    both = meshgen.Mesh(xy=np.vstack([rest.xy, mesh.xy + 4.0]), tri=np.vstack([rest.tri, mesh.tri + rest.n]).astype(np.int32),
+                        boundary=np.concatenate([rest.boundary, mesh.boundary]))
+    _check(sls, both, 5)
