@@ -30,7 +30,7 @@ template <>
 struct Coords32<0> {  // AoS: one float2 per node
     static __device__ __forceinline__ float2 get(const float *p, int64_t, int64_t i)
     {
-        return __ldg(reinterpret_cast<const float2 *>(p) + i);
+        return __ldcg(reinterpret_cast<const float2 *>(p) + i);
     }
     static __device__ __forceinline__ void put(float *p, int64_t, int64_t i, float2 v)
     {
@@ -42,7 +42,7 @@ template <>
 struct Coords32<1> {  // SoA: x[n] then y[n]
     static __device__ __forceinline__ float2 get(const float *p, int64_t n, int64_t i)
     {
-        return make_float2(__ldg(p + i), __ldg(p + n + i));
+        return make_float2(__ldcg(p + i), __ldcg(p + n + i));
     }
     static __device__ __forceinline__ void put(float *p, int64_t n, int64_t i, float2 v)
     {
@@ -377,8 +377,6 @@ __global__ void __launch_bounds__(kBlock32, kBlocks32)
     pass_f32_kernel(const __grid_constant__ PassArgs a, const __grid_constant__ WindowShape shape)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    if (pass_is_skipped(a.stats, a.q, a.tol_active, a.thr_bits)) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.stats[a.q].executed = 1u;
     const float *in = reinterpret_cast<const float *>(a.in);
     float *out = reinterpret_cast<float *>(a.out);
     const int tid = threadIdx.x, warp = tid >> 5, nthr = blockDim.x, nwarps = nthr >> 5;
@@ -437,6 +435,9 @@ __global__ void __launch_bounds__(kBlock32, kBlocks32)
     fetch_ids(1);
     copies_done();
     __syncthreads();
+    after_previous();
+    if (pass_is_skipped(a.stats, a.q, a.tol_active, a.thr_bits)) return;
+    if (blockIdx.x == 0 && tid == 0) a.stats[a.q].executed = 1u;
     fetch_data(0);
     unsigned best = 0u, nacc = 0u;
     for (int i = 0; i < n; ++i) {
@@ -514,7 +515,7 @@ cudaError_t launch_pass_f32(const PassArgs &a, int layout, int block, int grid, 
 {
     if (a.win_count < grid) grid = a.win_count > 0 ? (int)a.win_count : 1;
     void *args[] = {const_cast<PassArgs *>(&a), const_cast<WindowShape *>(&shape)};
-    return cudaLaunchKernel(kernel32(layout, shape.bits), dim3(grid), dim3(block), args, smem_f32(shape), s);
+    return launch_early(kernel32(layout, shape.bits), grid, block, args, smem_f32(shape), s);
 }
 
 // Also allows the kernel the shared memory that the shape takes; a launch in

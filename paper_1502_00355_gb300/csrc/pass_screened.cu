@@ -732,7 +732,10 @@ __device__ __forceinline__ void work_subtile(const PassArgs &a, Queue *q, const 
 // per window says that it is there and that window i - 1, whose buffer the
 // next copies overwrite, is finished.  (With one buffer of staged entries the
 // copies wait for that barrier, and a second one says that they are there.)
-template <int LAYOUT, int BITS, bool HALO>
+//
+// EARLY: the kernel may have started before the one in front of it ended
+// (after_previous); whether the pass is to run is known only then.
+template <int LAYOUT, int BITS, bool HALO, bool EARLY>
 __device__ __forceinline__ void run_windows(const PassArgs &a, const Block &blk, int64_t w0, int n, int64_t stride,
                                             Tally &tally, unsigned &nskip, bool &full)
 {
@@ -805,10 +808,17 @@ __device__ __forceinline__ void run_windows(const PassArgs &a, const Block &blk,
     __syncthreads();
     fetch_ids(0);
     fetch_ids(1);
-    check_idle(0);
-    check_idle(1);
+    if (!EARLY) {
+        check_idle(0);
+        check_idle(1);
+    }
     copies_done();
     __syncthreads();
+    if (EARLY) {
+        after_previous();
+        if (pass_is_skipped(a.stats, a.q, a.tol_active, a.thr_bits)) return;
+        if (blockIdx.x == 0 && tid == 0) a.stats[a.q].executed = 1u;
+    }
     if (blk.stage) fetch_data(0);
     for (int i = 0; i < n; ++i) {
         if (!blk.stage) {  // one buffer: window i - 1 has to be finished first
@@ -834,7 +844,7 @@ __device__ __forceinline__ void run_windows(const PassArgs &a, const Block &blk,
         if (rest) continue;
         for (int sub = warp; sub < 4; sub += nwarps) {
             if (HALO && a.skip && ah->idle[i & 3][sub]) continue;
-            work_subtile<LAYOUT, BITS, false, HALO>(a, blk.q, xy, blk.half, h, blk.rows + (i & 1) * blk.rows_words,
+            work_subtile<LAYOUT, BITS, EARLY, HALO>(a, blk.q, xy, blk.half, h, blk.rows + (i & 1) * blk.rows_words,
                                                     sub, tally, full);
         }
     }
@@ -852,16 +862,20 @@ __global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
     pass_screened_kernel(const __grid_constant__ PassArgs a, const __grid_constant__ WindowShape shape)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (pass_is_skipped(a.stats, a.q, a.tol_active, a.thr_bits)) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.stats[a.q].executed = 1u;
+    // (the masks of skip_unchanged are read where a window's header is: no early start)
+    if (HALO || a.win_count == 0) {  // the launch over an empty list has no window to start with
+        if (!HALO) after_previous();
+        if (pass_is_skipped(a.stats, a.q, a.tol_active, a.thr_bits)) return;
+        if (blockIdx.x == 0 && threadIdx.x == 0) a.stats[a.q].executed = 1u;
+    }
     const Block blk = block_memory(smem_raw, shape);
     Tally tally{0u, 0u};
     unsigned nskip = 0u;  // node updates this warp left as they were (lane 0)
     bool full = false;
     if ((int64_t)blockIdx.x < a.win_count)
-        run_windows<LAYOUT, BITS, HALO>(a, blk, a.win_first + blockIdx.x,
-                                  (int)((a.win_count - blockIdx.x + gridDim.x - 1) / gridDim.x), gridDim.x, tally,
-                                  nskip, full);
+        run_windows<LAYOUT, BITS, HALO, !HALO>(a, blk, a.win_first + blockIdx.x,
+                                               (int)((a.win_count - blockIdx.x + gridDim.x - 1) / gridDim.x),
+                                               gridDim.x, tally, nskip, full);
     __syncthreads();
     if (blk.q->npending) tally = drain<LAYOUT, HALO>(a, blk.q, tally);
     if (nskip) atomicAdd(&a.stats[a.q].nodes_skipped, nskip);
@@ -1063,9 +1077,9 @@ __global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
         if (!active) continue;
         if (window == 0 && threadIdx.x == 0) s_args.stats[s_args.q].executed = 1u;
         if (WIDE && s_wide)
-            run_windows<LAYOUT, 16, false>(s_args, blk, window, (int)run, 1, tally, nskip, full);
+            run_windows<LAYOUT, 16, false, false>(s_args, blk, window, (int)run, 1, tally, nskip, full);
         else
-            run_windows<LAYOUT, 8, false>(s_args, blk, window, (int)run, 1, tally, nskip, full);
+            run_windows<LAYOUT, 8, false, false>(s_args, blk, window, (int)run, 1, tally, nskip, full);
     }
 }
 
@@ -1148,8 +1162,8 @@ cudaError_t launch_pass_screened(const PassArgs &a, int layout, int block, int g
     if (e != cudaSuccess) return e;
     if (a.win_count < grid) grid = a.win_count > 0 ? (int)a.win_count : 1;
     void *args[] = {const_cast<PassArgs *>(&a), const_cast<WindowShape *>(&shape)};
-    return cudaLaunchKernel(a.halo ? kernel_of<true>(layout, shape.bits) : kernel_of<false>(layout, shape.bits),
-                            dim3(grid), dim3(block), args, smem_for(shape), s);
+    if (a.halo) return cudaLaunchKernel(kernel_of<true>(layout, shape.bits), dim3(grid), dim3(block), args, smem_for(shape), s);
+    return launch_early(kernel_of<false>(layout, shape.bits), grid, block, args, smem_for(shape), s);
 }
 
 bool resident_fits(const PassArgs &a, int layout, int block, const WindowShape &shape)
