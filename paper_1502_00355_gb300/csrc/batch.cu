@@ -77,7 +77,7 @@ sls_status build_graph(sls_batch *B)
     cudaError_t err = cudaSuccess;
     for (int r = 0; r < B->rounds && err == cudaSuccess; ++r)
         err = launch_batch_pass(B->d_jobs, B->d_tasks, B->round_tasks[r], r, B->layout, B->block, B->grid,
-                                B->shape, B->stream, B->chunk, B->d_claim + r);
+                                B->shape, B->stream, B->chunk, B->d_claim + r, true);
     cudaError_t e2 = cudaStreamEndCapture(B->stream, &g);
     if (err != cudaSuccess) {
         if (g) cudaGraphDestroy(g);

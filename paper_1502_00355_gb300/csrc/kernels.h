@@ -35,16 +35,16 @@ cudaError_t launch_resident(const PassArgs &a, int layout, int block, const Wind
 // chunk > 0: tasks per block chunk, taken in a grid stride; chunk < 0: chunks
 // of -chunk tasks claimed in order from *claim (zero at the launch); 0 = one
 // contiguous share of the task list per block.  shape covers every job's
-// windows.
+// windows.  own_graph: the library captures the launch into a graph of its own.
 cudaError_t launch_batch_pass(const JobDesc *jobs, const WindowTask *tasks, int64_t ntasks, int round, int layout,
                               int block, int grid, const WindowShape &shape, cudaStream_t s, int64_t chunk,
-                              unsigned long long *claim);
+                              unsigned long long *claim, bool own_graph = false);
 int batch_pass_occupancy(int layout, int block, const WindowShape &shape);
 // The window tasks of the na jobs of a table (job j's tasks from task_off[j]).
 cudaError_t launch_expand_tasks(const JobDesc *jobs, const int64_t *task_off, int na, WindowTask *tasks,
                                 cudaStream_t s);
 // Record of round `round` of each of the na jobs (pass round - base_round,
-// clamped to the job's last pass) into out[0 .. na).
+// clamped to the job's last pass) into out[0 .. na), page-locked host memory.
 cudaError_t launch_gather_round(const JobDesc *jobs, int na, int round, PassStats *out, cudaStream_t s);
 
 // Copy-back form: out -> in after pass q (skipped when pass q was skipped).

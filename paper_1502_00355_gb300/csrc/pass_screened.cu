@@ -998,9 +998,11 @@ __global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
 // The queue is worked off and the statistics flushed whenever the block moves
 // to another job, so every record gets exactly its own job's counts.
 // WIDE: some job's lists may have 16-bit entries.
+// (The tables may be written by the kernel in front, so they are not
+// __restrict__: a load known never to change could move above after_previous.)
 template <int LAYOUT, bool WIDE>
 __global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
-    batch_pass_kernel(const JobDesc *__restrict__ jobs, const WindowTask *__restrict__ tasks, int64_t ntasks,
+    batch_pass_kernel(const JobDesc *jobs, const WindowTask *tasks, int64_t ntasks,
                       int round, int64_t chunk, unsigned long long *claim, const __grid_constant__ WindowShape shape)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1019,6 +1021,7 @@ __global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
         return s_claim;
     };
     int64_t c0 = dynamic ? claim_next() : (int64_t)blockIdx.x * per;  // first task of the current chunk
+    after_previous();  // (a round has its own claim counter)
     int64_t t = c0;
     int cur_job = -1;
     Tally tally{0u, 0u};
@@ -1186,7 +1189,7 @@ cudaError_t launch_resident(const PassArgs &a, int layout, int block, const Wind
 
 cudaError_t launch_batch_pass(const JobDesc *jobs, const WindowTask *tasks, int64_t ntasks, int round, int layout,
                               int block, int grid, const WindowShape &shape, cudaStream_t s, int64_t chunk,
-                              unsigned long long *claim)
+                              unsigned long long *claim, bool own_graph)
 {
     cudaError_t e = ensure_constants();
     if (e != cudaSuccess) return e;
@@ -1194,14 +1197,17 @@ cudaError_t launch_batch_pass(const JobDesc *jobs, const WindowTask *tasks, int6
     if (chunk < 0 && !claim) return cudaErrorInvalidValue;
     if (ntasks < grid) grid = (int)ntasks;
     void *args[] = {&jobs, &tasks, &ntasks, &round, &chunk, &claim, const_cast<WindowShape *>(&shape)};
-    return cudaLaunchKernel(batch_kernel_of(layout, shape.bits), dim3(grid), dim3(block), args, smem_for(shape), s);
+    return launch_early(batch_kernel_of(layout, shape.bits), grid, block, args, smem_for(shape), s, own_graph);
 }
 
 namespace {
 
-__global__ void gather_round_kernel(const JobDesc *__restrict__ jobs, int na, int round, PassStats *out)
+// `out` is page-locked host memory: the records arrive without a copy behind
+// the kernel.
+__global__ void gather_round_kernel(const JobDesc *jobs, int na, int round, PassStats *out)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    after_previous();
     if (j >= na) return;
     const JobDesc &J = jobs[j];
     int q = round - J.base_round;
@@ -1233,8 +1239,8 @@ cudaError_t launch_expand_tasks(const JobDesc *jobs, const int64_t *task_off, in
 cudaError_t launch_gather_round(const JobDesc *jobs, int na, int round, PassStats *out, cudaStream_t s)
 {
     if (na <= 0) return cudaSuccess;
-    gather_round_kernel<<<(na + 127) / 128, 128, 0, s>>>(jobs, na, round, out);
-    return cudaGetLastError();
+    void *args[] = {&jobs, &na, &round, &out};
+    return launch_early((const void *)gather_round_kernel, (na + 127) / 128, 128, args, 0, s);
 }
 
 int batch_pass_occupancy(int layout, int block, const WindowShape &shape)

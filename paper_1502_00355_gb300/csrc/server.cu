@@ -208,8 +208,7 @@ struct sls_server {
     WindowTask *d_tasks = nullptr;
     size_t jobs_cap = 0, jobs_hcap[2] = {0, 0}, toff_cap = 0, toff_hcap[2] = {0, 0}, tasks_cap = 0;
     PassStats *h_round[2] = {nullptr, nullptr};  // pinned: a round's record of each job it ran over
-    PassStats *d_round[2] = {nullptr, nullptr};  // the same records gathered on the device
-    size_t round_cap[2] = {0, 0}, dround_cap[2] = {0, 0};
+    size_t round_cap[2] = {0, 0};
     cudaEvent_t ev_start[2] = {nullptr, nullptr}, ev_done[2] = {nullptr, nullptr};
     int64_t ntasks = 0;
     int block = 256, grid = 0;
@@ -661,8 +660,7 @@ void scheduler_loop(sls_server *S)
                 }
                 dirty = false;
             }
-            if (!grow_host(S->h_round[slot], S->round_cap[slot], na) ||
-                !grow_dev(S->d_round[slot], S->dround_cap[slot], na)) {
+            if (!grow_host(S->h_round[slot], S->round_cap[slot], na)) {
                 S->sched_error = "out of pinned host memory";
                 break;
             }
@@ -670,11 +668,8 @@ void scheduler_loop(sls_server *S)
             if (e == cudaSuccess)
                 e = launch_batch_pass(S->d_jobs, S->d_tasks, S->ntasks, S->round, S->opt.layout, S->block, S->grid,
                                       S->shape, S->stream, kServerChunk, nullptr);
-            // every job's record of this round, gathered by one kernel, read back by one copy
-            if (e == cudaSuccess) e = launch_gather_round(S->d_jobs, (int)na, S->round, S->d_round[slot], S->stream);
-            if (e == cudaSuccess)
-                e = cudaMemcpyAsync(S->h_round[slot], S->d_round[slot], sizeof(PassStats) * na,
-                                    cudaMemcpyDeviceToHost, S->stream);
+            // every job's record of this round, gathered into host memory by one kernel
+            if (e == cudaSuccess) e = launch_gather_round(S->d_jobs, (int)na, S->round, S->h_round[slot], S->stream);
             if (e == cudaSuccess) e = cudaEventRecord(S->ev_done[slot], S->stream);
             if (e != cudaSuccess) {
                 S->sched_error = cudaGetErrorString(e);
@@ -934,7 +929,6 @@ sls_status sls_server_destroy(sls_server *S)
         cudaFreeHost(S->h_jobs[b]);
         cudaFreeHost(S->h_toff[b]);
         cudaFreeHost(S->h_round[b]);
-        cudaFree(S->d_round[b]);
         if (S->ev_start[b]) cudaEventDestroy(S->ev_start[b]);
         if (S->ev_done[b]) cudaEventDestroy(S->ev_done[b]);
     }

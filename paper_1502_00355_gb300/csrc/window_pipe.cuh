@@ -54,11 +54,13 @@ __device__ __forceinline__ void after_previous()
 
 // Launches `kernel`, which calls after_previous(), to start early; in a stream
 // that is being captured it is an ordinary launch (the graph then has only
-// full dependencies, as its owner may expect).
-inline cudaError_t launch_early(const void *kernel, int grid, int block, void **args, size_t smem, cudaStream_t s)
+// full dependencies, as its owner may expect) unless the library itself is
+// capturing it (own_graph).
+inline cudaError_t launch_early(const void *kernel, int grid, int block, void **args, size_t smem, cudaStream_t s,
+                                bool own_graph = false)
 {
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) {
+    if (!own_graph && cudaStreamIsCapturing(s, &capture) != cudaSuccess) {
         cudaGetLastError();  // the legacy stream while another one is being captured: the launch will say so
         capture = cudaStreamCaptureStatusNone;
     }
