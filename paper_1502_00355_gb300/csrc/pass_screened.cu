@@ -95,20 +95,26 @@ struct Block {
     uint32_t *rows;           // hot rows
     char *xy;                 // staged entries: coordinates, then head/tail splits
     uint32_t ids_words, rows_words, half, stage;  // buffer sizes: words, words, bytes of one array, bytes
-                                                  // from one buffer to the other (0: there is one)
+                                                  // from one buffer to the other (0: there is one, of the
+                                                  // rows too)
 };
 
 // Buffers of staged entries: one where two would leave an SM with few blocks.
 // Colour classes (about 510 entries a window) run 233 us a sweep with one and
 // 281 with two (1500 x 1100 grid), a random numbering kept as it is (900
 // entries) 111 against 144 us a pass; local numberings (at most 255) gain 8%
-// from the second.
+// from the second.  The lists' rows, fetched with the entries, have as many
+// buffers: with one instead of two, 38 sweeps of that grid take 7.06 instead
+// of 7.33 ms.  (Shared memory by colour class, 37 to 51 KB, made each class's
+// kernel faster by itself, 38 against 44 us, but the sweeps slower, 7.46
+// against 7.14 ms: launches of unlike sizes overlap less.)
 constexpr int kTwoBufferEntries = 320;
+static_assert(kTwoBufferEntries >= 255, "8-bit lists");
 __host__ __device__ inline int buffers_for(const WindowShape &s) { return s.entries <= kTwoBufferEntries ? 2 : 1; }
 size_t smem_for(const WindowShape &s)
 {
-    return sizeof(Queue) + sizeof(Ahead) + 2 * 4 * (size_t)ids_words_of(s) + 2 * 128 * (size_t)s.hot +
-           (size_t)buffers_for(s) * 32 * (size_t)(s.entries + 1);
+    return sizeof(Queue) + sizeof(Ahead) + 2 * 4 * (size_t)ids_words_of(s) +
+           (size_t)buffers_for(s) * (128 * (size_t)s.hot + 32 * (size_t)(s.entries + 1));
 }
 
 struct Tally {
@@ -148,6 +154,7 @@ __device__ __forceinline__ void note_move(Queue *q, unsigned long long b2)
     atomicMax(reinterpret_cast<int *>(&q->best_low), __float_as_int(__double2float_rd(bitsd(b2))));
 }
 
+template <bool TWO>
 __device__ __forceinline__ Block block_memory(unsigned char *smem, const WindowShape &s)
 {
     Block b;
@@ -156,8 +163,8 @@ __device__ __forceinline__ Block block_memory(unsigned char *smem, const WindowS
     b.ids = reinterpret_cast<uint32_t *>(smem + sizeof(Queue) + sizeof(Ahead));
     b.ids_words = ids_words_of(s);
     b.rows = b.ids + 2 * b.ids_words;
+    b.xy = reinterpret_cast<char *>(b.rows + (TWO ? 2 : buffers_for(s)) * 32 * s.hot);
     b.rows_words = 32u * (uint32_t)s.hot;
-    b.xy = reinterpret_cast<char *>(b.rows + 2 * b.rows_words);
     b.half = (uint32_t)(s.entries + 1) * 16u;
     b.stage = buffers_for(s) == 2 ? 2u * b.half : 0u;
     // the padding entries: -0 for the sums, NaN for the rings
@@ -735,12 +742,15 @@ __device__ __forceinline__ void work_subtile(const PassArgs &a, Queue *q, const 
 //
 // EARLY: the kernel may have started before the one in front of it ended
 // (after_previous); whether the pass is to run is known only then.
-template <int LAYOUT, int BITS, bool HALO, bool EARLY>
+// TWO: there are two buffers whatever the windows (8-bit lists: at most 255
+// entries).
+template <int LAYOUT, int BITS, bool HALO, bool EARLY, bool TWO>
 __device__ __forceinline__ void run_windows(const PassArgs &a, const Block &blk, int64_t w0, int n, int64_t stride,
                                             Tally &tally, unsigned &nskip, bool &full)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthr = blockDim.x, nwarps = nthr >> 5;
     Ahead *ah = blk.ahead;
+    const bool two = blk.stage != 0u;
 
     auto fetch_header = [&](int i) {
         if (i < n && tid < 2)
@@ -761,7 +771,7 @@ __device__ __forceinline__ void run_windows(const PassArgs &a, const Block &blk,
         const uint32_t *h = ah->hdr[i & 3];
         const uint32_t count = win::hdr_count(h[2]), nhalo = win::hdr_halo(h[2]);
         const uint32_t *src = a.win_rows + ((size_t)h[0] + win::halo_rows(nhalo)) * 32u;
-        uint32_t *rows = blk.rows + (i & 1) * blk.rows_words;
+        uint32_t *rows = blk.rows + (TWO || two ? i & 1 : 0) * blk.rows_words;
         for (uint32_t k = 4 * tid; k < 32u * h[5]; k += 4 * nthr) copy16(rows + k, src + k);
         const uint32_t *ids = blk.ids + (i & 1) * blk.ids_words;
         char *xy = blk.xy + (i & 1) * blk.stage + 16;
@@ -819,9 +829,9 @@ __device__ __forceinline__ void run_windows(const PassArgs &a, const Block &blk,
         if (pass_is_skipped(a.stats, a.q, a.tol_active, a.thr_bits)) return;
         if (blockIdx.x == 0 && tid == 0) a.stats[a.q].executed = 1u;
     }
-    if (blk.stage) fetch_data(0);
+    if (two) fetch_data(0);
     for (int i = 0; i < n; ++i) {
-        if (!blk.stage) {  // one buffer: window i - 1 has to be finished first
+        if (!two) {  // one buffer: window i - 1 has to be finished first
             copies_done();
             __syncthreads();
             fetch_data(i);
@@ -837,15 +847,16 @@ __device__ __forceinline__ void run_windows(const PassArgs &a, const Block &blk,
             tally = drain<LAYOUT, HALO>(a, blk.q, tally);
             full = false;
         }
-        if (blk.stage) fetch_data(i + 1);
+        if (two) fetch_data(i + 1);
         fetch_ids(i + 2);
         fetch_header(i + 3);
         check_idle(i + 2);
         if (rest) continue;
         for (int sub = warp; sub < 4; sub += nwarps) {
             if (HALO && a.skip && ah->idle[i & 3][sub]) continue;
-            work_subtile<LAYOUT, BITS, EARLY, HALO>(a, blk.q, xy, blk.half, h, blk.rows + (i & 1) * blk.rows_words,
-                                                    sub, tally, full);
+            work_subtile<LAYOUT, BITS, EARLY, HALO>(a, blk.q, xy, blk.half, h,
+                                                    blk.rows + (TWO || two ? i & 1 : 0) * blk.rows_words, sub, tally,
+                                                    full);
         }
     }
 }
@@ -868,14 +879,14 @@ __global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
         if (pass_is_skipped(a.stats, a.q, a.tol_active, a.thr_bits)) return;
         if (blockIdx.x == 0 && threadIdx.x == 0) a.stats[a.q].executed = 1u;
     }
-    const Block blk = block_memory(smem_raw, shape);
+    const Block blk = block_memory<BITS == 8>(smem_raw, shape);
     Tally tally{0u, 0u};
     unsigned nskip = 0u;  // node updates this warp left as they were (lane 0)
     bool full = false;
     if ((int64_t)blockIdx.x < a.win_count)
-        run_windows<LAYOUT, BITS, HALO, !HALO>(a, blk, a.win_first + blockIdx.x,
-                                               (int)((a.win_count - blockIdx.x + gridDim.x - 1) / gridDim.x),
-                                               gridDim.x, tally, nskip, full);
+        run_windows<LAYOUT, BITS, HALO, !HALO, BITS == 8>(
+            a, blk, a.win_first + blockIdx.x, (int)((a.win_count - blockIdx.x + gridDim.x - 1) / gridDim.x), gridDim.x,
+            tally, nskip, full);
     __syncthreads();
     if (blk.q->npending) tally = drain<LAYOUT, HALO>(a, blk.q, tally);
     if (nskip) atomicAdd(&a.stats[a.q].nodes_skipped, nskip);
@@ -930,7 +941,7 @@ __global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
     __shared__ PassArgs s_args;
     __shared__ bool s_stop;
     const int tid = threadIdx.x, warp = tid >> 5, nthr = blockDim.x, nwarps = nthr >> 5;
-    const Block blk = block_memory(smem_raw, shape);
+    const Block blk = block_memory<BITS == 8>(smem_raw, shape);
     if (tid == 0) {
         s_args = a0;
         s_stop = pass_is_skipped(a0.stats, a0.q, a0.tol_active, a0.thr_bits);
@@ -1009,7 +1020,7 @@ __global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
     __shared__ PassArgs s_args;
     __shared__ int64_t s_claim;
     __shared__ int s_active, s_wide, s_windows;
-    const Block blk = block_memory(smem_raw, shape);
+    const Block blk = block_memory<!WIDE>(smem_raw, shape);
     const bool dynamic = chunk < 0;
     const int64_t nblocks = gridDim.x;
     const int64_t per = chunk > 0 ? chunk : (dynamic ? -chunk : (ntasks + nblocks - 1) / nblocks);
@@ -1080,9 +1091,9 @@ __global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
         if (!active) continue;
         if (window == 0 && threadIdx.x == 0) s_args.stats[s_args.q].executed = 1u;
         if (WIDE && s_wide)
-            run_windows<LAYOUT, 16, false, false>(s_args, blk, window, (int)run, 1, tally, nskip, full);
+            run_windows<LAYOUT, 16, false, false, false>(s_args, blk, window, (int)run, 1, tally, nskip, full);
         else
-            run_windows<LAYOUT, 8, false, false>(s_args, blk, window, (int)run, 1, tally, nskip, full);
+            run_windows<LAYOUT, 8, false, false, !WIDE>(s_args, blk, window, (int)run, 1, tally, nskip, full);
     }
 }
 
