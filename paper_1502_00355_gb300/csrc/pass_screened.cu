@@ -862,12 +862,12 @@ __device__ __forceinline__ void run_windows(const PassArgs &a, const Block &blk,
 }
 
 // The kernels are compiled for 7 blocks of 128 threads per SM (72 registers):
-// 2048^2 runs 201 us a pass with 7, 207 with 6 and 218 with 8, whose 64
-// registers spill.
+// 2048^2 ran 201 us a pass with 7, 207 with 6 and 218 with 8, whose 64
+// registers spill, when this was chosen (174 now).
 constexpr int kBlocksPerSm = 7;
 
 // HALO: the mesh keeps the masks of skip_unchanged (apart: their code costs
-// other meshes registers, 217 against 202 us a pass on 2048^2).
+// other meshes registers, 217 against 202 us a pass on 2048^2 at the time).
 template <int LAYOUT, int BITS, bool HALO>
 __global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
     pass_screened_kernel(const __grid_constant__ PassArgs a, const __grid_constant__ WindowShape shape)
@@ -898,8 +898,8 @@ __global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
 // window's lists in shared memory and runs pass after pass, with a grid-wide
 // barrier between passes instead of a launch.  What is left of a pass is its
 // own chain of dependent steps (coordinates from L2, the sums, the ring walk,
-// the queue, the barrier).  A 64^2 mesh runs 9.3 us a pass against 13.5 with a
-// launch each, 100,000 Delaunay points 19 against 23; past one window per
+// the queue, the barrier).  A 64^2 mesh runs 9.3 us a pass against 13.5 with an
+// ordinary launch each, 100,000 Delaunay points 16 to 19 against 23; past one window per
 // resident block (about 136,000 nodes) the blocks would have to fetch their
 // lists again every pass, as separate launches do.
 
