@@ -151,9 +151,10 @@ __device__ __noinline__ uint2 update_by_record(const PassArgs &a, const float *i
 // pass_screened.cu, here with 8-byte entries and no splits.  Every step of
 // alpha's tree is the definition's operation (before and after the move in
 // the halves of packed pairs); only its last, the division, is replaced by a
-// product with the approximate reciprocal, within 3 units in the last place.
-// The minima of the approximate qualities differ from the exact ones by no
-// more, so a difference above 16 units decides the test; what is left (about a
+// product with the approximate reciprocal, within 3 units in the last place
+// (or of 2^-149, below the normal range).  The minima of the approximate
+// qualities differ from the exact ones by no more, so a difference above 16
+// units, and above 1e-36, decides the test; what is left (about a
 // node in a thousand) is evaluated with IEEE divisions, a lane per triangle
 // and side.
 //
@@ -332,8 +333,10 @@ __device__ __forceinline__ void work32(const PassArgs &a, const float *in, float
             const bool fine = m.smin > 1e-30f && m.smax > 1e-30f && m.smax < 1e30f && far < 1e30f;
             if (act && !fine) record = true;
             act = act && fine;
+            // (a quality below the normal range is a whole number of units of 2^-149,
+            // and a quick one off by about a unit: the absolute part of the margin)
             const float gap = m.n - m.o;
-            if (act && fabsf(gap) > 2e-6f * fmaxf(fabsf(m.o), fabsf(m.n))) verdict = gap > 0.0f ? 1 : -1;
+            if (act && fabsf(gap) > fmaf(2e-6f, fmaxf(fabsf(m.o), fabsf(m.n)), 1e-36f)) verdict = gap > 0.0f ? 1 : -1;
             // the others: lane t takes step t before the move, lane 16 + t after it
             for (unsigned open = __ballot_sync(0xffffffffu, act && verdict == 0); open; open &= open - 1u) {
                 const uint32_t src = (uint32_t)__ffs((int)open) - 1u, t = lane & 15u;
