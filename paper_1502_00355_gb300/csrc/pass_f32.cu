@@ -241,7 +241,7 @@ __device__ __forceinline__ void step32(Minima32 &m, const Vertex32 &P, const Ver
     m.o = fminf(m.o, ko * scr::rcp_ring(so));
     m.n = fminf(m.n, kn * scr::rcp_ring(sn));
     m.smin = fminf(m.smin, fminf(so, sn));
-    m.smax = fmaxf(m.smax, fmaxf(so, sn));
+    m.smax = max_nan(m.smax, max_nan(so, sn));
 }
 
 // To the subtile's largest step number l, two steps at a time.  Lists of
@@ -328,7 +328,9 @@ __device__ __forceinline__ void work32(const PassArgs &a, const float *in, float
             const Minima32 m = irregular ? walk32<true, BITS>(xy, l, steps, list, p, c, slots, rev)
                                          : walk32<false, BITS>(xy, l, steps, list, p, c, slots, 0u);
             // normal sums and finite points: the quick quotients are within 3 units
-            // (an infinite neighbour makes some sum infinite, or all of them NaN)
+            // (an infinite or NaN coordinate among the node's, the centre's and the
+            // neighbours' makes some sum infinite or NaN, and smax with it: the
+            // definition's quality is 0 there, the quick one has no value)
             const float far = fmaxf(fmaxf(fabsf(p.x), fabsf(p.y)), fmaxf(fabsf(c.x), fabsf(c.y)));
             const bool fine = m.smin > 1e-30f && m.smax > 1e-30f && m.smax < 1e30f && far < 1e30f;
             if (act && !fine) record = true;

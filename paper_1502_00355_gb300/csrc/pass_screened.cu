@@ -248,14 +248,6 @@ __device__ __noinline__ Tally drain(const PassArgs &a, Queue *q, Tally tally)
 // ---- the ring walk: screen.cuh's ring form, both sides of the move in the
 // halves of packed FP32 pairs.
 
-// The larger of two, NaN when either is.
-__device__ __forceinline__ float max_nan(float a, float b)
-{
-    float r;
-    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-    return r;
-}
-
 // What the walk knows of the node.
 struct RingWalk {
     const char *split;         // staged head/tail splits

@@ -122,6 +122,14 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
     return r;
 }
 
+// The larger of two, NaN when either is.
+__device__ __forceinline__ float max_nan(float a, float b)
+{
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+
 // Words of the halo ids of a window, whole 16-byte copies.
 __host__ __device__ inline uint32_t ids_words_of(const WindowShape &s) { return ((uint32_t)s.halo + 3u) & ~3u; }
 

@@ -1,6 +1,7 @@
 """Binary32 passes where the quick quotients of the accept test are not to be
 trusted: qualities below the normal range (coordinates of subnormal extent in
-one direction), against the oracle's binary32 definition, bit for bit."""
+one direction) and coordinates that are not finite, against the oracle's
+binary32 definition, bit for bit."""
 import numpy as np
 import pytest
 
@@ -73,3 +74,21 @@ def test_meshes_of_subnormal_width(sls, units, axis, opts):
         return
     for strict in (False, True):
         _check(sls, mesh, mesh.xy, 6, strict, **opts)
+
+
+@pytest.mark.parametrize("opts", [dict(), dict(layout="soa", block_size=32)], ids=["aos", "soa"])
+@pytest.mark.parametrize("strict", [False, True])
+def test_coordinates_that_are_not_numbers(sls, opts, strict):
+    # a quality with a NaN in its edge sum is 0 by definition; NaN nodes among
+    # finite ones, NaN in one coordinate only, and the infinity that a double
+    # beyond the binary32 range becomes
+    grid = meshgen.jittered_grid(41, 37, 0.35, 32)
+    rng = np.random.default_rng(33)
+    for bad in ((np.nan, np.nan), (np.nan, None), (None, np.nan), (1e300, 0.5)):
+        start = grid.xy.copy()
+        for i in rng.choice(grid.n, 40, replace=False):
+            for c in range(2):
+                if bad[c] is not None:
+                    start[i, c] = bad[c]
+        for iters in (1, 2, 5):
+            _check(sls, grid, start, iters, strict, **opts)
