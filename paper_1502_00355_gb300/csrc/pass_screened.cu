@@ -650,8 +650,12 @@ __device__ __forceinline__ bool update_lane(const PassArgs &a, Queue *q, const c
 
 // ---- a block's windows ----------------------------------------------------------
 
-// Nodes of a subtile that their records decide, a warp each.
-template <int LAYOUT, bool COHERENT, bool HALO>
+// Nodes of a subtile that their records decide, a warp each.  Coordinates come
+// from L2: all kernels but those with masks (HALO) start early or run several
+// passes, so they may be resident while the coordinates that they will read
+// are still being written, and the read-only path (__ldg) is for data that
+// nobody writes while the kernel lives.
+template <int LAYOUT, bool HALO>
 __device__ __noinline__ Tally by_record(const PassArgs &a, Queue *q, int32_t node, unsigned left, Tally tally)
 {
     while (left) {
@@ -660,7 +664,7 @@ __device__ __noinline__ Tally by_record(const PassArgs &a, Queue *q, int32_t nod
         const int32_t nd = __shfl_sync(0xffffffffu, node, src);
         unsigned long long b2;
         bool acc, moved;
-        exact_update_warp<LAYOUT, COHERENT>(a, nd, b2, acc, moved);
+        exact_update_warp<LAYOUT, !HALO>(a, nd, b2, acc, moved);
         if ((threadIdx.x & 31) == 0) {
             note_move(q, b2);
             tally.nacc += acc ? 1u : 0u;
@@ -690,7 +694,7 @@ __device__ __forceinline__ void split_staged(char *xy, uint32_t half, uint32_t s
 
 // Updates the nodes of subtile `sub` of a staged window (h: its header, rows:
 // its hot rows in shared memory).
-template <int LAYOUT, int BITS, bool COHERENT, bool HALO>
+template <int LAYOUT, int BITS, bool HALO>
 __device__ __forceinline__ void work_subtile(const PassArgs &a, Queue *q, const char *xy, uint32_t half,
                                              const uint32_t *h, const uint32_t *rows, int sub, Tally &tally,
                                              bool &full)
@@ -720,7 +724,7 @@ __device__ __forceinline__ void work_subtile(const PassArgs &a, Queue *q, const 
         }
     }
     const unsigned left = __ballot_sync(0xffffffffu, record);
-    if (left) tally = by_record<LAYOUT, COHERENT, HALO>(a, q, node, left, tally);
+    if (left) tally = by_record<LAYOUT, HALO>(a, q, node, left, tally);
 }
 
 // Works windows w0, w0 + stride, ... (n of them).  Every thread of the block
@@ -846,8 +850,8 @@ __device__ __forceinline__ void run_windows(const PassArgs &a, const Block &blk,
         if (rest) continue;
         for (int sub = warp; sub < 4; sub += nwarps) {
             if (HALO && a.skip && ah->idle[i & 3][sub]) continue;
-            work_subtile<LAYOUT, BITS, EARLY, HALO>(a, blk.q, xy, blk.half, h,
-                                                    blk.rows + (TWO || two ? i & 1 : 0) * blk.rows_words, sub, tally,
+            work_subtile<LAYOUT, BITS, HALO>(a, blk.q, xy, blk.half, h,
+                                             blk.rows + (TWO || two ? i & 1 : 0) * blk.rows_words, sub, tally,
                                                     full);
         }
     }
@@ -976,7 +980,7 @@ __global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
         Tally tally{0u, 0u};
         bool full = false;  // (one window: the queue is worked off after it)
         for (int sub = warp; sub < 4; sub += nwarps)
-            work_subtile<LAYOUT, BITS, true, false>(a, blk.q, blk.xy, blk.half, h, blk.rows, sub, tally, full);
+            work_subtile<LAYOUT, BITS, false>(a, blk.q, blk.xy, blk.half, h, blk.rows, sub, tally, full);
         __syncthreads();
         if (blk.q->npending) tally = drain<LAYOUT, false>(a, blk.q, tally);
         flush(blk.q, a.stats + a.q, tally);
