@@ -136,6 +136,24 @@ struct Coords<1> {  // SoA: x[n] then y[n]
     }
 };
 
+// Interleaved coordinates in a caller's device buffer, which is aligned to its
+// doubles but perhaps not to pairs of them (a view at an odd offset): one
+// 16-byte access where it is (wide), else two of 8 bytes.
+inline bool pair_aligned(const void *p) { return ((uintptr_t)p & 15u) == 0u; }
+__device__ __forceinline__ double2 load_pair(const double *p, int64_t i, bool wide)
+{
+    return wide ? __ldg(reinterpret_cast<const double2 *>(p) + i) : make_double2(__ldg(p + 2 * i), __ldg(p + 2 * i + 1));
+}
+__device__ __forceinline__ void store_pair(double *p, int64_t i, double2 v, bool wide)
+{
+    if (wide) {
+        reinterpret_cast<double2 *>(p)[i] = v;
+    } else {
+        p[2 * i] = v.x;
+        p[2 * i + 1] = v.y;
+    }
+}
+
 // The same coordinates as raw 64-bit patterns.  Code that only moves or
 // inspects coordinates uses these, so no value is ever held in an FP64
 // register (the compiler copies FP64 registers with FP64-pipe instructions).

@@ -470,11 +470,11 @@ __global__ void copy_back_f32_kernel(const float *__restrict__ src, float *__res
 }
 
 // interleaved doubles -> floats in the mesh's layout (round to nearest)
-__global__ void narrow_kernel(const double2 *__restrict__ aos, float *dst, int64_t n, int layout)
+__global__ void narrow_kernel(const double *__restrict__ aos, float *dst, int64_t n, int layout, bool wide)
 {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const double2 v = __ldg(aos + i);
+        const double2 v = load_pair(aos, i, wide);
         const float x = __double2float_rn(v.x), y = __double2float_rn(v.y);
         if (layout == 0) {
             reinterpret_cast<float2 *>(dst)[i] = make_float2(x, y);
@@ -486,7 +486,7 @@ __global__ void narrow_kernel(const double2 *__restrict__ aos, float *dst, int64
 }
 
 // floats in the mesh's layout -> interleaved doubles (exact)
-__global__ void widen_kernel(const float *__restrict__ src, double2 *aos, int64_t n, int layout)
+__global__ void widen_kernel(const float *__restrict__ src, double *aos, int64_t n, int layout, bool wide)
 {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
@@ -499,7 +499,7 @@ __global__ void widen_kernel(const float *__restrict__ src, double2 *aos, int64_
             x = __ldg(src + i);
             y = __ldg(src + n + i);
         }
-        aos[i] = make_double2((double)x, (double)y);
+        store_pair(aos, i, make_double2((double)x, (double)y), wide);
     }
 }
 
@@ -544,13 +544,13 @@ cudaError_t launch_copy_back_f32(const float *src, float *dst, int64_t count, co
 
 cudaError_t launch_narrow(const double *aos, float *dst, int64_t n, int layout, int grid, cudaStream_t s)
 {
-    narrow_kernel<<<grid, 256, 0, s>>>(reinterpret_cast<const double2 *>(aos), dst, n, layout);
+    narrow_kernel<<<grid, 256, 0, s>>>(aos, dst, n, layout, pair_aligned(aos));
     return cudaGetLastError();
 }
 
 cudaError_t launch_widen(const float *src, double *aos, int64_t n, int layout, int grid, cudaStream_t s)
 {
-    widen_kernel<<<grid, 256, 0, s>>>(src, reinterpret_cast<double2 *>(aos), n, layout);
+    widen_kernel<<<grid, 256, 0, s>>>(src, aos, n, layout, pair_aligned(aos));
     return cudaGetLastError();
 }
 

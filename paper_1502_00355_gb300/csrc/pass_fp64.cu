@@ -183,18 +183,18 @@ __global__ void __launch_bounds__(256) histogram_kernel(const double *xy, int64_
         if (s_counts[b]) atomicAdd(&counts[b], (unsigned long long)s_counts[b]);
 }
 
-__global__ void soa_to_aos_kernel(const double *__restrict__ soa, double2 *__restrict__ aos, int64_t n)
+__global__ void soa_to_aos_kernel(const double *__restrict__ soa, double *__restrict__ aos, int64_t n, bool wide)
 {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-        aos[i] = make_double2(__ldg(soa + i), __ldg(soa + n + i));
+        store_pair(aos, i, make_double2(__ldg(soa + i), __ldg(soa + n + i)), wide);
 }
 
-__global__ void aos_to_soa_kernel(const double2 *__restrict__ aos, double *__restrict__ soa, int64_t n)
+__global__ void aos_to_soa_kernel(const double *__restrict__ aos, double *__restrict__ soa, int64_t n, bool wide)
 {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const double2 v = __ldg(aos + i);
+        const double2 v = load_pair(aos, i, wide);
         soa[i] = v.x;
         soa[n + i] = v.y;
     }
@@ -260,8 +260,8 @@ namespace {
 // of a domain-decomposed mesh); an id outside [0, n) sets *bad and is skipped.
 template <int LAYOUT>
 __global__ void gather_nodes_kernel(const double *__restrict__ xy, int64_t n, const int32_t *__restrict__ idx,
-                                    int64_t k, const uint32_t *__restrict__ inv, double2 *__restrict__ out,
-                                    unsigned *bad)
+                                    int64_t k, const uint32_t *__restrict__ inv, double *__restrict__ out,
+                                    bool wide, unsigned *bad)
 {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < k; t += stride) {
@@ -270,15 +270,15 @@ __global__ void gather_nodes_kernel(const double *__restrict__ xy, int64_t n, co
             atomicOr(bad, 1u);
             continue;
         }
-        out[t] = Coords<LAYOUT>::get(xy, n, inv ? (int64_t)__ldg(inv + i) : (int64_t)i);
+        store_pair(out, t, Coords<LAYOUT>::get(xy, n, inv ? (int64_t)__ldg(inv + i) : (int64_t)i), wide);
     }
 }
 
 // The listed nodes' coordinates written into both arrays of the ping-pong.
 template <int LAYOUT>
 __global__ void scatter_nodes_kernel(double *xy0, double *xy1, int64_t n, const int32_t *__restrict__ idx,
-                                     int64_t k, const uint32_t *__restrict__ inv, const double2 *__restrict__ in,
-                                     unsigned *bad)
+                                     int64_t k, const uint32_t *__restrict__ inv, const double *__restrict__ in,
+                                     bool wide, unsigned *bad)
 {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < k; t += stride) {
@@ -287,7 +287,7 @@ __global__ void scatter_nodes_kernel(double *xy0, double *xy1, int64_t n, const 
             atomicOr(bad, 1u);
             continue;
         }
-        const double2 v = __ldg(in + t);
+        const double2 v = load_pair(in, t, wide);
         const int64_t j = inv ? (int64_t)__ldg(inv + i) : (int64_t)i;
         Coords<LAYOUT>::put(xy0, n, j, v);
         Coords<LAYOUT>::put(xy1, n, j, v);
@@ -301,9 +301,9 @@ cudaError_t launch_gather_nodes(const double *xy, int layout, int64_t n, const i
 {
     if (k <= 0) return cudaSuccess;
     if (layout == 0)
-        gather_nodes_kernel<0><<<grid, 256, 0, s>>>(xy, n, idx, k, inv, reinterpret_cast<double2 *>(out), bad);
+        gather_nodes_kernel<0><<<grid, 256, 0, s>>>(xy, n, idx, k, inv, out, pair_aligned(out), bad);
     else
-        gather_nodes_kernel<1><<<grid, 256, 0, s>>>(xy, n, idx, k, inv, reinterpret_cast<double2 *>(out), bad);
+        gather_nodes_kernel<1><<<grid, 256, 0, s>>>(xy, n, idx, k, inv, out, pair_aligned(out), bad);
     return cudaGetLastError();
 }
 
@@ -311,11 +311,10 @@ cudaError_t launch_scatter_nodes(double *xy0, double *xy1, int layout, int64_t n
                                  const uint32_t *inv, const double *in, unsigned *bad, int grid, cudaStream_t s)
 {
     if (k <= 0) return cudaSuccess;
-    const double2 *v = reinterpret_cast<const double2 *>(in);
     if (layout == 0)
-        scatter_nodes_kernel<0><<<grid, 256, 0, s>>>(xy0, xy1, n, idx, k, inv, v, bad);
+        scatter_nodes_kernel<0><<<grid, 256, 0, s>>>(xy0, xy1, n, idx, k, inv, in, pair_aligned(in), bad);
     else
-        scatter_nodes_kernel<1><<<grid, 256, 0, s>>>(xy0, xy1, n, idx, k, inv, v, bad);
+        scatter_nodes_kernel<1><<<grid, 256, 0, s>>>(xy0, xy1, n, idx, k, inv, in, pair_aligned(in), bad);
     return cudaGetLastError();
 }
 
@@ -367,24 +366,24 @@ __global__ void permute_kernel(const T *__restrict__ src, T *__restrict__ dst, i
 // dst (interleaved doubles, the caller's numbering)[perm[k]] = src[k] (exact widening of floats)
 template <class T, int LAYOUT>
 __global__ void unpermute_to_aos_kernel(const T *__restrict__ src, int64_t n, const uint32_t *__restrict__ perm,
-                                        double2 *__restrict__ dst)
+                                        double *__restrict__ dst, bool wide)
 {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += stride) {
         T x, y;
         Pair<T, LAYOUT>::get(src, n, k, x, y);
-        dst[perm[k]] = make_double2((double)x, (double)y);
+        store_pair(dst, perm[k], make_double2((double)x, (double)y), wide);
     }
 }
 
 // dst[k] = src (interleaved doubles, the caller's numbering)[perm[k]], rounded to T
 template <class T, int LAYOUT>
-__global__ void permute_from_aos_kernel(const double2 *__restrict__ src, int64_t n, const uint32_t *__restrict__ perm,
-                                        T *__restrict__ dst)
+__global__ void permute_from_aos_kernel(const double *__restrict__ src, int64_t n, const uint32_t *__restrict__ perm,
+                                        T *__restrict__ dst, bool wide)
 {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += stride) {
-        const double2 v = src[perm[k]];
+        const double2 v = load_pair(src, perm[k], wide);
         Pair<T, LAYOUT>::put(dst, n, k, (T)v.x, (T)v.y);
     }
 }
@@ -418,14 +417,15 @@ cudaError_t launch_unpermute_to_aos(const double *src, int layout, bool f32, int
                                     double *dst_aos, int grid, cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
-    double2 *d = reinterpret_cast<double2 *>(dst_aos);
+    double *d = dst_aos;
+    const bool w = pair_aligned(d);
     if (f32) {
         const float *f = reinterpret_cast<const float *>(src);
-        if (layout == 0) unpermute_to_aos_kernel<float, 0><<<grid, 256, 0, s>>>(f, n, perm, d);
-        else unpermute_to_aos_kernel<float, 1><<<grid, 256, 0, s>>>(f, n, perm, d);
+        if (layout == 0) unpermute_to_aos_kernel<float, 0><<<grid, 256, 0, s>>>(f, n, perm, d, w);
+        else unpermute_to_aos_kernel<float, 1><<<grid, 256, 0, s>>>(f, n, perm, d, w);
     } else {
-        if (layout == 0) unpermute_to_aos_kernel<double, 0><<<grid, 256, 0, s>>>(src, n, perm, d);
-        else unpermute_to_aos_kernel<double, 1><<<grid, 256, 0, s>>>(src, n, perm, d);
+        if (layout == 0) unpermute_to_aos_kernel<double, 0><<<grid, 256, 0, s>>>(src, n, perm, d, w);
+        else unpermute_to_aos_kernel<double, 1><<<grid, 256, 0, s>>>(src, n, perm, d, w);
     }
     return cudaGetLastError();
 }
@@ -434,14 +434,15 @@ cudaError_t launch_permute_from_aos(const double *src_aos, int layout, bool f32,
                                     double *dst, int grid, cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
-    const double2 *v = reinterpret_cast<const double2 *>(src_aos);
+    const double *v = src_aos;
+    const bool w = pair_aligned(v);
     if (f32) {
         float *f = reinterpret_cast<float *>(dst);
-        if (layout == 0) permute_from_aos_kernel<float, 0><<<grid, 256, 0, s>>>(v, n, perm, f);
-        else permute_from_aos_kernel<float, 1><<<grid, 256, 0, s>>>(v, n, perm, f);
+        if (layout == 0) permute_from_aos_kernel<float, 0><<<grid, 256, 0, s>>>(v, n, perm, f, w);
+        else permute_from_aos_kernel<float, 1><<<grid, 256, 0, s>>>(v, n, perm, f, w);
     } else {
-        if (layout == 0) permute_from_aos_kernel<double, 0><<<grid, 256, 0, s>>>(v, n, perm, dst);
-        else permute_from_aos_kernel<double, 1><<<grid, 256, 0, s>>>(v, n, perm, dst);
+        if (layout == 0) permute_from_aos_kernel<double, 0><<<grid, 256, 0, s>>>(v, n, perm, dst, w);
+        else permute_from_aos_kernel<double, 1><<<grid, 256, 0, s>>>(v, n, perm, dst, w);
     }
     return cudaGetLastError();
 }
@@ -456,13 +457,13 @@ cudaError_t launch_unpermute_u8(const uint8_t *src, int64_t n, const uint32_t *p
 
 cudaError_t launch_soa_to_aos(const double *soa, double *aos, int64_t n, int grid, cudaStream_t s)
 {
-    soa_to_aos_kernel<<<grid, 256, 0, s>>>(soa, reinterpret_cast<double2 *>(aos), n);
+    soa_to_aos_kernel<<<grid, 256, 0, s>>>(soa, aos, n, pair_aligned(aos));
     return cudaGetLastError();
 }
 
 cudaError_t launch_aos_to_soa(const double *aos, double *soa, int64_t n, int grid, cudaStream_t s)
 {
-    aos_to_soa_kernel<<<grid, 256, 0, s>>>(reinterpret_cast<const double2 *>(aos), soa, n);
+    aos_to_soa_kernel<<<grid, 256, 0, s>>>(aos, soa, n, pair_aligned(aos));
     return cudaGetLastError();
 }
 
