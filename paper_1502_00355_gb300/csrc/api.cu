@@ -182,6 +182,16 @@ sls_status sls_smooth(sls_mesh *M, int32_t max_iter, double tol_rel, sls_info *i
     return SLS_OK;
 }
 
+// For the tests, not declared in the header: the poll limit of the mesh's next
+// launch that runs several passes (so that a wait between its blocks runs
+// out).  SLS_ERR_INVALID when the mesh's passes are launched one by one.
+sls_status sls_test_resident(sls_mesh *M, uint32_t polls)
+{
+    if (!M || !M->resident) return fail(SLS_ERR_INVALID, "not a mesh whose passes share one launch");
+    M->next_polls = polls;
+    return SLS_OK;
+}
+
 sls_status sls_get_coords(const sls_mesh *M, double *xy_out, int32_t dst_is_device)
 {
     if (!M || !xy_out) return fail(SLS_ERR_INVALID, "mesh and xy_out must not be NULL");

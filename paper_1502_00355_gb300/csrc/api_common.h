@@ -69,6 +69,7 @@ struct sls_mesh {
     unsigned *xfer_bad = nullptr; // gather/scatter: set when an id was out of range
     int block = 256, grid = 0;
     bool resident = false;        // all passes of a call in one launch (pass_screened.cu)
+    unsigned next_polls = 0u;     // poll limit of the next such launch; 0 = kPollLimit (sls_test_resident)
     bool screened = true;         // screened kernel (else the plain FP64 kernel)
     sls_info last{};
 };

@@ -24,12 +24,16 @@ int pass_screened_occupancy(int layout, int block, const WindowShape &shape);
 // Passes a.q .. a.q + passes - 1 of a mesh with at most one window per resident
 // block (resident_fits), in one cooperative launch that stops at the
 // tolerance like separate ones; the passes ping-pong between a.in and a.out.
-// barrier: kBarrierWords device words, zero at the launch; word 1 is set when a
-// wait between the blocks ran out, and the passes are then incomplete.
+// barrier: kBarrierWords device words, 8-byte aligned; word 0 zero at the launch,
+// word 1 at the call's first.  Word 1 is set when a wait between the blocks ran
+// out (poll_limit polls): the passes are then incomplete, and further launches
+// with it set do nothing.
 constexpr int kBarrierWords = 2;
+// A poll takes about a microsecond; a pass of such a mesh some tens of them.
+constexpr unsigned kPollLimit = 1u << 22;
 bool resident_fits(const PassArgs &a, int layout, int block, const WindowShape &shape);
 cudaError_t launch_resident(const PassArgs &a, int layout, int block, const WindowShape &shape, int passes,
-                            unsigned *barrier, cudaStream_t s);
+                            unsigned *barrier, unsigned poll_limit, cudaStream_t s);
 
 // One round of the batched / served form over all active jobs' tasks.
 // chunk > 0: tasks per block chunk, taken in a grid stride; chunk < 0: chunks

@@ -328,9 +328,10 @@ sls_status mesh_run(sls_mesh *M, int32_t max_iter, double tol_rel, sls_info &inf
             a.in = M->xy[M->cur ^ (launched & 1)];
             a.out = M->xy[M->cur ^ (launched & 1) ^ 1];
             if (launched > 0)
-                SLS_CUDA_TRY(cudaMemsetAsync(barrier, 0, sizeof(unsigned) * kBarrierWords, M->stream), "cudaMemset");
+                SLS_CUDA_TRY(cudaMemsetAsync(barrier, 0, sizeof(unsigned), M->stream), "cudaMemset");
             SLS_CUDA_TRY(launch_resident(a, M->opt.layout, M->block, M->windows.shape, end - launched, barrier,
-                                         M->stream), "pass kernel");
+                                         M->next_polls ? M->next_polls : kPollLimit, M->stream), "pass kernel");
+            M->next_polls = 0u;
             ++kernels;
         }
         for (int q = launched; q < end && !M->resident; ++q) {

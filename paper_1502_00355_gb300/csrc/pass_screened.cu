@@ -899,29 +899,35 @@ __global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
 // resident block (about 136,000 nodes) the blocks would have to fetch their
 // lists again every pass, as separate launches do.
 
-struct GridBarrier {
+struct __align__(8) GridBarrier {
     unsigned int arrived;  // blocks that arrived, over all passes of the launch
-    unsigned int lost;     // a wait ran out: nobody waits any more
+    unsigned int lost;     // a wait ran out: nobody waits or computes any more, in this launch or in a
+                           // later one of the call (the call's end reads it)
 };
 
-// Polls before a waiting block gives up (a poll takes about a microsecond; a
-// pass of such a mesh some tens of them).
-constexpr unsigned kPollLimit = 1u << 22;
+__device__ __forceinline__ unsigned long long barrier_words(GridBarrier *b)
+{
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(b) : "memory");
+    return v;  // arrived, lost << 32
+}
 
-// All threads call it; false when some block's wait ran out.  Writes to global
-// memory before it are visible after it to reads from L2.
-__device__ __forceinline__ bool grid_barrier(GridBarrier *b, unsigned target)
+// All threads call it; false when some block's wait ran out (after `limit`
+// polls).  Writes to global memory before it are visible after it to reads
+// from L2.
+__device__ __forceinline__ bool grid_barrier(GridBarrier *b, unsigned target, unsigned limit)
 {
     __shared__ bool s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         atomicAdd(&b->arrived, 1u);
-        unsigned seen = 0u, polls = 0u;
+        unsigned long long seen = 0ull;
+        unsigned polls = 0u;
         do {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&b->arrived) : "memory");
-        } while (seen < target && ++polls < kPollLimit);
-        s_ok = seen >= target;
+            seen = barrier_words(b);
+        } while ((unsigned)seen < target && (seen >> 32) == 0ull && ++polls < limit);
+        s_ok = (unsigned)seen >= target && (seen >> 32) == 0ull;
         if (!s_ok) atomicExch(&b->lost, 1u);
     }
     __syncthreads();
@@ -931,7 +937,7 @@ __device__ __forceinline__ bool grid_barrier(GridBarrier *b, unsigned target)
 template <int LAYOUT, int BITS>
 __global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
     resident_kernel(const __grid_constant__ PassArgs a0, const __grid_constant__ WindowShape shape, int passes,
-                    GridBarrier *barrier)
+                    GridBarrier *barrier, unsigned poll_limit)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ PassArgs s_args;
@@ -940,7 +946,7 @@ __global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
     const Block blk = block_memory<BITS == 8>(smem_raw, shape);
     if (tid == 0) {
         s_args = a0;
-        s_stop = pass_is_skipped(a0.stats, a0.q, a0.tol_active, a0.thr_bits);
+        s_stop = pass_is_skipped(a0.stats, a0.q, a0.tol_active, a0.thr_bits) || (barrier_words(barrier) >> 32) != 0ull;
     }
     // the window's header, halo ids and lists, once
     uint32_t *h = blk.ahead->hdr[0];
@@ -991,7 +997,7 @@ __global__ void __launch_bounds__(kBlockMax, kBlocksPerSm)
             s_args.out = (done & 1) ? const_cast<double *>(a0.in) : a0.out;
             s_args.q += 1;
         }
-        if (!grid_barrier(barrier, (unsigned)done * gridDim.x)) return;
+        if (!grid_barrier(barrier, (unsigned)done * gridDim.x, poll_limit)) return;
     }
 }
 
@@ -1183,13 +1189,13 @@ bool resident_fits(const PassArgs &a, int layout, int block, const WindowShape &
 }
 
 cudaError_t launch_resident(const PassArgs &a, int layout, int block, const WindowShape &shape, int passes,
-                            unsigned *barrier, cudaStream_t s)
+                            unsigned *barrier, unsigned poll_limit, cudaStream_t s)
 {
     static_assert(sizeof(GridBarrier) == kBarrierWords * sizeof(unsigned), "barrier words");
     cudaError_t e = ensure_constants();
     if (e != cudaSuccess) return e;
     GridBarrier *b = reinterpret_cast<GridBarrier *>(barrier);
-    void *args[] = {const_cast<PassArgs *>(&a), const_cast<WindowShape *>(&shape), &passes, &b};
+    void *args[] = {const_cast<PassArgs *>(&a), const_cast<WindowShape *>(&shape), &passes, &b, &poll_limit};
     return cudaLaunchCooperativeKernel(resident_kernel_of(layout, shape.bits), dim3((unsigned)a.win_count), dim3(block),
                                        args, smem_for(shape), s);
 }
