@@ -182,13 +182,18 @@ sls_status sls_smooth(sls_mesh *M, int32_t max_iter, double tol_rel, sls_info *i
     return SLS_OK;
 }
 
-// For the tests, not declared in the header: the poll limit of the mesh's next
-// launch that runs several passes (so that a wait between its blocks runs
-// out).  SLS_ERR_INVALID when the mesh's passes are launched one by one.
+// For the tests, not declared in the header.  polls > 0: the poll limit of the
+// mesh's next launch that runs several passes (so that a wait between its
+// blocks runs out); 0: such a launch is tried next although the mesh is too
+// large for it (the driver refuses it).  SLS_ERR_INVALID when the mesh's passes
+// could not share a launch at any size, or (polls > 0) do not.
 sls_status sls_test_resident(sls_mesh *M, uint32_t polls)
 {
-    if (!M || !M->resident) return fail(SLS_ERR_INVALID, "not a mesh whose passes share one launch");
+    if (!M || !M->screened || M->opt.form != 0 || M->opt.copy_back || M->opt.skip_unchanged || M->opt.l2_window ||
+        (polls && !M->resident))
+        return fail(SLS_ERR_INVALID, "not a mesh whose passes share one launch");
     M->next_polls = polls;
+    M->resident = true;
     return SLS_OK;
 }
 

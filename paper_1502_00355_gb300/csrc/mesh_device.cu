@@ -315,25 +315,35 @@ sls_status mesh_run(sls_mesh *M, int32_t max_iter, double tol_rel, sls_info &inf
     const bool form_b = M->opt.form == 1;
     const int cb = form_b ? 0 : M->opt.copy_back;
     unsigned *const barrier = reinterpret_cast<unsigned *>(M->stats - 1);
-    // the resident form stops at the tolerance by itself; between its launches
-    // other work gets its turn
-    const int chunk = M->resident ? kResidentPasses : M->opt.passes_per_check;
     const int nseg = (int)M->colour_off.size() - 1;
     int launched = 0;
     int64_t kernels = 0;
     while (launched < max_iter) {
-        const int end = std::min(launched + chunk, (int)max_iter);
+        int end = launched;
         if (M->resident) {
+            // this form stops at the tolerance by itself; between its launches
+            // other work gets its turn
+            end = std::min(launched + kResidentPasses, (int)max_iter);
             a.q = launched;
             a.in = M->xy[M->cur ^ (launched & 1)];
             a.out = M->xy[M->cur ^ (launched & 1) ^ 1];
             if (launched > 0)
                 SLS_CUDA_TRY(cudaMemsetAsync(barrier, 0, sizeof(unsigned), M->stream), "cudaMemset");
-            SLS_CUDA_TRY(launch_resident(a, M->opt.layout, M->block, M->windows.shape, end - launched, barrier,
-                                         M->next_polls ? M->next_polls : kPollLimit, M->stream), "pass kernel");
+            const cudaError_t e = launch_resident(a, M->opt.layout, M->block, M->windows.shape, end - launched, barrier,
+                                                  M->next_polls ? M->next_polls : kPollLimit, M->stream);
             M->next_polls = 0u;
-            ++kernels;
+            if (e == cudaErrorCooperativeLaunchTooLarge) {
+                // not all blocks can be resident together after all (the device's
+                // SMs are counted, of which this process may have a share): a
+                // launch for each pass, from now on
+                cudaGetLastError();
+                M->resident = false;
+            } else {
+                SLS_CUDA_TRY(e, "pass kernel");
+                ++kernels;
+            }
         }
+        if (!M->resident) end = std::min(launched + M->opt.passes_per_check, (int)max_iter);
         for (int q = launched; q < end && !M->resident; ++q) {
             a.q = q;
             if (form_b) {

@@ -42,3 +42,48 @@ def test_a_wait_that_runs_out(sls, layout, passes, tol):
         want, winfo, _ = oracle.OracleMesh(mesh.xy, mesh.tri, mesh.boundary).smooth(mesh.xy, 20)
         assert np.array_equal(g.coords(), want) and info["accepted_last"] == winfo["accepted_last"]
         assert info["launches"] == 1
+
+
+@pytest.mark.parametrize("numbering", ["morton", "random"])
+@pytest.mark.parametrize("passes, tol", [(37, 0.0), (200, 1e-4)])
+def test_a_refused_launch_falls_back(sls, numbering, passes, tol):
+    # more windows than blocks can be resident together: the driver refuses the
+    # cooperative launch, and the passes are launched one by one
+    mesh = meshgen.jittered_grid(601, 457, 0.35, 62, numbering=numbering)
+    want, winfo, wacc = oracle.OracleMesh(mesh.xy, mesh.tri, mesh.boundary, openmp=True).smooth(mesh.xy, passes, tol=tol)
+    with sls.Mesh(mesh.xy, mesh.tri, mesh.boundary, record_accept=True) as g:
+        assert sls.lib().sls_test_resident(g.handle, 0) == 0
+        for _ in range(2):
+            g.set_coords(mesh.xy)
+            info = g.smooth(passes, tol)
+            assert np.array_equal(g.coords(), want) and np.array_equal(g.accept_mask(), wacc)
+            for key in ("iterations", "converged", "accepted_last", "maxd2_last"):
+                assert info[key] == winfo[key], key
+            assert info["launches"] >= winfo["iterations"]
+
+
+def test_two_such_meshes_at_once(sls):
+    # two threads, each with a mesh that fills the GPU's resident blocks: the
+    # launches cannot run side by side and must not wait for each other's blocks
+    import threading
+    mesh = meshgen.jittered_grid(421, 311, 0.35, 63)
+    want, _, _ = oracle.OracleMesh(mesh.xy, mesh.tri, mesh.boundary, openmp=True).smooth(mesh.xy, 25)
+    bad = []
+
+    def work():
+        try:
+            with sls.Mesh(mesh.xy, mesh.tri, mesh.boundary) as g:
+                for _ in range(20):
+                    g.set_coords(mesh.xy)
+                    info = g.smooth(25)
+                    if info["launches"] != 1 or not np.array_equal(g.coords(), want):
+                        bad.append(info)
+        except Exception as e:  # noqa: BLE001 (reported by the main thread)
+            bad.append(e)
+
+    threads = [threading.Thread(target=work) for _ in range(3)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join(120.0)
+    assert not bad and not any(t.is_alive() for t in threads)
