@@ -84,7 +84,8 @@ int device_sm_count();
 unsigned long long current_context_id();
 // Loads the allocation-free entry point's scratch array on the current
 // device (noalloc.cu); sls_mesh_create calls it, so sls_smooth_noalloc on a
-// mesh never loads code or data itself.
+// mesh never loads code or data itself (a renumbered mesh's creation loads the
+// kernels of its numbering too, load_numbering_kernels).
 sls_status noalloc_prepare();
 sls_options resolve_options(const sls_options *opt);
 sls_status check_options(const sls_options &o);

@@ -95,6 +95,9 @@ cudaError_t launch_unpermute_to_aos(const double *src, int layout, bool f32, int
 // dst[k] = src_aos (interleaved doubles, the caller's numbering)[perm[k]], rounded to floats with f32
 cudaError_t launch_permute_from_aos(const double *src_aos, int layout, bool f32, int64_t n, const uint32_t *perm,
                                     double *dst, int grid, cudaStream_t s);
+// Loads the kernels with which the allocation-free form maps the coordinates
+// of a renumbered mesh, which may not load code itself.
+cudaError_t load_numbering_kernels();
 // dst[perm[k]] = src[k]
 cudaError_t launch_unpermute_u8(const uint8_t *src, int64_t n, const uint32_t *perm, uint8_t *dst, int grid,
                                 cudaStream_t s);

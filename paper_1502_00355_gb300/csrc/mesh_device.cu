@@ -113,6 +113,9 @@ static sls_status finish_creation(sls_mesh *M)
                       resident_fits(a, M->opt.layout, M->block, M->windows.shape);
     }
     if ((st = build_tile_halo(M, M->stream)) != SLS_OK) return st;
+    // (noalloc_prepare: a renumbered mesh's call needs two kernels more)
+    if (M->perm && M->opt.layout == 0 && !M->f32 && M->opt.form == 0)
+        SLS_CUDA_TRY(load_numbering_kernels(), "mesh create");
     // a batch or the allocation-free form runs the mesh on other streams
     SLS_CUDA_TRY(cudaStreamSynchronize(M->stream), "mesh create");
     return SLS_OK;

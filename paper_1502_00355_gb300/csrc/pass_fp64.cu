@@ -430,6 +430,14 @@ cudaError_t launch_unpermute_to_aos(const double *src, int layout, bool f32, int
     return cudaGetLastError();
 }
 
+cudaError_t load_numbering_kernels()
+{
+    cudaFuncAttributes a;
+    cudaError_t e = cudaFuncGetAttributes(&a, (const void *)permute_kernel<double, 0>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, (const void *)unpermute_to_aos_kernel<double, 0>);
+    return e;
+}
+
 cudaError_t launch_permute_from_aos(const double *src_aos, int layout, bool f32, int64_t n, const uint32_t *perm,
                                     double *dst, int grid, cudaStream_t s)
 {
