@@ -96,7 +96,10 @@ SLS_SC_HD float trunc_float(unsigned long long b)
 // Screening constants (unit roundoff e = 2^-24).  A local coordinate of a
 // neighbour carries an error below 2e|X| + 2^-44 M (head/tail truncation; M
 // bounds the node's coordinate magnitude plus the ring's extent), which is
-// below 3e R wherever R >= 2^-20 M; the screen requires that.  The centre's
+// below 3e R for one R at least as large as every local coordinate of the ring
+// wherever R >= 2^-20 M; the screen requires that of the furthest neighbour's
+// (frame_ok).  How near other neighbours are does not matter: their error is
+// measured against R, and so is the bound.  The centre's
 // local coordinate is within 2e of its exact value (relative).  For a
 // triangle whose three vertices' local coordinates are bounded by R, with
 // g = R^2 / s (s the computed sum of squared edges), the FP32 alpha differs
@@ -117,6 +120,10 @@ constexpr float kGMax = 1000.0f;
 constexpr float kTwoSqrt3f = 3.46410161514f;
 constexpr float kLocalRange = 1048576.0f;  // 2^20: R * 2^20 >= M keeps the head/tail error below e R
 
+// (local_offset, screen_alpha, edge_ba2 and bound_ok are the screen of one
+// triangle by itself, from which the constants above are derived.  The pass uses
+// the ring form below; the CPU tests pin the constants with both.)
+
 // Offset of a neighbour (bit patterns bx, by) from the node whose head/tail
 // splits are (phx, plx), (phy, ply); ok &= both splits are valid.
 SLS_SC_HD void local_offset(unsigned long long bx, unsigned long long by, float phx, float plx, float phy,
@@ -128,17 +135,16 @@ SLS_SC_HD void local_offset(unsigned long long bx, unsigned long long by, float 
     Ly = (hy - phy) + (ly - ply);
 }
 
-// Whether the local frame of a node is usable: rmin / rmax the smallest and
-// largest local coordinate magnitude of its neighbours (largest including the
-// centre's offset), M bounding the node's coordinate magnitude plus rmax.
-SLS_SC_HD bool frame_ok(float rmin, float rmax, float M)
+// Whether the local frame of a node is usable: rn the largest local coordinate
+// magnitude of its neighbours, rN the larger of it and the centre's, M bounding
+// the node's coordinate magnitude plus rN.  (A smaller rn asks for more.)
+SLS_SC_HD bool frame_ok(float rn, float rN, float M)
 {
-    return (rmin >= 1e-14f) & (rmax <= 1e15f) & (rmin * kLocalRange >= M);
+    return (rn >= 1e-14f) & (rN <= 1e15f) & (rn * kLocalRange >= M);
 }
 
 // FP32 alpha of the triangle (X, A, B) for the screen (sk: orientation sign
-// times 2 sqrt(3); ba2 = |B - A|^2); sv receives the edge sum.  The second
-// candidate loop of the kernel calls it again and gets the same bits.
+// times 2 sqrt(3); ba2 = |B - A|^2); sv receives the edge sum.
 SLS_SC_HD float screen_alpha(float Xx, float Xy, float Ax, float Ay, float Bx, float By, float ba2, float sk,
                              float &sv)
 {
