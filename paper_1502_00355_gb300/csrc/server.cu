@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "api_common.h"
+#include "footprint.h"
 #include "kernels.h"
 
 using namespace sls;
@@ -225,26 +226,7 @@ struct sls_server {
 
 namespace {
 
-// Device bytes a job holds once built: two coordinate arrays, node offsets,
-// adjacency words, the window stream, the numbering map, one statistics
-// record per pass.
-size_t built_footprint(int64_t n, uint64_t adj_words, size_t stream_bytes, int32_t max_iter)
-{
-    return 2 * sizeof(double) * 2 * (size_t)n + sizeof(uint32_t) * (size_t)(n + 1) + sizeof(uint32_t) * adj_words +
-           stream_bytes + sizeof(uint32_t) * (size_t)n + sizeof(PassStats) * (size_t)std::max(1, max_iter);
-}
-
-// A bound on what a job holds while it is built: the built footprint with
-// at most n + 9m adjacency words (a meta word per node; per corner of a
-// triangle at most two neighbours and one triangle code) and a window stream
-// whose every subtile has rings of the longest kind and whose every
-// neighbour is in a halo, plus the build's scratch (triangles, incidences,
-// neighbour candidates, counts and flags).
-size_t admission_bound(int64_t n, int64_t m, int32_t max_iter)
-{
-    return built_footprint(n, (uint64_t)(n + 9 * m), 76 * (size_t)n + 24 * (size_t)m, max_iter) + 74 * (size_t)n +
-           48 * (size_t)m + 65536;
-}
+size_t stats_bytes(int32_t max_iter) { return sizeof(PassStats) * (size_t)std::max(1, max_iter); }
 
 void fail_job(sls_server *S, ServerJob &J, sls_status st, const std::string &msg)
 {
@@ -341,7 +323,7 @@ sls_status build_job(ServerJob &J, bool group, bool numbers, cudaStream_t s, siz
     if (e == cudaSuccess) e = cudaEventRecord(J.uploaded, s);
     if (e != cudaSuccess) return cuda_err(e, "build");
     *footprint = built_footprint(n, da.adj_words,
-                                 J.windows.rows_bytes + 32 * (size_t)J.windows.count, J.max_iter);
+                                 J.windows.rows_bytes + 32 * (size_t)J.windows.count, stats_bytes(J.max_iter));
     return SLS_OK;
 }
 
@@ -850,7 +832,7 @@ sls_status sls_submit(sls_server *S, const double *xy, int64_t n, const int32_t 
     J->m = m;
     J->max_iter = max_iter;
     J->tol = tol_rel;
-    J->reserved = admission_bound(n, m, max_iter);
+    J->reserved = admission_bound(n, m, stats_bytes(max_iter));
     std::lock_guard<std::mutex> lk(S->mu);
     J->id = S->next_id++;
     S->jobs[J->id] = J;
