@@ -28,7 +28,9 @@
 //     (no cancellation) and decides all but rounding-level ties.
 //  7. What is left goes to the block's queue: one item per quality to be
 //     evaluated in FP64, with the coordinates it needs, so that full warps
-//     evaluate independent items side by side on the narrow FP64 pipe.
+//     evaluate independent items side by side on the narrow FP64 pipe.  A warp
+//     most of whose nodes are left, or that finds the queue full, looks closer
+//     and evaluates its items itself, 32 at a time.
 //
 // Coordinates are moved as 64-bit patterns, never held in FP64 registers
 // unless they take part in FP64 arithmetic: the compiler copies FP64
@@ -364,27 +366,259 @@ __device__ __noinline__ Minima walk_irregular(RingWalk w, uint32_t l, const uint
     return walk_ring<true, BITS>(w, l, list);
 }
 
+// Writes a node that a screen has decided; the centre differs from it.
+template <int LAYOUT>
+__device__ __forceinline__ void finish_screened(const PassArgs &a, Queue *q, int32_t node, bool accept, ulonglong2 p,
+                                                ulonglong2 c, float Cx, float Cy)
+{
+    if (accept) {
+        // the exact squared move is needed only where it can be the block's
+        // largest: the screen's offset gives it to within a few units of 2^-24
+        const float about = fmaf(Cx, Cx, Cy * Cy) * 1.000001f + 1e-37f;
+        if (about >= *const_cast<volatile float *>(&q->best_low)) {
+            const double dx = __dsub_rn(bitsd(c.x), bitsd(p.x)), dy = __dsub_rn(bitsd(c.y), bitsd(p.y));
+            note_move(q, dbits(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy))));
+        }
+    }
+    CoordBits<LAYOUT>::put(a.out, a.n, node, accept ? c : p);
+    if (a.accept) a.accept[node] = accept ? 1 : 0;
+}
+
+// Position of bit number k (from 0) of the set bits of m.
+__device__ __forceinline__ uint32_t set_bit(unsigned m, uint32_t k)
+{
+    uint32_t at = 0u;
+#pragma unroll
+    for (uint32_t w = 16u; w > 0u; w >>= 1) {
+        const uint32_t below = __popc(m & ((1u << w) - 1u));
+        if (k >= below) {
+            k -= below;
+            m >>= w;
+            at += w;
+        }
+    }
+    return at;
+}
+
+// A quality as a signed integer of the same order (-0 below +0, which no
+// comparison of the minima sees: they are compared as doubles).
+__device__ __forceinline__ long long quality_key(double q)
+{
+    const long long b = __double_as_longlong(q);
+    return b < 0 ? b ^ 0x7fffffffffffffffll : b;
+}
+__device__ __forceinline__ double key_quality(long long k)
+{
+    return __longlong_as_double(k < 0 ? k ^ 0x7fffffffffffffffll : k);
+}
+
+// FP32 offset of the centre from the node (relative error below 2^-23).  With
+// equal sign and exponent field the difference is a whole number of units in
+// the last place; otherwise one FP64 subtraction.
+__device__ __forceinline__ void offset_of(ulonglong2 c, ulonglong2 p, float &Cx, float &Cy)
+{
+    const uint32_t hx = (uint32_t)(p.x >> 32), hy = (uint32_t)(p.y >> 32);
+    const uint32_t ex = (hx >> 20) & 0x7ffu, ey = (hy >> 20) & 0x7ffu;
+    const uint32_t other = ((uint32_t)((c.x ^ p.x) >> 32) | (uint32_t)((c.y ^ p.y) >> 32)) & 0xfff00000u;
+    if (other == 0u && ex - 949u <= 200u && ey - 949u <= 200u) {
+        // unit in the last place, with the sign of the coordinate
+        const float ux = __uint_as_float((hx & 0x80000000u) | ((ex - 948u) << 23));
+        const float uy = __uint_as_float((hy & 0x80000000u) | ((ey - 948u) << 23));
+        Cx = __ll2float_rn((long long)(c.x - p.x)) * ux;
+        Cy = __ll2float_rn((long long)(c.y - p.y)) * uy;
+    } else {
+        Cx = trunc_float(dbits(__dsub_rn(bitsd(c.x), bitsd(p.x))));
+        Cy = trunc_float(dbits(__dsub_rn(bitsd(c.y), bitsd(p.y))));
+    }
+}
+
+// Decides the open nodes of a warp (mask) without the queue: those for which it
+// has no room, or all of a warp with many.  For each node, lane t looks at step t
+// before the move and lane 16 + t after it.  First the screen again, closer: each
+// side with its own radius, edge sums and largest quality (the walk has one bound
+// for both sides and all qualities), and without the steps' numbers.  A node still
+// open has the steps that can attain a side's minimum evaluated in FP64, 32 at a
+// time from as many nodes as it takes: a node by itself would leave most lanes of
+// the narrow FP64 pipe idle.  Returns per lane 1 accepted, 2 moved.
+//
+// What bounds it: the FP64 pipe (46 operations an item).  Meshes most of whose
+// nodes are open, 1009 x 701 nodes, us a pass: flattened to 1e-3 of their height
+// 237, to 1e-5 921, 1e5 away from the origin 907, rows graded by 1e6 335; a node
+// at a time and without the closer screen 689, 1706, 1683, 662; one thread per node
+// gathering for itself 319, 1274, 1159, 470.
+//
+// It holds little and finds again what it can (offsets, a node that has to wait
+// for the next 32 items; one register for the lane's counts): the pass's own loop
+// has to do without the registers that it takes, and spills (2% of every mesh's
+// pass when it kept them).
+template <int LAYOUT, int BITS>
+__device__ __noinline__ uint32_t settle_open(const PassArgs &a, Queue *q, const char *xy, uint32_t half,
+                                             const uint32_t *list, uint32_t cold, bool irregular, int32_t node,
+                                             ulonglong2 c, uint32_t meta0, unsigned mask)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    // the lane's state: bits 0..4 and 5..9 its item's node (by lane) and step (bit 9:
+    // after the move); of its own node among the items held: 10..14 the first, 15..19
+    // how many, 20..23 of those before the move; 24 accepted, 25 moved
+    uint32_t state = 0u;
+    uint32_t fill = 0u;  // items held
+    do {
+        bool evaluate = mask == 0u;
+        if (mask) {
+            const uint32_t src = (uint32_t)__ffs((int)mask) - 1u, t = lane & 15u;
+            const bool after = lane >= 16u;
+            const uint32_t meta = __shfl_sync(0xffffffffu, meta0, src), own = (win::meta_place(meta) + 1u) * 16u;
+            float Cx, Cy;
+            {
+                ulonglong2 cs;
+                cs.x = __shfl_sync(0xffffffffu, c.x, src);
+                cs.y = __shfl_sync(0xffffffffu, c.y, src);
+                offset_of(cs, *reinterpret_cast<const ulonglong2 *>(xy + own), Cx, Cy);
+            }
+            const float4 h = *reinterpret_cast<const float4 *>(xy + half + own);
+            bool step = false;
+            float v = FLT_MAX, s = FLT_MAX;  // cross / s and s of the lane's step and side
+            float rn = 0.0f, sgn = 1.0f;
+            RingVertex P, Q;
+            P.x = P.y = Q.x = Q.y = 0.0f;
+            if (t < win::meta_steps(meta)) {
+                const uint32_t *ring = list + (int)src - (int)lane;
+                const float4 hP = *reinterpret_cast<const float4 *>(xy + half + List<BITS>::at(ring, t));
+                const float4 hQ = *reinterpret_cast<const float4 *>(xy + half + List<BITS>::at(ring, t + 1u));
+                P = ring_vertex(hP.x, hP.y, hP.z, hP.w, h.x, h.y, h.z, h.w, Cx, Cy);
+                Q = ring_vertex(hQ.x, hQ.y, hQ.z, hQ.w, h.x, h.y, h.z, h.w, Cx, Cy);
+                rn = fmaxf(fmaxf(fabsf(P.x), fabsf(P.y)), fmaxf(fabsf(Q.x), fabsf(Q.y)));
+                step = true;
+                if (irregular) {
+                    const uint32_t *row = a.win_rows + (size_t)cold * 32u + src;
+                    step = ((__ldg(row) >> (2u * t)) & 3u) != 3u;
+                    if ((__ldg(row + 32) >> t) & 1u) sgn = -1.0f;
+                }
+                if (step) {
+                    float vo, vn, so, sn;
+                    ring_values(P, Q, vo, vn, so, sn);
+                    v = sgn * (after ? vn : vo);
+                    s = after ? sn : so;
+                }
+            }
+            float least = v, most = step ? fabsf(v) : 0.0f, smin = s;  // of the side's 16 lanes
+#pragma unroll
+            for (int w = 8; w > 0; w >>= 1) {
+                least = fminf(least, __shfl_xor_sync(0xffffffffu, least, w));
+                most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, w));
+                smin = fminf(smin, __shfl_xor_sync(0xffffffffu, smin, w));
+                rn = fmaxf(rn, __shfl_xor_sync(0xffffffffu, rn, w));
+            }
+            const float rN = fmaxf(rn, fmaxf(fabsf(Cx), fabsf(Cy)));
+            const float M = fmaxf(fabsf(h.x), fabsf(h.z)) * 1.0001f + rN;
+            const float g = side_g(after ? rN : rn, smin), amax = kTwoSqrt3f * most;
+            const bool ok = frame_ok(rn, rN, M) & bound_ok(smin, g, amax);
+            const float b = side_bound(amax, g), up = kTwoSqrt3f * least + b, lo = kTwoSqrt3f * least - b;
+            const unsigned cands = __ballot_sync(0xffffffffu, step && !(ok && kTwoSqrt3f * v - b > up));
+            const bool both = __all_sync(0xffffffffu, ok);
+            const bool above = __shfl_sync(0xffffffffu, lo, 16) > __shfl_sync(0xffffffffu, up, 0);
+            const bool below = __shfl_sync(0xffffffffu, up, 16) < __shfl_sync(0xffffffffu, lo, 0);
+            int verdict = both ? (above ? 1 : (below ? -1 : 0)) : 0;
+            const unsigned first = cands & 0xffffu;
+            if (both && verdict == 0 && first == cands >> 16 && (first & (first - 1u)) == 0u) {
+                verdict = diff_screen(P.x, P.y, Q.x, Q.y, Cx, Cy, sgn, M * M);
+                verdict = __shfl_sync(0xffffffffu, verdict, __ffs((int)first) - 1);
+            }
+            const uint32_t cnt = __popc(cands);
+            if (verdict != 0) {
+                mask &= mask - 1u;
+                if (lane == src) {
+                    finish_screened<LAYOUT>(a, q, node, verdict > 0,
+                                            *reinterpret_cast<const ulonglong2 *>(xy + own), c, Cx, Cy);
+                    if (verdict > 0) state |= 3u << 24;
+                    atomicSub(&q->nexact, 1u);  // (counted as open before; added up when the block's counts are)
+                }
+            } else if (fill + cnt <= 32u) {
+                mask &= mask - 1u;
+                if (lane >= fill && lane < fill + cnt)
+                    state = (state & ~0x3ffu) | src | (set_bit(cands, lane - fill) << 5);
+                if (lane == src) state |= (fill << 10) | (cnt << 15) | (__popc(first) << 20);
+                fill += cnt;
+            } else {  // it comes again once there is room
+                evaluate = true;
+            }
+        }
+        if (evaluate && fill > 0u) {
+            const uint32_t of = state & 31u, ts = (state >> 5) & 15u;
+            const uint32_t own = (win::meta_place(__shfl_sync(0xffffffffu, meta0, of)) + 1u) * 16u;
+            long long key;
+            {
+                ulonglong2 x;
+                x.x = __shfl_sync(0xffffffffu, c.x, of);
+                x.y = __shfl_sync(0xffffffffu, c.y, of);
+                const uint32_t *row = a.win_rows + (size_t)cold * 32u + of;
+                key = quality_key(bitsd(0x7ff0000000000000ull));
+                if (lane < fill) {
+                    if (!(state & 0x200u)) x = *reinterpret_cast<const ulonglong2 *>(xy + own);
+                    const uint32_t *ring = list + (int)of - (int)lane;
+                    const ulonglong2 A = *reinterpret_cast<const ulonglong2 *>(xy + List<BITS>::at(ring, ts));
+                    const ulonglong2 B = *reinterpret_cast<const ulonglong2 *>(xy + List<BITS>::at(ring, ts + 1u));
+                    key = quality_key(step_quality(x, A.x, A.y, B.x, B.y, __ldg(row), __ldg(row + 32), ts));
+                }
+            }
+            const uint32_t i0 = (state >> 10) & 31u, n = (state >> 15) & 31u, n_old = (state >> 20) & 15u;
+            const uint32_t most = __reduce_max_sync(0xffffffffu, n);
+            long long k_old = quality_key(bitsd(0x7ff0000000000000ull)), k_new = k_old;
+            for (uint32_t k = 0; k < most; ++k) {
+                const long long u = __shfl_sync(0xffffffffu, key, (int)((i0 + k) & 31u));
+                if (k < n_old) k_old = u < k_old ? u : k_old;
+                else if (k < n) k_new = u < k_new ? u : k_new;
+            }
+            if (n) {
+                unsigned long long b2;
+                bool acc, moved;
+                const ulonglong2 p =
+                    *reinterpret_cast<const ulonglong2 *>(xy + (win::meta_place(meta0) + 1u) * 16u);
+                finish_exact<LAYOUT>(a, node, make_double2(bitsd(p.x), bitsd(p.y)), make_double2(bitsd(c.x), bitsd(c.y)),
+                                     key_quality(k_old), key_quality(k_new), b2, acc, moved);
+                note_move(q, b2);
+                state |= ((acc ? 1u : 0u) | (moved ? 2u : 0u)) << 24;
+            }
+            state &= ~0xfffc00u;
+            fill = 0u;
+        }
+    } while (mask | fill);
+    return state >> 24;
+}
+
 // What a lane knows of a node that its screen left open.
 struct Open {
     float Cx, Cy;        // the centre's offset
     float b, up_o, up_n; // a step is a candidate unless its value less b lies above the side's up
     uint32_t own, steps;
+    uint32_t meta;
 };
+
+// Open nodes of a warp from which it settles them itself (settle_open): its items
+// then fill the FP64 pipe's lanes without the block's queue, and the closer screen
+// decides a part.  A mesh flattened to 1e-3 (15 of 32 nodes open) takes 264 us a
+// pass without this, 237 with 16, 217 with 12; 100,000 Delaunay points, few of whose
+// warps have as many, take 1.36 ms a call with 16, 1.37 with 12 and 1.41 with 8.
+constexpr int kManyOpen = 16;
 
 // The nodes of a warp that its screen left open (mask): for each, lane t looks
 // at step t before the move and lane 16 + t after it; the steps that can
-// attain a side's minimum go into the queue or, when that has no room, are
-// evaluated at once.  list: a lane's ring; cold: the subtile's slots row.
-// Returns per lane 1 accepted, 2 moved (decided at once), 8 queue full enough
-// to be worked off.
+// attain a side's minimum go into the queue.  The others: settle_open.  list: a
+// lane's ring; cold: the subtile's slots row.  Returns per lane 1 accepted, 2
+// moved (decided here), 8 queue full enough to be worked off.
 template <int LAYOUT, int BITS>
-__device__ __noinline__ uint32_t settle_open(const PassArgs &a, Queue *q, const char *xy, uint32_t half,
-                                             const uint32_t *list, uint32_t cold, bool irregular, int32_t node,
-                                             ulonglong2 c, Open o, unsigned mask)
+__device__ __noinline__ uint32_t work_open(const PassArgs &a, Queue *q, const char *xy, uint32_t half,
+                                           const uint32_t *list, uint32_t cold, bool irregular, int32_t node,
+                                           ulonglong2 c, Open o, unsigned mask)
 {
     const uint32_t lane = threadIdx.x & 31u, t = lane & 15u;
     const bool after = lane >= 16u;
     uint32_t out = 0u;
+    unsigned left = 0u;
+    if (__popc(mask) >= kManyOpen) {
+        left = mask;
+        mask = 0u;
+    }
     for (; mask; mask &= mask - 1u) {
         const uint32_t src = (uint32_t)__ffs((int)mask) - 1u;
         const uint32_t own = __shfl_sync(0xffffffffu, o.own, src), steps = __shfl_sync(0xffffffffu, o.steps, src);
@@ -446,45 +680,10 @@ __device__ __noinline__ uint32_t settle_open(const PassArgs &a, Queue *q, const 
         // no room: what was claimed stays empty
         if (i0 + lane < (uint32_t)kItems && lane < cnt) q->item[i0 + lane] = kNoItem;
         if (lane == 0u && e < (uint32_t)kPending) q->node[e] = -1;
-        const ulonglong2 p = *reinterpret_cast<const ulonglong2 *>(xy + own);
-        const ulonglong2 cs = make_ulonglong2(__shfl_sync(0xffffffffu, c.x, src), __shfl_sync(0xffffffffu, c.y, src));
-        double v = bitsd(0x7ff0000000000000ull);
-        if (cand) v = step_quality(after ? cs : p, P.x, P.y, Q.x, Q.y, __ldg(row), __ldg(row + 32), t);
-        for (int w = 8; w > 0; w >>= 1) {
-            const double u = __shfl_xor_sync(0xffffffffu, v, w);
-            if (u < v) v = u;
-        }
-        const double q_old = __shfl_sync(0xffffffffu, v, 0), q_new = __shfl_sync(0xffffffffu, v, 16);
-        if (lane == src) {
-            unsigned long long b2;
-            bool acc, moved;
-            finish_exact<LAYOUT>(a, node, make_double2(bitsd(p.x), bitsd(p.y)), make_double2(bitsd(c.x), bitsd(c.y)),
-                                 q_old, q_new, b2, acc, moved);
-            note_move(q, b2);
-            out |= (acc ? 1u : 0u) | (moved ? 2u : 0u);
-        }
+        left |= 1u << src;
     }
+    if (left) out |= settle_open<LAYOUT, BITS>(a, q, xy, half, list, cold, irregular, node, c, o.meta, left);
     return out;
-}
-
-// FP32 offset of the centre from the node (relative error below 2^-23).  With
-// equal sign and exponent field the difference is a whole number of units in
-// the last place; otherwise one FP64 subtraction.
-__device__ __forceinline__ void offset_of(ulonglong2 c, ulonglong2 p, float &Cx, float &Cy)
-{
-    const uint32_t hx = (uint32_t)(p.x >> 32), hy = (uint32_t)(p.y >> 32);
-    const uint32_t ex = (hx >> 20) & 0x7ffu, ey = (hy >> 20) & 0x7ffu;
-    const uint32_t other = ((uint32_t)((c.x ^ p.x) >> 32) | (uint32_t)((c.y ^ p.y) >> 32)) & 0xfff00000u;
-    if (other == 0u && ex - 949u <= 200u && ey - 949u <= 200u) {
-        // unit in the last place, with the sign of the coordinate
-        const float ux = __uint_as_float((hx & 0x80000000u) | ((ex - 948u) << 23));
-        const float uy = __uint_as_float((hy & 0x80000000u) | ((ey - 948u) << 23));
-        Cx = __ll2float_rn((long long)(c.x - p.x)) * ux;
-        Cy = __ll2float_rn((long long)(c.y - p.y)) * uy;
-    } else {
-        Cx = trunc_float(dbits(__dsub_rn(bitsd(c.x), bitsd(p.x))));
-        Cy = trunc_float(dbits(__dsub_rn(bitsd(c.y), bitsd(p.y))));
-    }
 }
 
 // A subtile's rows, for one lane.
@@ -638,8 +837,9 @@ __device__ __forceinline__ bool update_lane(const PassArgs &a, Queue *q, const c
             o.Cy = w.Cy;
             o.own = own;
             o.steps = steps;
+            o.meta = r.meta;
             const uint32_t done =
-                settle_open<LAYOUT, BITS>(a, q, xy, half, list, r.cold, r.irregular, node, cb, o, open);
+                work_open<LAYOUT, BITS>(a, q, xy, half, list, r.cold, r.irregular, node, cb, o, open);
             full = full || (done & 8u);
             if (done & 3u) res = done & 3u;
             tally.nacc += done & 1u;
