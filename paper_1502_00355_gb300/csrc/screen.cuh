@@ -120,9 +120,9 @@ constexpr float kGMax = 1000.0f;
 constexpr float kTwoSqrt3f = 3.46410161514f;
 constexpr float kLocalRange = 1048576.0f;  // 2^20: R * 2^20 >= M keeps the head/tail error below e R
 
-// (local_offset, screen_alpha, edge_ba2 and bound_ok are the screen of one
-// triangle by itself, from which the constants above are derived.  The pass uses
-// the ring form below; the CPU tests pin the constants with both.)
+// (local_offset, screen_alpha and edge_ba2 are the screen of one triangle by
+// itself, from which the constants above are derived.  The pass uses the ring form
+// below; the CPU tests pin the constants with both.)
 
 // Offset of a neighbour (bit patterns bx, by) from the node whose head/tail
 // splits are (phx, plx), (phy, ply); ok &= both splits are valid.
