@@ -21,6 +21,7 @@ struct PassStats {
 // bits of a list entry (window.cuh).
 struct WindowShape {
     int entries = 0, halo = 0, hot = 0, bits = 8;
+    int buffers32 = 2;  // buffers of rows and staged entries of the binary32 pass (choose_buffers32)
     void cover(const WindowShape &o)
     {
         entries = entries > o.entries ? entries : o.entries;

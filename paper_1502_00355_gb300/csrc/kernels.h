@@ -67,6 +67,9 @@ cudaError_t launch_histogram(const double *xy, int layout, int64_t n, const int3
 cudaError_t launch_pass_f32(const PassArgs &a, int layout, int block, int grid, const WindowShape &shape,
                             cudaStream_t s);
 int pass_f32_occupancy(int layout, int block, const WindowShape &shape);
+// How many windows' data a block of the binary32 pass holds (shape.buffers32),
+// for a mesh of so many windows.
+void choose_buffers32(int layout, int block, int64_t windows, WindowShape &shape);
 // Copy-back form of the binary32 pass (count floats; skipped when pass q was skipped).
 cudaError_t launch_copy_back_f32(const float *src, float *dst, int64_t count, const PassStats *stats, int q,
                                  int grid, cudaStream_t s);

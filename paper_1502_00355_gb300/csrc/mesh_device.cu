@@ -103,6 +103,7 @@ static sls_status finish_creation(sls_mesh *M)
         st = build_windows(M->n, M->opt.form == 1 ? M->colour_off : std::vector<int64_t>(), M->node_off, M->adj,
                            groups_lanes(M->opt), M->f32, M->stream, M->windows);
         if (st != SLS_OK) return st;
+        if (M->f32) choose_buffers32(M->opt.layout, M->block, M->windows.count, M->windows.shape);
         M->grid = device_sm_count() * (M->f32 ? pass_f32_occupancy(M->opt.layout, M->block, M->windows.shape)
                                               : pass_screened_occupancy(M->opt.layout, M->block, M->windows.shape));
     }

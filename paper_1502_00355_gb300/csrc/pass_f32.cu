@@ -10,6 +10,7 @@
 // takes one node from start to end.
 #include <cfloat>
 
+#include "api_common.h"
 #include "kernels.h"
 #include "screen.cuh"
 #include "window_pipe.cuh"
@@ -170,13 +171,13 @@ struct Block32 {
     Ahead *ahead;
     uint32_t *ids, *rows;
     char *xy;
-    uint32_t ids_words, rows_words, stage;
+    uint32_t ids_words, rows_words, stage;  // buffer sizes: words, words, bytes; the last two 0 where there is one
 };
 
 size_t smem_f32(const WindowShape &s)
 {
-    return sizeof(Ahead) + 2 * 4 * (size_t)ids_words_of(s) + 2 * 128 * (size_t)(s.hot + win::kColdRows) +
-           2 * 8 * (size_t)(s.entries + 1);
+    return sizeof(Ahead) + 2 * 4 * (size_t)ids_words_of(s) +
+           (size_t)s.buffers32 * (128 * (size_t)(s.hot + win::kColdRows) + 8 * (size_t)(s.entries + 1));
 }
 
 __device__ __forceinline__ float2 entry32(const char *xy, uint32_t off)
@@ -376,8 +377,8 @@ __device__ __forceinline__ void work32(const PassArgs &a, const float *in, float
 }
 
 // One pass over a mesh's windows, or over those of one colour class of Form B
-// (in place).  a.in / a.out hold floats.
-template <int LAYOUT, int BITS>
+// (in place).  a.in / a.out hold floats.  TWO: shape.buffers32 is 2.
+template <int LAYOUT, int BITS, bool TWO>
 __global__ void __launch_bounds__(kBlock32, kBlocks32)
     pass_f32_kernel(const __grid_constant__ PassArgs a, const __grid_constant__ WindowShape shape)
 {
@@ -391,8 +392,9 @@ __global__ void __launch_bounds__(kBlock32, kBlocks32)
     b.ids_words = ids_words_of(shape);
     b.rows = b.ids + 2 * b.ids_words;
     b.rows_words = 32u * (uint32_t)(shape.hot + (int)win::kColdRows);
-    b.xy = reinterpret_cast<char *>(b.rows + 2 * b.rows_words);
-    b.stage = (uint32_t)(shape.entries + 1) * 8u;
+    b.xy = reinterpret_cast<char *>(b.rows + (TWO ? 2 : 1) * b.rows_words);
+    b.stage = TWO ? (uint32_t)(shape.entries + 1) * 8u : 0u;
+    if (!TWO) b.rows_words = 0u;
     if (tid < 2) *reinterpret_cast<float2 *>(b.xy + tid * b.stage) = make_float2(-0.0f, -0.0f);  // the padding entries
 
     // windows blockIdx.x, + gridDim.x, ...: headers three ahead, halo ids two,
@@ -443,12 +445,18 @@ __global__ void __launch_bounds__(kBlock32, kBlocks32)
     after_previous();
     if (pass_is_skipped(a.stats, a.q, a.tol_active, a.thr_bits)) return;
     if (blockIdx.x == 0 && tid == 0) a.stats[a.q].executed = 1u;
-    fetch_data(0);
+    if (TWO) fetch_data(0);
     unsigned best = 0u, nacc = 0u;
     for (int i = 0; i < n; ++i) {
         copies_done();
         __syncthreads();
-        fetch_data(i + 1);
+        if (TWO) {
+            fetch_data(i + 1);
+        } else {  // window i - 1 is finished
+            fetch_data(i);
+            copies_done();
+            __syncthreads();
+        }
         fetch_ids(i + 2);
         fetch_header(i + 3);
         for (int sub = warp; sub < 4; sub += nwarps)
@@ -507,11 +515,14 @@ __global__ void widen_kernel(const float *__restrict__ src, double *aos, int64_t
 
 namespace {
 
-const void *kernel32(int layout, int bits)
+template <int LAYOUT>
+const void *kernel32_of(const WindowShape &s)
 {
-    if (layout == 0) return bits == 8 ? (const void *)pass_f32_kernel<0, 8> : (const void *)pass_f32_kernel<0, 16>;
-    return bits == 8 ? (const void *)pass_f32_kernel<1, 8> : (const void *)pass_f32_kernel<1, 16>;
+    if (s.bits == 8) return (const void *)pass_f32_kernel<LAYOUT, 8, true>;  // (at most 255 entries)
+    return s.buffers32 == 2 ? (const void *)pass_f32_kernel<LAYOUT, 16, true>
+                            : (const void *)pass_f32_kernel<LAYOUT, 16, false>;
 }
+const void *kernel32(int layout, const WindowShape &s) { return layout == 0 ? kernel32_of<0>(s) : kernel32_of<1>(s); }
 
 }  // namespace
 
@@ -520,19 +531,36 @@ cudaError_t launch_pass_f32(const PassArgs &a, int layout, int block, int grid, 
 {
     if (a.win_count < grid) grid = a.win_count > 0 ? (int)a.win_count : 1;
     void *args[] = {const_cast<PassArgs *>(&a), const_cast<WindowShape *>(&shape)};
-    return launch_early(kernel32(layout, shape.bits), grid, block, args, smem_f32(shape), s);
+    return launch_early(kernel32(layout, shape), grid, block, args, smem_f32(shape), s);
 }
 
 // Also allows the kernel the shared memory that the shape takes; a launch in
 // another context would need it again, and meshes belong to their context.
 int pass_f32_occupancy(int layout, int block, const WindowShape &shape)
 {
-    const void *f = kernel32(layout, shape.bits);
+    const void *f = kernel32(layout, shape);
     int nb = 0;
     if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess)
         cudaGetLastError();
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, block, smem_f32(shape));
     return nb > 0 ? nb : 1;
+}
+
+// A second buffer, into which the next window is copied while one is worked on,
+// costs blocks where windows are wide: 1009 x 701 nodes, us a pass with one and with
+// two buffers, random ids kept (about 900 entries a window) 37.3 and 49.4, SoA 49.0
+// and 75.9; Form B (colour classes, about 510) 58.8 and 64.1; rows of the grid
+// kept (about 390) 29.2 and 28.9.  With about a window a block it has nothing to do
+// either, but fewer blocks an SM then spread the windows evenly, where early
+// launches would fill some SMs first: 100,000 Delaunay points, random ids kept (782
+// windows) 25.8 with one, 19.9 with two.
+void choose_buffers32(int layout, int block, int64_t windows, WindowShape &shape)
+{
+    constexpr int kTwoBuffers = 448;
+    shape.buffers32 = 2;
+    if (shape.entries > kTwoBuffers &&
+        windows > 2 * (int64_t)device_sm_count() * pass_f32_occupancy(layout, block, shape))
+        shape.buffers32 = 1;
 }
 
 cudaError_t launch_copy_back_f32(const float *src, float *dst, int64_t count, const PassStats *stats, int q,
