@@ -148,7 +148,7 @@ sls_status build_device_mesh(sls_mesh *M, double *d_xy, int32_t *d_tri, const ui
 // (mesh_build_gpu.cu): fills M->node_order.
 sls_status build_node_order(sls_mesh *M, cudaStream_t s);
 // The tile lists and masks of unchanged-tile skipping (mesh_build_gpu.cu),
-// when opt.skip_unchanged is set.
+// when opt.skip_unchanged is set and some tile can be skipped at all.
 sls_status build_tile_halo(sls_mesh *M, cudaStream_t s);
 void mesh_release(sls_mesh *M);
 sls_status mesh_run(sls_mesh *M, int32_t max_iter, double tol_rel, sls_info &info);

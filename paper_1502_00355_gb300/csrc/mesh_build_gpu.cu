@@ -833,9 +833,10 @@ __global__ void colour_max_kernel(const int32_t *__restrict__ colour, int64_t n,
 // Unchanged-tile skipping: for tile t (nodes 32t .. 32t+31), the tiles that
 // hold its nodes and the neighbours of its free nodes, each with the mask of
 // those nodes; (kHaloNever, 0) when more than kHaloEntries tiles are involved
-// (such a tile is always computed).  One thread per tile.
+// (such a tile is always computed).  *skippable counts the others.  One thread per
+// tile.
 __global__ void tile_halo_kernel(const uint32_t *__restrict__ node_off, const uint32_t *__restrict__ adj,
-                                 int64_t n, int64_t ntiles, uint2 *halo)
+                                 int64_t n, int64_t ntiles, uint2 *halo, unsigned *skippable)
 {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= ntiles) return;
@@ -867,6 +868,7 @@ __global__ void tile_halo_kernel(const uint32_t *__restrict__ node_off, const ui
             masks[e] |= 1u << (j & 31);
         }
     }
+    if (!over) atomicAdd(skippable, 1u);
     uint2 *h = halo + t * kHaloEntries;
     for (int e = 0; e < kHaloEntries; ++e)
         h[e] = over ? make_uint2(e == 0 ? kHaloNever : 0u, 0u)
@@ -884,9 +886,23 @@ sls_status build_tile_halo(sls_mesh *M, cudaStream_t s)
     GB_TRY(pool_alloc((void **)&M->accm, sizeof(uint32_t) * (size_t)nt, s), "tile masks");
     for (int k = 0; k < 2; ++k) GB_TRY(cudaMemsetAsync(M->chg[k], 0xff, sizeof(uint32_t) * (size_t)nt, s), "tile masks");
     GB_TRY(cudaMemsetAsync(M->accm, 0, sizeof(uint32_t) * (size_t)nt, s), "tile masks");
-    tile_halo_kernel<<<(unsigned)((nt + 127) / 128), 128, 0, s>>>(M->node_off, M->adj, M->n, nt, M->halo);
+    DevBuf b_cnt;
+    unsigned *cnt = nullptr, skippable = 0u;
+    sls_status st = dalloc(b_cnt, 1, &cnt, "tile halo", Alloc{s});
+    if (st != SLS_OK) return st;
+    GB_TRY(cudaMemsetAsync(cnt, 0, sizeof(unsigned), s), "tile halo");
+    tile_halo_kernel<<<(unsigned)((nt + 127) / 128), 128, 0, s>>>(M->node_off, M->adj, M->n, nt, M->halo, cnt);
     GB_TRY(cudaGetLastError(), "tile halo");
+    GB_TRY(cudaMemcpyAsync(&skippable, cnt, sizeof skippable, cudaMemcpyDeviceToHost, s), "tile halo");
     GB_TRY(cudaStreamSynchronize(s), "tile halo");
+    if (skippable == 0u) {
+        // a numbering so far from local that no tile can ever be skipped: the
+        // passes without the masks, which also start early (random ids, 1009 x 701
+        // nodes: 66.5 us a pass against 77.1, SoA 84.4 against 98.9)
+        for (void *p : {(void *)M->halo, (void *)M->chg[0], (void *)M->chg[1], (void *)M->accm}) pool_free(p, s);
+        M->halo = nullptr;
+        M->chg[0] = M->chg[1] = M->accm = nullptr;
+    }
     return SLS_OK;
 }
 
