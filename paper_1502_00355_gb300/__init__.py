@@ -305,7 +305,7 @@ class Batch:
 
     @property
     def shape(self) -> tuple[int, int]:
-        """(threads per block, warp chunk) of the launches."""
+        """(threads per block, tasks a block takes at a time) of the launches."""
         b, c = C.c_int32(), C.c_int64()
         _check(lib().sls_batch_shape(self._h, C.byref(b), C.byref(c)), "sls_batch_shape")
         return b.value, c.value

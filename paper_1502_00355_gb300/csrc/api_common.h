@@ -135,7 +135,8 @@ void pool_free(void *p, cudaStream_t s);
 // ranges to cover one after another (Form B: the colour classes' bounds),
 // empty = one segment of all n nodes.  group: nodes dealt to the lanes by ring
 // length inside a window.  cyclic: ring lists padded for the binary32 walk.
-// Synchronises s.
+// Waits for s between its two kernels; the second one, which writes the rows, may
+// still run when it returns.
 sls_status build_windows(int64_t n, const std::vector<int64_t> &segments, const uint32_t *node_off,
                          const uint32_t *adj, bool group, bool cyclic, cudaStream_t s, WindowStream &out);
 // Whether options o deal a window's nodes to the lanes by ring length: not

@@ -173,11 +173,11 @@ sls_status reset(sls_batch *B)
 }
 
 // Picks the launch shape by timing a whole batch smooth for each candidate,
-// restoring the starting coordinates after every trial: the block size (32-
-// node tasks a CTA runs at once, 4 per 128 threads) and the chunk of
-// consecutive tasks a warp takes: one contiguous share of the list (0), 64
-// in a grid stride, or 32 claimed from a per-round counter.  Every round of a call is one node of one
-// CUDA graph, so all passes of a call are one launch whatever the shape.
+// restoring the starting coordinates after every trial: the block size (a task,
+// a window of 128 nodes, is worked on by one block) and the chunk of consecutive
+// tasks a block takes: one contiguous share of the list (0), or 16 claimed from a
+// per-round counter.  Every round of a call is one node of one CUDA graph, so all
+// passes of a call are one launch whatever the shape.
 sls_status autotune(sls_batch *B, bool tune_block)
 {
     struct Shape {
@@ -185,11 +185,15 @@ sls_status autotune(sls_batch *B, bool tune_block)
         int64_t chunk;
     };
     std::vector<Shape> cands;
-    const int blocks[2] = {64, 128};  // the kernel is built for 6 blocks of <= 128
-    // chunks of 1 to 16 tasks measured 11-60% slower on the 2,048-mesh
-    // workload: a warp that changes job drains its deferred nodes at partial
-    // width, so short chunks run the exact FP64 path with few lanes active
-    const int64_t chunks[3] = {0, 64, -32};  // < 0: claimed from a per-round counter
+    const int blocks[2] = {64, 128};  // the kernel is built for 7 blocks of <= 128
+    // A block that changes job or chunk fetches its first windows afresh and works
+    // off its queue at partial width, so short chunks cost; long ones leave blocks
+    // without work.  ms a call, block 128, chunks 0 | in a stride 1, 4, 16, 64 |
+    // claimed 1, 4, 16, 32:
+    //   48 meshes (21,264 tasks)   9.15 | 12.9 10.2 13.6 30.9 | 12.5  9.7 13.7 20.7
+    //   512 meshes                 62.5 | 97.7 71.3 65.7 79.6 | 94.7 67.7 61.9 64.7
+    //   256 meshes of 1,023 nodes  0.60 | 0.69 0.70 1.47 4.75 | 0.68 0.80 1.97 3.33
+    const int64_t chunks[2] = {0, -16};  // < 0: claimed from a per-round counter
     for (int b : blocks) {
         if (!tune_block && b != B->block) continue;
         for (int64_t c : chunks) cands.push_back(Shape{b, c});
@@ -318,7 +322,7 @@ sls_status sls_batch_create(sls_mesh *const *meshes, int32_t k, const int32_t *i
         return fail_free(fail(SLS_ERR_OOM, "batch allocation failed"));
     }
     if (cudaMemcpy(B->d_tasks, tasks.data(), sizeof(WindowTask) * B->ntasks, cudaMemcpyHostToDevice) != cudaSuccess)
-        return fail_free(fail(SLS_ERR_CUDA, "upload warp tasks"));
+        return fail_free(fail(SLS_ERR_CUDA, "upload tasks"));
     B->d_start.assign(k, nullptr);
     for (int j = 0; j < k; ++j) {
         sls_mesh *M = B->meshes[j];

@@ -201,7 +201,7 @@ struct sls_server {
     std::vector<std::thread> builders;
     std::thread sched, retirer;
 
-    // job table and warp tasks of the active set; the host staging and the
+    // job table and window tasks of the active set; the host staging and the
     // round records are double-buffered by round parity, because round r+1
     // is launched before the records of round r are read
     JobDesc *d_jobs = nullptr, *h_jobs[2] = {nullptr, nullptr};
@@ -400,7 +400,7 @@ bool grow_dev(T *&d, size_t &cap, size_t need)
     return true;
 }
 
-// Rebuilds the job table and the warp-task list of the active set for the
+// Rebuilds the job table and the task list of the active set for the
 // round launched next, whose parity is `slot`: the table and each job's
 // first task are staged on the host, the task list is expanded on the device.
 bool rebuild_table(sls_server *S, int slot)
