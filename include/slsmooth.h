@@ -358,8 +358,9 @@ sls_status sls_server_destroy(sls_server *srv);
  *            serves as the second buffer of the ping-pong, so its contents
  *            are unspecified on return
  *   xy_out   device, 2n float64: receives the result (distinct from xy_in);
- *            both buffers aligned to 16 bytes (SLS_ERR_INVALID otherwise; the
- *            other entry points take device coordinates at any float64)
+ *            both buffers aligned to 16 bytes (SLS_ERR_INVALID otherwise, unless
+ *            max_iter is 0; the other entry points take device coordinates at any
+ *            float64)
  *   max_iter 0 .. SLS_NOALLOC_MAX_PASSES; larger values are rejected with
  *            SLS_ERR_INVALID
  *   stream   cudaStream_t, or NULL for the mesh's stream; the call returns

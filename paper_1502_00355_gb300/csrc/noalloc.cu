@@ -79,7 +79,7 @@ extern "C" sls_status sls_smooth_noalloc(const sls_mesh *M, double *xy_in, doubl
     if (!M || !xy_in || !xy_out) return fail(SLS_ERR_INVALID, "mesh, xy_in and xy_out must not be NULL");
     if (xy_in == xy_out) return fail(SLS_ERR_INVALID, "xy_in and xy_out must be distinct buffers");
     // the passes read and write nodes of 16 bytes
-    if (!pair_aligned(xy_in) || !pair_aligned(xy_out))
+    if (max_iter > 0 && (!pair_aligned(xy_in) || !pair_aligned(xy_out)))
         return fail(SLS_ERR_INVALID, "sls_smooth_noalloc needs buffers aligned to 16 bytes");
     if (M->opt.layout != 0) return fail(SLS_ERR_INVALID, "sls_smooth_noalloc needs a mesh with the AoS layout");
     if (M->opt.form != 0 || M->f32) return fail(SLS_ERR_INVALID, "sls_smooth_noalloc runs FP64 Form A only");

@@ -36,14 +36,15 @@
 // unless they take part in FP64 arithmetic: the compiler copies FP64
 // registers with FP64-pipe instructions.
 //
-// What bounds it: instruction issue (65% of slots), the FP64 pipe (58%) and
-// the latency of shared-memory loads together; HBM stands at about a sixth of
-// the measured copy rate.  Gathering and splitting a coordinate once per
-// window (1.4 times a node) instead of once per neighbour visit (6.5 times)
-// took 1,653 warp instructions per 32 nodes to 1,140 and 23.5 FP64
-// instructions to 13.7.  Measured, to the tolerance, against one thread per
-// node gathering for itself: 2048^2 jittered grid 293.7 -> 200.8 us a pass,
-// 1024^2 96.9 -> 59.2, 4096^2 942 -> 660.
+// What bounds it: instruction issue (65% of slots in an early pass of a 2048^2
+// grid), the FP64 pipe (58% there; half of the time over a 4096^2 run to the
+// tolerance) and the latency of shared-memory loads together; HBM stands at about
+// a sixth of the measured copy rate.  Gathering and splitting a coordinate once
+// per window (1.4 times a node) instead of once per neighbour visit (6.5 times)
+// took 1,653 warp instructions per 32 nodes to 1,148 and 23.5 FP64 instructions to
+// 13.8.  Measured, to the tolerance, against one thread per node gathering for
+// itself: 2048^2 jittered grid 293.7 -> 200.8 us a pass, 1024^2 96.9 -> 59.2,
+// 4096^2 942 -> 630..700 (by GPU; clustered about fewer centres 1058 -> 741).
 #include <atomic>
 #include <cfloat>
 #include <mutex>
@@ -591,7 +592,7 @@ struct Open {
     float Cx, Cy;        // the centre's offset
     float b, up_o, up_n; // a step is a candidate unless its value less b lies above the side's up
     uint32_t own, steps;
-    uint32_t meta;
+    uint32_t meta;       // the lane's meta word
 };
 
 // Open nodes of a warp from which it settles them itself (settle_open): its items

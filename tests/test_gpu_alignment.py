@@ -65,4 +65,5 @@ def test_noalloc_refuses_odd_offsets(sls):
             with pytest.raises(sls.SlsError) as e:
                 g.smooth_noalloc(a, b, 2)
             assert e.value.code == 1
+            assert g.smooth_noalloc(a, b, 0)["iterations"] == 0  # (a copy)
         assert g.smooth_noalloc(even, torch.empty_like(even), 2)["iterations"] == 2
