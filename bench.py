@@ -44,16 +44,16 @@ PROFILE_FIGURES = {
     "pass_screened": {
         "files": ["pass_screened.cu", "screen.cuh", "window.cuh", "window_pipe.cuh", "window_build.cu", "node_exact.cuh",
                   "div_small.cuh", "device.cuh"],
-        "sha256": "92e72e8d8b25131d481cd3faf46df4a0fc5f8ccb700709b6853dec15eaa18740",
-        "dram_bytes_per_node": (172718848 + 41475840) / (2048 * 2048),
-        "fp64_warp_inst_per_32_nodes": (1498820 + 301032 + 12061) / (2048 * 2048 / 32),
+        "sha256": "77b7a1a958e8a786be54c546334da5b42e530f8dc3dd369663dd1a21b43f4ac3",
+        "dram_bytes_per_node": (172729088 + 41547264) / (2048 * 2048),
+        "fp64_warp_inst_per_32_nodes": (1498730 + 300972 + 12061) / (2048 * 2048 / 32),
         "source": "profiles/pass_screened_grid2048.md (2048x2048 capture, per node)",
     },
     "batch_pass": {
         "files": ["pass_screened.cu", "screen.cuh", "window.cuh", "window_pipe.cuh", "window_build.cu", "node_exact.cuh",
                   "div_small.cuh", "device.cuh", "batch.cu"],
-        "sha256": "738678658f668f452a38fafb349286d4b3cf5434e77e48b767b76aa8207b82b4",
-        "dram_per_alg_byte": (493175808 + 159224064) / 994046024,
+        "sha256": "a30b84045d93b6f5f35af3804e1aaa248fbc10ea0d920814d3eb78245061d250",
+        "dram_per_alg_byte": (494562048 + 161026560) / 994046024,
         "source": "profiles/batch_pass_batch256.md (round 0 of a 256-mesh batch, scaled by algorithmic bytes)",
     },
 }

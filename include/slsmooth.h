@@ -249,8 +249,8 @@ sls_status sls_trim_memory(size_t keep_bytes);
  * sls_batch_reset.  The launch shape is autotuned by timing one full batch
  * smooth per candidate, restoring the saved coordinates after each trial:
  * the chunk of consecutive 128-node tasks a block takes (one contiguous
- * share of the list per block, or 16 claimed in order from a per-round
- * counter) and, with opt == NULL or
+ * share of the list per block, or 16 or 32 claimed in order from a
+ * per-round counter) and, with opt == NULL or
  * opt->block_size == 0, the block size (64 or 128 threads); an explicit
  * block_size must be 32, 64, 96 or 128 (SLS_ERR_INVALID otherwise). */
 sls_status sls_batch_create(sls_mesh *const *meshes, int32_t k, const int32_t *iters,

@@ -175,8 +175,8 @@ sls_status reset(sls_batch *B)
 // Picks the launch shape by timing a whole batch smooth for each candidate,
 // restoring the starting coordinates after every trial: the block size (a task,
 // a window of 128 nodes, is worked on by one block) and the chunk of consecutive
-// tasks a block takes: one contiguous share of the list (0), or 16 claimed from a
-// per-round counter.  Every round of a call is one node of one CUDA graph, so all
+// tasks a block takes: one contiguous share of the list (0), or 16 or 32 claimed
+// from a per-round counter.  Every round of a call is one node of one CUDA graph, so all
 // passes of a call are one launch whatever the shape.
 sls_status autotune(sls_batch *B, bool tune_block)
 {
@@ -189,11 +189,12 @@ sls_status autotune(sls_batch *B, bool tune_block)
     // A block that changes job or chunk fetches its first windows afresh and works
     // off its queue at partial width, so short chunks cost; long ones leave blocks
     // without work.  ms a call, block 128, chunks 0 | in a stride 1, 4, 16, 64 |
-    // claimed 1, 4, 16, 32:
+    // claimed 1, 4, 16, 32, 64:
     //   48 meshes (21,264 tasks)   9.15 | 12.9 10.2 13.6 30.9 | 12.5  9.7 13.7 20.7
     //   512 meshes                 62.5 | 97.7 71.3 65.7 79.6 | 94.7 67.7 61.9 64.7
+    //   2,048 meshes              259.5 |                267.5 |          249.4 246.5 250.5
     //   256 meshes of 1,023 nodes  0.60 | 0.69 0.70 1.47 4.75 | 0.68 0.80 1.97 3.33
-    const int64_t chunks[2] = {0, -16};  // < 0: claimed from a per-round counter
+    const int64_t chunks[3] = {0, -16, -32};  // < 0: claimed from a per-round counter
     for (int b : blocks) {
         if (!tune_block && b != B->block) continue;
         for (int64_t c : chunks) cands.push_back(Shape{b, c});
