@@ -44,7 +44,7 @@ PROFILE_FIGURES = {
     "pass_screened": {
         "files": ["pass_screened.cu", "screen.cuh", "window.cuh", "window_pipe.cuh", "window_build.cu", "node_exact.cuh",
                   "div_small.cuh", "device.cuh"],
-        "sha256": "77b7a1a958e8a786be54c546334da5b42e530f8dc3dd369663dd1a21b43f4ac3",
+        "sha256": "be8cfa230a685d3fb4fdacdd5df0fc60f075d7dc69aad13b50a40dd14c108eb9",
         "dram_bytes_per_node": (172729088 + 41547264) / (2048 * 2048),
         "fp64_warp_inst_per_32_nodes": (1498730 + 300972 + 12061) / (2048 * 2048 / 32),
         "source": "profiles/pass_screened_grid2048.md (2048x2048 capture, per node)",
@@ -52,7 +52,7 @@ PROFILE_FIGURES = {
     "batch_pass": {
         "files": ["pass_screened.cu", "screen.cuh", "window.cuh", "window_pipe.cuh", "window_build.cu", "node_exact.cuh",
                   "div_small.cuh", "device.cuh", "batch.cu"],
-        "sha256": "a30b84045d93b6f5f35af3804e1aaa248fbc10ea0d920814d3eb78245061d250",
+        "sha256": "16ac4f04aadb43770ba0d295c5632a572eec7212df498a47bc9643b22592e155",
         "dram_per_alg_byte": (494562048 + 161026560) / 994046024,
         "source": "profiles/batch_pass_batch256.md (round 0 of a 256-mesh batch, scaled by algorithmic bytes)",
     },

@@ -522,6 +522,13 @@ const void *kernel32_of(const WindowShape &s)
     return s.buffers32 == 2 ? (const void *)pass_f32_kernel<LAYOUT, 16, true>
                             : (const void *)pass_f32_kernel<LAYOUT, 16, false>;
 }
+// Wide windows of separate x and y arrays take two 4-byte copies a coordinate, which
+// go through L1: with all the blocks an SM could hold, shared memory leaves little
+// of it.  1009 x 701 nodes, us a pass with 9 (8 in Form B), 6, 5, 4, 3 blocks: random
+// ids kept 48.2, 47.8, 59.6, 54.1, 70.2; Form B, random ids 124.8, 84.6, 90.0, 81.8,
+// 97.4, Morton order 61.1, 60.7, 62.7, 60.5, 69.8.
+constexpr int kWideSoaBlocks = 6;
+bool wide_soa(int layout, const WindowShape &s) { return layout == 1 && s.bits == 16 && s.buffers32 == 1; }
 const void *kernel32(int layout, const WindowShape &s) { return layout == 0 ? kernel32_of<0>(s) : kernel32_of<1>(s); }
 
 }  // namespace
@@ -531,7 +538,8 @@ cudaError_t launch_pass_f32(const PassArgs &a, int layout, int block, int grid, 
 {
     if (a.win_count < grid) grid = a.win_count > 0 ? (int)a.win_count : 1;
     void *args[] = {const_cast<PassArgs *>(&a), const_cast<WindowShape *>(&shape)};
-    return launch_early(kernel32(layout, shape), grid, block, args, smem_f32(shape), s);
+    return launch_early(kernel32(layout, shape), grid, block, args, smem_f32(shape), s, false,
+                        wide_soa(layout, shape) ? kWideSoaBlocks : 0);
 }
 
 // Also allows the kernel the shared memory that the shape takes; a launch in
@@ -543,6 +551,7 @@ int pass_f32_occupancy(int layout, int block, const WindowShape &shape)
     if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess)
         cudaGetLastError();
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, block, smem_f32(shape));
+    if (wide_soa(layout, shape) && nb > kWideSoaBlocks) nb = kWideSoaBlocks;
     return nb > 0 ? nb : 1;
 }
 

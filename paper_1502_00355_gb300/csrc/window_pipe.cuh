@@ -55,25 +55,34 @@ __device__ __forceinline__ void after_previous()
 // Launches `kernel`, which calls after_previous(), to start early; in a stream
 // that is being captured it is an ordinary launch (the graph then has only
 // full dependencies, as its owner may expect) unless the library itself is
-// capturing it (own_graph).
+// capturing it (own_graph).  blocks > 0: prefer the shared-memory carve-out of so
+// many blocks an SM, which leaves the rest to L1.
 inline cudaError_t launch_early(const void *kernel, int grid, int block, void **args, size_t smem, cudaStream_t s,
-                                bool own_graph = false)
+                                bool own_graph = false, int blocks = 0)
 {
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     if (!own_graph && cudaStreamIsCapturing(s, &capture) != cudaSuccess) {
         cudaGetLastError();  // the legacy stream while another one is being captured: the launch will say so
         capture = cudaStreamCaptureStatusNone;
     }
-    cudaLaunchAttribute early[1] = {};
-    early[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    early[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attrs[2] = {};
+    int n = 0;
+    if (capture == cudaStreamCaptureStatusNone) {
+        attrs[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attrs[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (blocks > 0) {  // (1 KB a block is the system's; of the SM's 228 KB)
+        const size_t percent = ((size_t)blocks * (smem + 1024) * 100 + 228 * 1024 - 1) / (228 * 1024);
+        attrs[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        attrs[n++].val.sharedMemCarveout = (unsigned)(percent < 100 ? percent : 100);
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cfg.attrs = early;
-    cfg.numAttrs = capture == cudaStreamCaptureStatusNone ? 1 : 0;
+    cfg.attrs = attrs;
+    cfg.numAttrs = n;
     return cudaLaunchKernelExC(&cfg, kernel, args);
 }
 
