@@ -44,7 +44,7 @@ PROFILE_FIGURES = {
     "pass_screened": {
         "files": ["pass_screened.cu", "screen.cuh", "window.cuh", "window_pipe.cuh", "window_build.cu", "node_exact.cuh",
                   "div_small.cuh", "device.cuh"],
-        "sha256": "be8cfa230a685d3fb4fdacdd5df0fc60f075d7dc69aad13b50a40dd14c108eb9",
+        "sha256": "ad08dd89b208ac6a6f7e708221a27b0562a0cb7f7fbb7df50be44465b17953db",
         "dram_bytes_per_node": (172729088 + 41547264) / (2048 * 2048),
         "fp64_warp_inst_per_32_nodes": (1498730 + 300972 + 12061) / (2048 * 2048 / 32),
         "source": "profiles/pass_screened_grid2048.md (2048x2048 capture, per node)",
@@ -52,7 +52,7 @@ PROFILE_FIGURES = {
     "batch_pass": {
         "files": ["pass_screened.cu", "screen.cuh", "window.cuh", "window_pipe.cuh", "window_build.cu", "node_exact.cuh",
                   "div_small.cuh", "device.cuh", "batch.cu"],
-        "sha256": "16ac4f04aadb43770ba0d295c5632a572eec7212df498a47bc9643b22592e155",
+        "sha256": "fbbdef14dca1b169425b61742ccbf35d93051bdd0f7ef6ee3c767c7c381b9699",
         "dram_per_alg_byte": (494562048 + 161026560) / 994046024,
         "source": "profiles/batch_pass_batch256.md (round 0 of a 256-mesh batch, scaled by algorithmic bytes)",
     },

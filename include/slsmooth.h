@@ -134,7 +134,8 @@ typedef struct sls_info {
     int32_t converged;     /* 1 if the tolerance stopped the run                              */
     int64_t accepted_last; /* accepted free nodes in the last executed pass                   */
     double max_d2_last;    /* largest squared move in the last executed pass                  */
-    int64_t fp64_fallbacks;/* accept tests the screened kernel re-did in FP64 (last call)     */
+    int64_t fp64_fallbacks;/* accept tests the screened kernel left open and re-did in FP64,
+                              or by a closer screen where many are (last call)               */
     int64_t launches;      /* kernel launches issued by the last sls_smooth call (passes
                               launched after the tolerance was met return at once; a small
                               mesh's passes share one launch; 0 from the batched and served

@@ -532,7 +532,6 @@ __device__ __noinline__ uint32_t settle_open(const PassArgs &a, Queue *q, const 
                     finish_screened<LAYOUT>(a, q, node, verdict > 0,
                                             *reinterpret_cast<const ulonglong2 *>(xy + own), c, Cx, Cy);
                     if (verdict > 0) state |= 3u << 24;
-                    atomicSub(&q->nexact, 1u);  // (counted as open before; added up when the block's counts are)
                 }
             } else if (fill + cnt <= 32u) {
                 mask &= mask - 1u;

@@ -68,6 +68,20 @@ def test_same_bits(sls, name, opts):
         assert info[k] == winfo[k], k
 
 
+@pytest.mark.parametrize("name", ["flat 1e-3", "flat 1e-5", "graded", "far"])
+def test_the_same_counts_every_time(sls, name):
+    # which nodes find the queue full depends on the order of the warps; what a
+    # call reports does not
+    mesh = MESHES[name]()
+    infos = []
+    with sls.Mesh(mesh.xy, mesh.tri, mesh.boundary, copy_back=True) as g:
+        for _ in range(6):
+            g.set_coords(mesh.xy)
+            infos.append(g.smooth(20))
+    assert infos[0]["fp64_fallbacks"] > mesh.n
+    assert all(i == infos[0] for i in infos)
+
+
 @pytest.mark.parametrize("layout", ["aos", "soa"])
 def test_in_a_batch(sls, layout):
     names = sorted(MESHES)
