@@ -170,7 +170,8 @@ sls_status sls_mesh_create(const double *xy, int64_t n, const int32_t *tri, int6
 /* Runs up to max_iter Jacobi passes of Smart Laplacian smoothing (Eq. 2 with
  * the accept test of Section 3.3.4), continuing from the handle's current
  * coordinates.  tol_rel <= 0 disables the tolerance stop.  info may be NULL.
- * Blocks until the passes are done. */
+ * Blocks until the passes are done.  After SLS_ERR_TIMEOUT the coordinates are
+ * unspecified; sls_set_coords makes the handle good again. */
 sls_status sls_smooth(sls_mesh *mesh, int32_t max_iter, double tol_rel, sls_info *info);
 
 /* Copies the current coordinates (2n float64, interleaved) to xy_out, which is
